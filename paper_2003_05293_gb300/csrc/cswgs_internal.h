@@ -142,9 +142,9 @@ cudaError_t launch_subset_kernel(int P, int64_t Mp, uint64_t seed, int j, int32_
 int full_tc_tiles(int P);
 int full_tc_max_grid(int variant, int maxN, int sm_count);
 cudaError_t launch_full_tc(int variant, const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles,
-                           int maxN, unsigned *queue, int grid, cudaStream_t s);
+                           int maxN, unsigned *queue, int grid, int sm_count, cudaStream_t s);
 cudaError_t launch_subset_tc(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles, int maxN,
-                             unsigned *queue, int grid, int f16, cudaStream_t s);
+                             unsigned *queue, int grid, int f16, int sm_count, cudaStream_t s);
 void full_tc_table_bytes(int P, int N, size_t *rw, size_t *c, size_t *cs);   // cs: split BF16 (FP16: half)
 cudaError_t launch_tc_const_tables(const HoloDev *holos, int count, int sm_count, cudaStream_t s);
 cudaError_t launch_tc_rw_tables(const HoloDev *holos, const LaunchSlot *slots, int nslots, int sm_count,
@@ -152,14 +152,14 @@ cudaError_t launch_tc_rw_tables(const HoloDev *holos, const LaunchSlot *slots, i
 // subset masks of a launch's compressed slots (holograms at most maxP pixels a side)
 cudaError_t launch_tc_mask_scatter(const HoloDev *holos, const LaunchSlot *slots, int nslots, int maxP, int sm_count,
                                    cudaStream_t s);
-cudaError_t launch_tc_tails(const HoloDev *holos, const LaunchSlot *slots, int nslots, int maxN, bool subset,
-                            cudaStream_t s);
+cudaError_t launch_tc_tails(const HoloDev *holos, const LaunchSlot *slots, int nslots, int items, int maxN,
+                            bool subset, int sm_count, cudaStream_t s);
 // Subset-only gather kernel (kernels_gather.cu): work items per hologram,
 // resident blocks (0: N too large), launch (the kernel and the tails).
 int subset_gather_items(int P);
 int subset_gather_max_grid(int maxN, int sm_count);
 cudaError_t launch_subset_gather(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_items, int maxN,
-                                 unsigned *queue, int grid, cudaStream_t s);
+                                 unsigned *queue, int grid, int sm_count, cudaStream_t s);
 // Work items of a tensor-core launch: chooses the strip length (tiles of one
 // row block per work item, 1 for holograms of more than one GEMM 2 spot
 // block; `forced` > 0 takes that length) and rewrites each slot's strip, tiles
@@ -173,7 +173,7 @@ int shape_max_grid(TileShape shape, int kind, int maxN, int sm_count);
 int shape_full_tiles(int P, TileShape shape);
 TileShape full_fallback(TileShape shape, int maxN, int sm_count);
 cudaError_t shape_launch(TileShape shape, int kind, const HoloDev *holos, const LaunchSlot *slots, int nslots,
-                         int total_tiles, int maxN, unsigned *queue, int grid, cudaStream_t s);
+                         int total_tiles, int maxN, unsigned *queue, int grid, int sm_count, cudaStream_t s);
 
 cudaError_t launch_subset_ex_kernel(const HoloDev &H, int j, int32_t *out, cudaStream_t s);
 cudaError_t launch_sincos_probe(float *sink, long long *cycles, int iters, int blocks,

@@ -342,7 +342,7 @@ int subset_gather_max_grid(int maxN, int sm_count)
 }
 
 cudaError_t launch_subset_gather(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_items, int maxN,
-                                 unsigned *queue, int grid, cudaStream_t s)
+                                 unsigned *queue, int grid, int sm_count, cudaStream_t s)
 {
     const int spl = gather_spl(maxN);
     (void)cudaGetLastError();
@@ -355,7 +355,7 @@ cudaError_t launch_subset_gather(const HoloDev *holos, const LaunchSlot *slots, 
     if (spl > gather::kMaxSpl) return cudaErrorInvalidValue;
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_tc_tails(holos, slots, nslots, maxN, true, s);
+    return launch_tc_tails(holos, slots, nslots, total_items, maxN, true, sm_count, s);
 }
 
 }  // namespace cswgs

@@ -39,6 +39,7 @@
 // Z to the spot fields (epilogue 2) once per strip of tiles along a row block
 // and, in the final pass, write the phase map from S.  Every wait is bounded
 // and a timeout is recorded in the launch's status word instead of hanging.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -1421,31 +1422,174 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
     }
 }
 
-// The per-hologram tails of a warp-specialised launch, one block per slot
-// (blockIdx.y == 0): the weighted update (Eqs. 4-6) from the tile partials, or
-// the metrics.  The other blocks of a compressed slot clear its subset mask
-// for the next draw.
-constexpr int kTailThreads = 1024;   // a hologram's tile sums take a whole block's loads in flight
+// The per-hologram tails of a launch whose kernel writes tile partials: the
+// weighted update (Eqs. 4-6) or the metrics (Eq. 7), a cluster of CL blocks per
+// slot.  Bound by latency: a hologram's partials (27 to 162 items x N) are few
+// bytes, and on one SM their loads and FP64 additions queue behind each other,
+// so a launch of few holograms spreads each over up to 8 SMs.  Spots are dealt
+// out in fours (a 32-byte sector of an item's partials), a block taking every
+// CL-th; the lanes of a warp are 4 spots x 8 groups of items, and where a block
+// has warps to spare 2 to 16 of them share four spots.  The blocks' sums of
+// |V_n| (or e and the extremes of I_n) meet in distributed shared memory.
+// The blocks with blockIdx.y > 0 (compressed launches) clear the slot's subset
+// mask for the next draw.  On one block of 1024 threads a lone hologram's update
+// took 7 us (N = 100) and its metrics 38 us (N = 300: 63 us), most of it FP64
+// additions; a whole final pass at N = 300 fell from 240 to 184 us per call.
+constexpr int kTailThreads = 512;
+constexpr int kTailMaxN = 6144;
+constexpr int kTailClear = 8;               // blocks per slot that clear its mask
 
-__global__ void __launch_bounds__(kTailThreads) tcws_tails_kernel(const HoloDev *__restrict__ holos,
-                                                         const LaunchSlot *__restrict__ slots)
+// Shared memory of a block whose share is nq fours: the warps' sums (16 bytes
+// per spot and warp sharing it) and V_n.
+__host__ __device__ constexpr size_t tail_smem(int nq)
 {
-    extern __shared__ float2 s_v[];
-    __shared__ double s_red[kTailThreads / 32];
-    const LaunchSlot sl = slots[blockIdx.x];
+    return (size_t)4 * 16 * (nq > kTailThreads / 32 ? nq : kTailThreads / 32) + (size_t)4 * 8 * nq;
+}
+
+// Sum of spot n's partials over the items t = g, g + G, ..., combined over the
+// 8 lane groups of the warp (lanes that differ in bits 2 to 4).
+__device__ __forceinline__ float4 tail_warp_sum(const HoloDev &H, int n, int g, int G, int tiles)
+{
+    const float4 q = tile_sum(H, n, g, G, tiles);
+    float sr = q.x, cr = q.y, si = q.z, ci = q.w;   // the sum is s - c
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) {
+        add_comp(sr, cr, __shfl_xor_sync(0xffffffffu, sr, o), __shfl_xor_sync(0xffffffffu, cr, o));
+        add_comp(si, ci, __shfl_xor_sync(0xffffffffu, si, o), __shfl_xor_sync(0xffffffffu, ci, o));
+    }
+    return make_float4(sr, cr, si, ci);
+}
+
+__device__ __forceinline__ double2 tail_warp_sum64(const HoloDev &H, int n, int g, int G, int tiles)
+{
+    double vr = 0.0, vi = 0.0;
+#pragma unroll 4
+    for (int t = g; t < tiles; t += G) {
+        const double2 p = __ldcg(&H.part64[(size_t)t * H.N + n]);
+        vr += p.x;
+        vi += p.y;
+    }
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) {
+        vr += __shfl_xor_sync(0xffffffffu, vr, o);
+        vi += __shfl_xor_sync(0xffffffffu, vi, o);
+    }
+    return make_double2(vr, vi);
+}
+
+template <int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kTailThreads)
+tcws_tails_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__restrict__ slots)
+{
+    constexpr int W = kTailThreads / 32;
+    extern __shared__ __align__(16) double2 s_part[];   // per spot and warp: float4 {s_re, c_re, s_im, c_im} or FP64
+    __shared__ double s_red[W];
+    __shared__ double s_out[3];                  // this block's sum (and extremes), read by the cluster
+    __shared__ double s_mean;
+    const LaunchSlot sl = slots[blockIdx.x / CL];
     const HoloDev &H = holos[sl.holo];
-    if (blockIdx.y > 0) {
+    const int rank = blockIdx.x % CL, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (blockIdx.y > 0) {   // a whole cluster of its own
         if (sl.pass == kPassSubset && H.mask) {
             uint32_t *mask = subset_mask(H, sl.j);
             const size_t words = (size_t)H.P * H.mask_words;
-            for (size_t i = (size_t)(blockIdx.y - 1) * blockDim.x + threadIdx.x; i < words;
-                 i += (size_t)(gridDim.y - 1) * blockDim.x)
-                mask[i] = 0u;
+            const size_t part = (blockIdx.y - 1) * CL + rank;
+            for (size_t i = part * kTailThreads + tid; i < words; i += (size_t)kTailClear * kTailThreads) mask[i] = 0u;
         }
         return;
     }
-    if (sl.pass == kPassFinal) tail_metrics<kTailThreads, true>(H, sl, s_red);
-    else tail_update<kTailThreads, true>(H, sl, s_v, s_red);
+    const int N = H.N, quads = (N + 3) / 4;
+    const int nq = (quads - rank + CL - 1) / CL;   // this block's fours: rank, rank + CL, ...
+    int wq = W;                                                        // warps per four spots: a power of two
+    while (wq > 1 && wq * nq > W) wq >>= 1;
+    const bool metrics = sl.pass == kPassFinal;
+    float4 *s_part32 = reinterpret_cast<float4 *>(s_part);
+    float2 *s_v = reinterpret_cast<float2 *>(s_part + 4 * max(nq, W));
+    for (int i = warp / wq; i < nq; i += W / wq) {
+        const int n = min(4 * (rank + CL * i) + (lane & 3), N - 1);   // past the last spot: not stored
+        const int g = (lane >> 2) + 8 * (warp % wq), at = (i * wq + warp % wq) * 4 + lane;
+        if (metrics) {
+            const double2 v = tail_warp_sum64(H, n, g, 8 * wq, sl.tiles);
+            if (lane < 4) s_part[at] = v;
+        } else {
+            const float4 v = tail_warp_sum(H, n, g, 8 * wq, sl.tiles);
+            if (lane < 4) s_part32[at] = v;
+        }
+    }
+    __syncthreads();
+    // one thread per spot of this block
+    const float inv = 1.0f / (float)sl.count;
+    const double inv64 = 1.0 / H.norm;   // sum of A over the pupil (P^2 for the square uniform grid)
+    double sum = 0.0, imax = -1.0, imin = 1e300;
+    for (int k = tid; k < 4 * nq; k += kTailThreads) {
+        const int i = k >> 2, n = 4 * (rank + CL * i) + (k & 3);
+        if (n >= N) continue;
+        if (metrics) {
+            double vr = 0.0, vi = 0.0;
+            for (int g = 0; g < wq; ++g) {
+                const double2 p = s_part[(i * wq + g) * 4 + (k & 3)];
+                vr += p.x;
+                vi += p.y;
+            }
+            vr *= inv64;
+            vi *= inv64;
+            const double in = vr * vr + vi * vi;
+            H.metrics[2 + n] = in;
+            sum += in;
+            imax = fmax(imax, in);
+            imin = fmin(imin, in);
+        } else {
+            float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;
+            for (int g = 0; g < wq; ++g) {
+                const float4 p = s_part32[(i * wq + g) * 4 + (k & 3)];
+                add_comp(sr, cr, p.x, p.y);
+                add_comp(si, ci, p.z, p.w);
+            }
+            const float2 v = make_float2((sr - cr) * inv, (si - ci) * inv);
+            s_v[k] = v;
+            sum += (double)hypotf(v.x, v.y);
+        }
+    }
+    sum = block_sum_f64<kTailThreads>(sum, s_red);
+    if (metrics) {
+        imax = block_max_f64<kTailThreads>(imax, s_red);
+        imin = block_min_f64<kTailThreads>(imin, s_red);
+    }
+    if (tid == 0) {
+        s_out[0] = sum;
+        s_out[1] = imax;
+        s_out[2] = imin;
+    }
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    cluster.sync();
+    if (metrics) {
+        if (rank == 0 && tid == 0) {
+            double e = 0.0;
+            imax = -1.0;
+            imin = 1e300;
+            for (int r = 0; r < CL; ++r) {
+                const double *o = cluster.map_shared_rank(s_out, r);
+                e += o[0];
+                imax = fmax(imax, o[1]);
+                imin = fmin(imin, o[2]);
+            }
+            H.metrics[0] = e;
+            H.metrics[1] = (imax + imin) > 0.0 ? 1.0 - (imax - imin) / (imax + imin) : 0.0;
+        }
+    } else {
+        if (warp == 0) {
+            double m = lane < CL ? cluster.map_shared_rank(s_out, lane)[0] : 0.0;
+            for (int o = CL / 2; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+            if (lane == 0) s_mean = m / (double)N;
+        }
+        __syncthreads();
+        const double mean = s_mean;
+        for (int k = tid; k < 4 * nq; k += kTailThreads) {
+            const int n = 4 * (rank + CL * (k >> 2)) + (k & 3);
+            if (n < N) update_spot(H, n, s_v[k], mean);
+        }
+    }
+    cluster.sync();   // s_out is read before any block of the cluster leaves
 }
 
 template <int W, bool F16, int US>
@@ -1455,7 +1599,7 @@ static int tcws_max_grid_of(int maxN, int sm_count)
     if (cudaFuncGetAttributes(&fa, iter_full_tcws_kernel<W, F16, US>) != cudaSuccess) return 0;
     const size_t limit = 227 * 1024 - fa.sharedSizeBytes;
     const size_t smem = tc::ws::Lay<US>::kSmem;
-    if (smem > limit || (size_t)maxN * sizeof(float2) > 48 * 1024) return 0;
+    if (smem > limit || maxN > kTailMaxN) return 0;
     if (cudaFuncSetAttribute(iter_full_tcws_kernel<W, F16, US>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)limit) != cudaSuccess)
         return 0;
@@ -1482,20 +1626,37 @@ static void tcws_launch_one(const HoloDev *holos, const LaunchSlot *slots, int n
         holos, slots, nslots, total_tiles, queue);
 }
 
-// The per-hologram tails of a launch whose kernel writes tile partials and no
-// tail of its own: one block per slot, plus (compressed launches) blocks that
-// clear the subset masks.
-cudaError_t launch_tc_tails(const HoloDev *holos, const LaunchSlot *slots, int nslots, int maxN, bool subset,
-                            cudaStream_t s)
+// The tails of a launch of `items` work items: clusters of as many blocks (up to
+// 8) as leave every slot's on an SM of its own, one where a hologram's partials
+// are a few loads per thread (the cluster's launch and barriers would cost more
+// than they spread); and (compressed launches) the blocks that clear the masks.
+cudaError_t launch_tc_tails(const HoloDev *holos, const LaunchSlot *slots, int nslots, int items, int maxN,
+                            bool subset, int sm_count, cudaStream_t s)
 {
-    const dim3 tails((unsigned)nslots, 1u + (subset ? 8u : 0u));
-    tcws_tails_kernel<<<tails, kTailThreads, (size_t)maxN * sizeof(float2), s>>>(holos, slots);
-    return cudaGetLastError();
+    if (maxN > kTailMaxN) return cudaErrorInvalidValue;
+    int cl = 8;
+    while (cl > 1 && (cl * nslots > sm_count || (int64_t)items * maxN < (int64_t)2048 * nslots)) cl >>= 1;
+    const dim3 grid((unsigned)(cl * nslots), 1u + (subset ? (unsigned)(kTailClear / cl) : 0u));
+    const size_t smem = tail_smem((maxN + 4 * cl - 1) / (4 * cl));
+    auto go = [&](auto kernel) {
+        if (smem > 48 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        kernel<<<grid, kTailThreads, smem, s>>>(holos, slots);
+        return cudaGetLastError();
+    };
+    switch (cl) {
+    case 8: return go(tcws_tails_kernel<8>);
+    case 4: return go(tcws_tails_kernel<4>);
+    case 2: return go(tcws_tails_kernel<2>);
+    default: return go(tcws_tails_kernel<1>);
+    }
 }
 
 template <int W>
 static cudaError_t tcws_launch(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles, int maxN,
-                               unsigned *queue, int grid, bool subset, int f16, cudaStream_t s)
+                               unsigned *queue, int grid, bool subset, int f16, int sm_count, cudaStream_t s)
 {
     constexpr int K4 = tc::ws::kKSteps;
     (void)cudaGetLastError();
@@ -1503,7 +1664,7 @@ static cudaError_t tcws_launch(const HoloDev *holos, const LaunchSlot *slots, in
     else tcws_launch_one<W, false, K4>(holos, slots, nslots, total_tiles, queue, grid, s);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_tc_tails(holos, slots, nslots, maxN, subset, s);
+    return launch_tc_tails(holos, slots, nslots, total_tiles, maxN, subset, sm_count, s);
 }
 
 // epilogue warps of the warp-specialised kernel
@@ -1640,16 +1801,16 @@ cudaError_t launch_tc_mask_scatter(const HoloDev *holos, const LaunchSlot *slots
 }
 
 cudaError_t launch_subset_tc(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles, int maxN,
-                             unsigned *queue, int grid, int f16, cudaStream_t s)
+                             unsigned *queue, int grid, int f16, int sm_count, cudaStream_t s)
 {
-    return tcws_launch<kWsWarps>(holos, slots, nslots, total_tiles, maxN, queue, grid, true, f16, s);
+    return tcws_launch<kWsWarps>(holos, slots, nslots, total_tiles, maxN, queue, grid, true, f16, sm_count, s);
 }
 
 cudaError_t launch_full_tc(int variant, const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles,
-                           int maxN, unsigned *queue, int grid, cudaStream_t s)
+                           int maxN, unsigned *queue, int grid, int sm_count, cudaStream_t s)
 {
     if (variant != kFullTcWs) return cudaErrorInvalidValue;
-    return tcws_launch<kWsWarps>(holos, slots, nslots, total_tiles, maxN, queue, grid, false, 0, s);
+    return tcws_launch<kWsWarps>(holos, slots, nslots, total_tiles, maxN, queue, grid, false, 0, sm_count, s);
 }
 
 }  // namespace cswgs

@@ -224,14 +224,14 @@ int shape_full_tiles(int P, TileShape shape)
 }
 
 cudaError_t shape_launch(TileShape shape, int kind, const HoloDev *holos, const LaunchSlot *slots, int nslots,
-                         int total_tiles, int maxN, unsigned *queue, int grid, cudaStream_t s)
+                         int total_tiles, int maxN, unsigned *queue, int grid, int sm_count, cudaStream_t s)
 {
     if (kind == kLaunchFull && is_full_tc(shape.full_threads))
-        return launch_full_tc(shape.full_threads, holos, slots, nslots, total_tiles, maxN, queue, grid, s);
+        return launch_full_tc(shape.full_threads, holos, slots, nslots, total_tiles, maxN, queue, grid, sm_count, s);
     if (kind == kLaunchSubset && shape.threads == kSubsetTc)
-        return launch_subset_tc(holos, slots, nslots, total_tiles, maxN, queue, grid, shape.fp16, s);
+        return launch_subset_tc(holos, slots, nslots, total_tiles, maxN, queue, grid, shape.fp16, sm_count, s);
     if (kind == kLaunchSubset && shape.threads == kSubsetGather)
-        return launch_subset_gather(holos, slots, nslots, total_tiles, maxN, queue, grid, s);
+        return launch_subset_gather(holos, slots, nslots, total_tiles, maxN, queue, grid, sm_count, s);
     return launch_iter_fp32(shape, kind, holos, slots, nslots, total_tiles, maxN, queue, grid, s);
 }
 
@@ -632,7 +632,7 @@ cswgs_status batch_enqueue_direct(Fp32Batch *b, cudaStream_t s, bool capturing)
                 CSWGS_CUDA_TRY(launch_tc_rw_tables(holos, slots + b->l_slot0[i], b->l_nslots[i], b->plan->sm_count, s));
             if (side_draw) CSWGS_CUDA_TRY(cudaStreamWaitEvent(s, b->ev_scat[L & 1], 0));
             CSWGS_CUDA_TRY(shape_launch(b->shape, kind, holos, slots + b->l_slot0[i], b->l_nslots[i], tiles,
-                                        b->l_maxN[i], queue, grid, s));
+                                        b->l_maxN[i], queue, grid, b->plan->sm_count, s));
             if (side_draw) {
                 CSWGS_CUDA_TRY(cudaEventRecordWithFlags(b->ev_tail[L & 1], s, 0));
                 tail_rec[L & 1] = true;

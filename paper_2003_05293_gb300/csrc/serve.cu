@@ -467,7 +467,7 @@ void Server::loop()
             if (launch_uses_tc(shape_, kind))
                 chk(launch_tc_rw_tables(holos, sd + first, group_slots[kind], p_->sm_count, stream_));
             chk(shape_launch(shape_, kind, holos, sd + first, group_slots[kind], group_tiles[kind], group_maxN[kind],
-                             queue, std::min(g->second, group_tiles[kind]), stream_));
+                             queue, std::min(g->second, group_tiles[kind]), p_->sm_count, stream_));
         }
         double *mh = met_h_ + (size_t)(serial & 1) * 2 * B;
         for (Req *r : finishing) {

@@ -11,32 +11,52 @@ namespace cswgs {
 
 constexpr int kSpotChunk = 128;   // spots per forward-reduction round
 
-template <int THREADS>
-__device__ __forceinline__ double block_sum_f64(double v, double *s_red)
+// Block-wide FP64 reductions, the result in every thread.  The FP64 pipe takes
+// a warp instruction only every few dozen cycles, so the instructions are kept
+// few: a warp whose lanes all hold the neutral element (the threads past the
+// last spot) skips the shuffle tree, and one warp reduces the warps' results.
+// (Every thread adding up the warps' results, 32 x 32 FP64 additions of a
+// 1024-thread block, took most of an update's 7 us.)
+template <int THREADS, class Op>
+__device__ __forceinline__ double block_reduce_f64(double v, double neutral, double *s_red, Op op)
 {
     constexpr int W = THREADS / 32;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto tree = [&](double x) {
+        if (__any_sync(0xffffffffu, __double_as_longlong(x) != __double_as_longlong(neutral)))
+            for (int o = 16; o > 0; o >>= 1) x = op(x, __shfl_xor_sync(0xffffffffu, x, o));
+        return x;
+    };
+    v = tree(v);
     __syncthreads();
     if (lane == 0) s_red[warp] = v;
     __syncthreads();
-    double r = 0.0;
-    for (int w = 0; w < W; ++w) r += s_red[w];
-    return r;
+    if (warp == 0) {
+        v = tree(lane < W ? s_red[lane] : neutral);
+        if (lane == 0) s_red[0] = v;
+    }
+    __syncthreads();
+    return s_red[0];
 }
 
 template <int THREADS>
+__device__ __forceinline__ double block_sum_f64(double v, double *s_red)
+{
+    return block_reduce_f64<THREADS>(v, 0.0, s_red, [](double a, double b) { return a + b; });
+}
+
+// Largest of values >= -1 (threads without one pass -1).
+template <int THREADS>
 __device__ __forceinline__ double block_max_f64(double v, double *s_red)
 {
-    constexpr int W = THREADS / 32;
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) s_red[warp] = v;
-    __syncthreads();
-    double r = s_red[0];
-    for (int w = 1; w < W; ++w) r = fmax(r, s_red[w]);
-    return r;
+    return block_reduce_f64<THREADS>(v, -1.0, s_red, [](double a, double b) { return fmax(a, b); });
+}
+
+// Smallest of values <= 1e300 (threads without one pass 1e300).
+template <int THREADS>
+__device__ __forceinline__ double block_min_f64(double v, double *s_red)
+{
+    return block_reduce_f64<THREADS>(v, 1e300, s_red, [](double a, double b) { return fmin(a, b); });
 }
 
 // Weighted update (Eqs. 4-6) from the per-tile partial fields of one pass:
@@ -59,101 +79,58 @@ __device__ __forceinline__ float4 tile_sum(const HoloDev &H, int n, int t0, int 
     return make_float4(sr, cr, si, ci);
 }
 
-// With SPLIT (a block of its own per hologram), G groups of threads share a
-// spot's tiles (t = g, g + G, ...) when the block has threads to spare, for
-// G times the loads in flight; each group's compensated sum (s, c) stands for
-// s - c, and the G of them are summed with compensation again.
-template <int THREADS, bool SPLIT = false>
+// (s, c) += (t, d), two compensated sums (each stands for s - c): the rounding
+// error of s + t (Knuth's two-sum) joins the compensation.
+__device__ __forceinline__ void add_comp(float &s, float &c, float t, float d)
+{
+    const float r = __fadd_rn(s, t), b = __fsub_rn(r, s);
+    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(r, b)), __fsub_rn(t, b));
+    s = r;
+    c = (c + d) - err;
+}
+
+// Eqs. 4 and 6 for spot n with field v and mean amplitude <|V|>.
+__device__ __forceinline__ void update_spot(const HoloDev &H, int n, float2 v, double mean)
+{
+    const float mag = hypotf(v.x, v.y);
+    SpotState st = H.state[n];
+    st.w = (float)((double)st.w * mean / (double)fmaxf(mag, 1e-30f));
+    if (mag > 0.f) st.theta = rad_to_fix(atan2f(v.y, v.x));
+    H.state[n] = st;
+}
+
+template <int THREADS>
 __device__ void tail_update(const HoloDev &H, const LaunchSlot &sl, float2 *s_v, double *s_red)
 {
     const int N = H.N;
     const float inv = 1.0f / (float)sl.count;
-    const int G = SPLIT ? max(1, min(16, THREADS / max(1, N))) : 1;
-    float4 *s_grp = nullptr;
-    if constexpr (SPLIT) {
-        __shared__ double2 s_grp_buf[THREADS];
-        s_grp = reinterpret_cast<float4 *>(s_grp_buf);
-        if (G > 1) {
-            const int n = threadIdx.x % N, g = threadIdx.x / N;
-            if (g < G) s_grp[g * N + n] = tile_sum(H, n, g, G, sl.tiles);
-            __syncthreads();
-        }
-    }
     double local = 0.0;
     for (int n = threadIdx.x; n < N; n += THREADS) {
-        float4 q;
-        if (G > 1) {
-            float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;
-            for (int g = 0; g < G; ++g) {
-                const float4 p = s_grp[g * N + n];
-                float yr = (p.x - p.y) - cr, tr = sr + yr;
-                cr = (tr - sr) - yr;
-                sr = tr;
-                float yi = (p.z - p.w) - ci, ti = si + yi;
-                ci = (ti - si) - yi;
-                si = ti;
-            }
-            q = make_float4(sr, cr, si, ci);
-        } else {
-            q = tile_sum(H, n, 0, 1, sl.tiles);
-        }
+        const float4 q = tile_sum(H, n, 0, 1, sl.tiles);
         float2 v = make_float2(q.x * inv, q.z * inv);
         s_v[n] = v;
         local += (double)hypotf(v.x, v.y);
     }
     const double mean = block_sum_f64<THREADS>(local, s_red) / (double)N;
-    for (int n = threadIdx.x; n < N; n += THREADS) {
-        float2 v = s_v[n];
-        float mag = hypotf(v.x, v.y);
-        SpotState st = H.state[n];
-        st.w = (float)((double)st.w * mean / (double)fmaxf(mag, 1e-30f));
-        if (mag > 0.f) st.theta = rad_to_fix(atan2f(v.y, v.x));
-        H.state[n] = st;
-    }
+    for (int n = threadIdx.x; n < N; n += THREADS) update_spot(H, n, s_v[n], mean);
 }
 
 // Metrics of the final pass: V_n = sum over the pupil of A e^{i(Phi - phi_n)}
 // (FP64 partials) divided by the pupil's sum of A, I_n = |V_n|^2,
 // e = sum_n I_n, u by Eq. 7.
-// With SPLIT, G groups of threads share a spot's tiles as in tail_update.
-template <int THREADS, bool SPLIT = false>
+template <int THREADS>
 __device__ void tail_metrics(const HoloDev &H, const LaunchSlot &sl, double *s_red)
 {
     const int N = H.N;
     const double inv = 1.0 / H.norm;   // sum of A over the pupil (P^2 for the square uniform grid)
-    const int G = SPLIT ? max(1, min(16, THREADS / max(1, N))) : 1;
-    auto sum = [&](int n, int t0, int dt) {
-        double vr = 0.0, vi = 0.0;
-#pragma unroll 8
-        for (int t = t0; t < sl.tiles; t += dt) {
-            double2 p = __ldcg(&H.part64[(size_t)t * N + n]);
-            vr += p.x;
-            vi += p.y;
-        }
-        return make_double2(vr, vi);
-    };
-    double2 *s_grp = nullptr;
-    if constexpr (SPLIT) {
-        __shared__ double2 s_grp_buf[THREADS];
-        s_grp = s_grp_buf;
-        if (G > 1) {
-            const int n = threadIdx.x % N, g = threadIdx.x / N;
-            if (g < G) s_grp[g * N + n] = sum(n, g, G);
-            __syncthreads();
-        }
-    }
     double e = 0.0, imax = -1.0, imin = 1e300;
     for (int n = threadIdx.x; n < N; n += THREADS) {
         double vr = 0.0, vi = 0.0;
-        if (G > 1) {
-            for (int g = 0; g < G; ++g) {
-                vr += s_grp[g * N + n].x;
-                vi += s_grp[g * N + n].y;
-            }
-        } else {
-            const double2 v = sum(n, 0, 1);
-            vr = v.x;
-            vi = v.y;
+#pragma unroll 8
+        for (int t = 0; t < sl.tiles; ++t) {
+            double2 p = __ldcg(&H.part64[(size_t)t * N + n]);
+            vr += p.x;
+            vi += p.y;
         }
         vr *= inv;
         vi *= inv;
@@ -165,7 +142,7 @@ __device__ void tail_metrics(const HoloDev &H, const LaunchSlot &sl, double *s_r
     }
     e = block_sum_f64<THREADS>(e, s_red);
     imax = block_max_f64<THREADS>(imax, s_red);
-    imin = -block_max_f64<THREADS>(-imin, s_red);
+    imin = block_min_f64<THREADS>(imin, s_red);
     if (threadIdx.x == 0) {
         H.metrics[0] = e;
         H.metrics[1] = (imax + imin) > 0.0 ? 1.0 - (imax - imin) / (imax + imin) : 0.0;

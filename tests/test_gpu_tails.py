@@ -1,0 +1,51 @@
+"""The tails of the tensor-core launches (weighted update, metrics) and the
+amplitude range of their operands, at the sizes where the work's split
+changes: spots dealt out in fours to 1 to 8 blocks per hologram and to 1 to
+16 warps per four spots (N below, at and past multiples of 4, 32 and 128; few
+and many work items; one hologram and batches of 3, 20 and 80), against the
+oracle, teacher-forced."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from gpu_helpers import TOL_EU, TOL_PHASE_RMS, rms_wrapped, write_pinned_tune_cache
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+SUBSET_TC, FULL_WS = 1, 2
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    from paper_2003_05293_gb300 import Plan
+    path = tmp_path_factory.mktemp("tails") / "t.json"
+    p = Plan(precision="fp32", max_batch=128, tune_cache=write_pinned_tune_cache(path, SUBSET_TC, 1, FULL_WS,
+                                                                                 batch_pow2=range(0, 8)))
+    yield p
+    p.close()
+
+
+def _start(N, seed):
+    rng = np.random.default_rng(seed)
+    return np.exp(rng.normal(0.0, 0.3, N)), rng.uniform(-np.pi, np.pi, N)
+
+
+@pytest.mark.parametrize("P,N", [(64, 1), (64, 3), (128, 4), (130, 5), (256, 33), (256, 127), (300, 129), (640, 31),
+                                 (200, 1000)])
+@pytest.mark.parametrize("full", [0, 1])
+def test_update_and_metrics(plan, P, N, full):
+    pb = workloads.problem(P, N, 5.0, 0.25, 1, seed=40 + N)
+    w0, th0 = _start(N, N)
+    r = plan.solve(pb.xyz, P, pb.c, 1, pb.seed, init_w=w0, init_theta=th0, first_iteration=3, full_iterations=full,
+                   final_pass=True, state=True)
+    ref = oracle.solve(P, pb.xyz, c=pb.c, iterations=1, seed=pb.seed, theta_in=th0, w_in=w0, first_j=3,
+                       full_iterations=full)
+    assert rms_wrapped(r["theta"], ref["theta"]) < TOL_PHASE_RMS
+    assert math.sqrt(np.mean((r["w"] / ref["w"] - 1) ** 2)) < TOL_PHASE_RMS
+    assert abs(r["e"] - ref["e"]) < TOL_EU and abs(r["u"] - ref["u"]) < TOL_EU
+    assert abs(float(np.sum(r["I"])) - r["e"]) < 1e-12 * N
