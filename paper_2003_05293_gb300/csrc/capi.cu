@@ -34,19 +34,20 @@ static cswgs_status solve_fp64(cswgs_plan_s *p, const HoloSpec &h, float *phase_
 {
     const int N = h.N, P = h.P;
     const int64_t M = (int64_t)P * P;
-    const int chunks = (int)((M + 4095) / 4096);
+    const int items = fp64_items(P, p->sm_count), words = mask_words_of(P);
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     size_t off = 0;
     size_t o_xyz = off; off += al(sizeof(double) * 3 * N);
     size_t o_amp = off; off += al(sizeof(double) * N);
     size_t o_iw = off; off += al(sizeof(double) * N);
     size_t o_it = off; off += al(sizeof(double) * N);
-    size_t o_coef = off; off += al(sizeof(double) * 3 * N);
+    size_t o_C = off; off += al(sizeof(double2) * (size_t)N * P);
+    size_t o_R = off; off += al(sizeof(double2) * (size_t)N * P);
     size_t o_w = off; off += al(sizeof(double) * N);
     size_t o_th = off; off += al(sizeof(double) * N);
-    size_t o_phi = off; off += al(sizeof(double) * M);
-    size_t o_pix = off; off += al(sizeof(int32_t) * std::max(h.Mp, 1));
-    size_t o_part = off; off += al(sizeof(double2) * (size_t)chunks * N);
+    size_t o_wt = off; off += al(sizeof(double2) * N);
+    size_t o_mask = off; off += al(sizeof(uint32_t) * (size_t)P * words);
+    size_t o_part = off; off += al(sizeof(double2) * (size_t)items * N);
     size_t o_met = off; off += al(sizeof(double) * (2 + N));
     size_t o_out = off; off += out_on_host ? al(sizeof(float) * M) : 0;
     CSWGS_TRY(p->f64_mem.ensure(off));
@@ -56,14 +57,14 @@ static cswgs_status solve_fp64(cswgs_plan_s *p, const HoloSpec &h, float *phase_
     wk.amp = h.has_amp ? reinterpret_cast<double *>(b + o_amp) : nullptr;
     wk.init_w = h.has_init_w ? reinterpret_cast<double *>(b + o_iw) : nullptr;
     wk.init_th = h.has_init_th ? reinterpret_cast<double *>(b + o_it) : nullptr;
-    wk.coef = reinterpret_cast<double *>(b + o_coef);
+    wk.C = reinterpret_cast<double2 *>(b + o_C);
+    wk.R = reinterpret_cast<double2 *>(b + o_R);
     wk.w = reinterpret_cast<double *>(b + o_w);
     wk.theta = reinterpret_cast<double *>(b + o_th);
-    wk.phi = reinterpret_cast<double *>(b + o_phi);
-    wk.pix = reinterpret_cast<int32_t *>(b + o_pix);
+    wk.weight = reinterpret_cast<double2 *>(b + o_wt);
+    wk.mask = reinterpret_cast<uint32_t *>(b + o_mask);
     wk.part = reinterpret_cast<double2 *>(b + o_part);
     wk.metrics = reinterpret_cast<double *>(b + o_met);
-    wk.chunks = chunks;
     cudaStream_t s = p->stream;
     CSWGS_CUDA_TRY(cudaMemcpyAsync(wk.xyz, h.xyz.data(), sizeof(double) * 3 * N, cudaMemcpyHostToDevice, s));
     if (wk.amp) CSWGS_CUDA_TRY(cudaMemcpyAsync(wk.amp, h.amp.data(), sizeof(double) * N, cudaMemcpyHostToDevice, s));
@@ -71,7 +72,7 @@ static cswgs_status solve_fp64(cswgs_plan_s *p, const HoloSpec &h, float *phase_
     if (wk.init_th) CSWGS_CUDA_TRY(cudaMemcpyAsync(wk.init_th, h.init_th.data(), sizeof(double) * N, cudaMemcpyHostToDevice, s));
     float *dev_out = out_on_host ? reinterpret_cast<float *>(b + o_out) : phase_out;
     CSWGS_CUDA_TRY(fp64_solve(wk, P, N, h.Mp, h.iterations, std::min(h.n_full, h.iterations), h.first_j,
-                              h.seed, h.final_pass, phase_out ? dev_out : nullptr, s));
+                              h.seed, h.final_pass, phase_out ? dev_out : nullptr, p->sm_count, s));
     std::vector<double> met(2 + N);
     if (h.final_pass) {
         CSWGS_CUDA_TRY(cudaMemcpyAsync(met.data(), wk.metrics, sizeof(double) * (2 + N), cudaMemcpyDeviceToHost, s));

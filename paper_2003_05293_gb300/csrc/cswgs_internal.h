@@ -179,19 +179,19 @@ cudaError_t launch_subset_ex_kernel(const HoloDev &H, int j, int32_t *out, cudaS
 cudaError_t launch_sincos_probe(float *sink, long long *cycles, int iters, int blocks,
                                 int threads, cudaStream_t s);
 
-// FP64 baseline solver (kernels_fp64.cu): one hologram, plain kernels.
+// FP64 baseline solver (kernels_fp64.cu): one hologram.
 struct Fp64Work {
     double *xyz, *amp, *init_w, *init_th;
-    double *coef;        // N x 3: turns per pixel (a, b, g)
+    double2 *C, *R;      // N x P each: column and row factors of Eq. 2
     double *w, *theta;   // N
-    double *phi;         // M
-    int32_t *pix;        // Mp
-    double2 *part;       // chunks x N
+    double2 *weight;     // N: w a e^{i theta}
+    uint32_t *mask;      // P rows of ceil(P / 32) words: the subset of a compressed iteration
+    double2 *part;       // fp64_items x N
     double *metrics;     // 2 + N
-    int chunks;
 };
+int fp64_items(int P, int sm_count);   // work items (blocks) of a pass
 cudaError_t fp64_solve(const Fp64Work &wk, int P, int N, int Mp, int iterations, int n_full,
                        int first_j, uint64_t seed, int final_pass, float *phase_out,
-                       cudaStream_t s);
+                       int sm_count, cudaStream_t s);
 
 }  // namespace cswgs
