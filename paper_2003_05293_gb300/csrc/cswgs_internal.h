@@ -140,6 +140,7 @@ cudaError_t launch_subset_kernel(int P, int64_t Mp, uint64_t seed, int j, int32_
                                  cudaStream_t s);
 // Tensor-core full-pass kernel (kernels_tc.cu).
 int full_tc_tiles(int P);
+int full_tc_spot_blocks(int N);
 int full_tc_max_grid(int variant, int maxN, int sm_count);
 cudaError_t launch_full_tc(int variant, const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles,
                            int maxN, unsigned *queue, int grid, int sm_count, cudaStream_t s);
@@ -162,10 +163,11 @@ cudaError_t launch_subset_gather(const HoloDev *holos, const LaunchSlot *slots, 
                                  unsigned *queue, int grid, int sm_count, cudaStream_t s);
 // Work items of a tensor-core launch: chooses the strip length (tiles of one
 // row block per work item, 1 for holograms of more than one GEMM 2 spot
-// block; `forced` > 0 takes that length) and rewrites each slot's strip, tiles
+// block; `forced` > 0 takes that length, the length taken goes to *chosen) and rewrites each slot's strip, tiles
 // and tile_begin; P[i], N[i] are slot i's hologram sizes.  Returns the
 // launch's work items.
-int full_tc_assign_strips(LaunchSlot *slots, int nslots, const int *P, const int *N, int grid, int forced);
+int full_tc_assign_strips(LaunchSlot *slots, int nslots, const int *P, const int *N, int grid, int forced,
+                          int *chosen = nullptr);
 
 // Either full-pass kernel, by tile shape (runtime.cu).
 bool shape_supported(TileShape shape);

@@ -1672,13 +1672,16 @@ constexpr int kWsWarps = 8;
 
 int full_tc_tiles(int P) { return tc::tiles(P); }
 
+int full_tc_spot_blocks(int N) { return tc::nspotblocks(N); }
+
 // Strip length of a launch: the one that minimises an estimate of its time in
 // tile times, (tiles + f items) / grid + S / 2: the work spread over the
 // resident blocks, a flush per work item (epilogue 2 and the hand-over of Z,
 // f = 1/2 a tile), and the tail left by the last strips (half a strip); or the
 // forced length.  A hologram with more than one spot block per GEMM 2 takes
 // strips of one tile.
-int full_tc_assign_strips(LaunchSlot *slots, int nslots, const int *P, const int *N, int grid, int forced)
+int full_tc_assign_strips(LaunchSlot *slots, int nslots, const int *P, const int *N, int grid, int forced,
+                          int *chosen)
 {
     using namespace tc;
     grid = std::max(1, grid);
@@ -1711,15 +1714,28 @@ int full_tc_assign_strips(LaunchSlot *slots, int nslots, const int *P, const int
         }
         return *std::max_element(heap.begin(), heap.end());
     };
+    // no launch ends before its work's share per block: lengths whose share is
+    // already worse than the best time need no simulation (of a mixed launch's
+    // 18 lengths, most; the simulation takes milliseconds of host time)
+    auto share = [&](int S) {
+        double w = 0.0;
+        for (int i = 0; i < nslots; ++i) {
+            const int st = strip_of(i, S), c = cols(i);
+            w += rows(i) * (c + kItemCost * ((c + st - 1) / st));
+        }
+        return w / grid;
+    };
     int best = forced > 0 ? forced : 1;
     double best_cost = 1e300;
     for (int S = 1; S <= smax && forced <= 0; ++S) {
+        if (share(S) + kStripCost * S >= best_cost) continue;
         const double cost = finish(S) + kStripCost * S;
         if (cost < best_cost - 1e-9) {
             best_cost = cost;
             best = S;
         }
     }
+    if (chosen) *chosen = best;
     int begin = 0;
     for (int i = 0; i < nslots; ++i) {
         const int st = strip_of(i, best);

@@ -136,7 +136,24 @@ cswgs_status Server::start()
     return CSWGS_OK;
 }
 
-size_t Server::footprint(const HoloSpec &s) const
+// The compressed iterations of a request on the tensor cores, in a server whose
+// shape runs them on the CUDA cores and its full passes on the tensor cores.
+// The shape is tuned for the first request; a CUDA-core compressed iteration
+// costs ~c N per pixel, a tensor-core one ~one step per block of 128 spots, so
+// the requests that follow may belong on the other kernel.  Measured at P =
+// 1152 in full launches: direct phasors 0.95 c N, tensor cores 3.3 (N = 10),
+// 3.8 (100), 11.3 (300) and ~35 (1000) ps per pixel and iteration: they meet
+// at c N = 4 per spot block.  (32 requests of N = 10, 100, 1000 at c = 1/8,
+// N = 10 first: 31 ms with every compressed iteration on the CUDA cores, 11.9
+// with this choice.)
+bool Server::tc_subset(const HoloSpec &s) const
+{
+    if (shape_.fp16 || uses_masks(shape_) || !is_full_tc(shape_.full_threads)) return false;
+    const double c = (double)s.Mp / (double)s.D;
+    return c * s.N > 4.0 * full_tc_spot_blocks(s.N);
+}
+
+size_t Server::footprint(const HoloSpec &s, bool masks) const
 {
     const size_t M = (size_t)s.P * s.P;
     const size_t tiles = (size_t)max_pass_tiles(s, shape_);
@@ -152,7 +169,7 @@ size_t Server::footprint(const HoloSpec &s) const
         b += al256(rw) + al256(c) + al256(cs);
         if (shape_.fp16 && shape_.threads == kSubsetTc) b += al256(cs / 2);
     }
-    if (uses_masks(shape_)) b += al256(sizeof(uint32_t) * (size_t)s.P * mask_words_of(s.P));
+    if (masks) b += al256(sizeof(uint32_t) * (size_t)s.P * mask_words_of(s.P));
     return b;
 }
 
@@ -214,7 +231,7 @@ void Server::place(Req &r)
             o += al256(cs / 2);
         }
     }
-    if (uses_masks(shape_)) {
+    if (uses_masks(shape_) || r.tc_subset) {
         // the subset mask starts clear (each compressed launch's tails clear it again)
         H.mask = reinterpret_cast<uint32_t *>(b + o);
         H.mask_words = mask_words_of(s.P);
@@ -251,7 +268,12 @@ cswgs_status Server::submit(const cswgs_request &q, uint64_t *ticket)
         shape_set_ = true;
         CSWGS_TRY(start());
     }
-    size_t need = footprint(r->spec);
+    r->tc_subset = tc_subset(r->spec);
+    size_t need = footprint(r->spec, uses_masks(shape_) || r->tc_subset);
+    if (r->tc_subset && need > arena_.capacity()) {   // no room for the mask: the shape's own kernel needs none
+        r->tc_subset = false;
+        need = footprint(r->spec, false);
+    }
     if (need > arena_.capacity()) {
         st_.rejected++;
         return set_error(CSWGS_ENOMEM, "request needs %zu device bytes; the serving cap is %zu", need,
@@ -291,7 +313,7 @@ void Server::loop()
     unsigned *queue = queue_d_.as<unsigned>();
     std::unique_lock<std::mutex> lk(mu_);
     int64_t inflight_prev = -1;   // serial of the previous launch, not yet waited for
-    std::map<std::pair<int, int>, int> grid_for;   // (kernel kind, max N) -> resident blocks
+    std::map<std::pair<int, int>, int> grid_for;   // (launch group, max N) -> resident blocks
     // a failed CUDA call is kept: every request finished after it reports CSWGS_ECUDA
     auto chk = [this](cudaError_t e) { note(e); };
     while (true) {
@@ -397,49 +419,64 @@ void Server::loop()
             continue;
         }
         // build launch `serial_`: one slot per request with work left, heaviest
-        // first; compressed-iteration slots first, then full-pass slots, each
-        // group run by its own kernel
+        // first within each group, each group run by its own kernel
         std::vector<Req *> order;
         for (auto &a : active_)
             if (a && !a->cancelled && pass_of(a->spec, a->L) >= 0) order.push_back(a.get());
         std::stable_sort(order.begin(), order.end(), [](Req *a, Req *b) { return a->spec.N > b->spec.N; });
-        int nslots = 0, group_slots[2] = {0, 0}, group_tiles[2] = {0, 0}, group_maxN[2] = {0, 0},
-            group_maxP[2] = {0, 0};
+        // groups: compressed iterations on the shape's kernel, the same on the
+        // tensor cores, full passes
+        constexpr int kGroups = 3;
+        const int kind_of[kGroups] = {kLaunchSubset, kLaunchSubset, kLaunchFull};
+        TileShape tc_shape = shape_;
+        tc_shape.threads = kSubsetTc;
+        tc_shape.ppt = 1;
+        const TileShape group_shape[kGroups] = {shape_, tc_shape, shape_};
+        int nslots = 0, group_slots[kGroups] = {}, group_tiles[kGroups] = {}, group_maxN[kGroups] = {},
+            group_maxP[kGroups] = {};
         std::vector<Req *> finishing;
-        for (int kind = 0; kind < 2; ++kind) {
+        for (int g = 0; g < kGroups; ++g) {
             for (Req *r : order) {
                 const int pass = pass_of(r->spec, r->L);
-                if ((pass == kPassSubset) != (kind == kLaunchSubset)) continue;
+                if ((pass == kPassSubset ? (r->tc_subset ? 1 : 0) : 2) != g) continue;
                 LaunchSlot &sl = sbuf[nslots++];
                 sl.holo = r->slot;
                 sl.pass = pass;
                 sl.j = r->spec.first_j + r->L;
                 sl.count = pass == kPassSubset ? r->spec.Mp : r->spec.D;
-                sl.tiles = pass_tiles(pass, r->spec.P, r->spec.Mp, shape_);
-                sl.tile_begin = group_tiles[kind];
+                sl.tiles = pass_tiles(pass, r->spec.P, r->spec.Mp, group_shape[g]);
+                sl.tile_begin = group_tiles[g];
                 sl.strip = 1;
                 sl.pad = 0;
-                group_tiles[kind] += sl.tiles;
-                group_slots[kind]++;
-                group_maxN[kind] = std::max(group_maxN[kind], r->spec.N);
-                group_maxP[kind] = std::max(group_maxP[kind], r->spec.P);
+                group_tiles[g] += sl.tiles;
+                group_slots[g]++;
+                group_maxN[g] = std::max(group_maxN[g], r->spec.N);
+                group_maxP[g] = std::max(group_maxP[g], r->spec.P);
                 if (pass == kPassFinal) finishing.push_back(r);
             }
         }
-        // the tensor-core kernel takes strips of tiles along a row block
-        for (int kind = 0, first = 0; kind < 2; first += group_slots[kind], ++kind) {
-            if (group_tiles[kind] == 0 || !launch_uses_tc(shape_, kind)) continue;
-            auto key = std::make_pair(kind, group_maxN[kind]);
-            auto g = grid_for.find(key);
-            if (g == grid_for.end())
-                g = grid_for.emplace(key, shape_max_grid(shape_, kind, group_maxN[kind], p_->sm_count)).first;
+        auto grid_of = [&](int g) {
+            auto key = std::make_pair(g, group_maxN[g]);
+            auto it = grid_for.find(key);
+            if (it == grid_for.end())
+                it = grid_for.emplace(key, shape_max_grid(group_shape[g], kind_of[g], group_maxN[g], p_->sm_count)).first;
+            return it->second;
+        };
+        // the tensor-core kernel takes strips of tiles along a row block; a
+        // group of the same sizes as in the step before takes the same ones
+        for (int g = 0, first = 0; g < kGroups; first += group_slots[g], ++g) {
+            if (group_tiles[g] == 0 || !launch_uses_tc(group_shape[g], kind_of[g])) continue;
             std::vector<int> sP, sN;
-            for (int i = first; i < first + group_slots[kind]; ++i) {
+            for (int i = first; i < first + group_slots[g]; ++i) {
                 sP.push_back(master_[sbuf[i].holo].P);
                 sN.push_back(master_[sbuf[i].holo].N);
             }
-            group_tiles[kind] = full_tc_assign_strips(sbuf + first, group_slots[kind], sP.data(), sN.data(),
-                                                      std::max(1, g->second), shape_.strip);
+            StripChoice &ch = strips_[g];
+            const bool same = ch.strip > 0 && ch.P == sP && ch.N == sN;
+            group_tiles[g] = full_tc_assign_strips(sbuf + first, group_slots[g], sP.data(), sN.data(),
+                                                   std::max(1, grid_of(g)), same ? ch.strip : shape_.strip, &ch.strip);
+            ch.P = std::move(sP);
+            ch.N = std::move(sN);
         }
         const int64_t serial = serial_++;
         HoloDev *hbuf = holos_h_[serial & 1];
@@ -455,19 +492,15 @@ void Server::loop()
         }
         chk(cudaMemcpyAsync(sd, sbuf, sizeof(LaunchSlot) * nslots, cudaMemcpyHostToDevice, stream_));
         chk(cudaEventRecord(start_ev_[serial & 1], stream_));
-        for (int kind = 0, first = 0; kind < 2; first += group_slots[kind], ++kind) {
-            if (group_tiles[kind] == 0) continue;
-            auto key = std::make_pair(kind, group_maxN[kind]);
-            auto g = grid_for.find(key);
-            if (g == grid_for.end())
-                g = grid_for.emplace(key, shape_max_grid(shape_, kind, group_maxN[kind], p_->sm_count)).first;
-            if (kind == kLaunchSubset && uses_masks(shape_))
-                chk(launch_tc_mask_scatter(holos, sd + first, group_slots[kind], group_maxP[kind], p_->sm_count,
-                                           stream_));
-            if (launch_uses_tc(shape_, kind))
-                chk(launch_tc_rw_tables(holos, sd + first, group_slots[kind], p_->sm_count, stream_));
-            chk(shape_launch(shape_, kind, holos, sd + first, group_slots[kind], group_tiles[kind], group_maxN[kind],
-                             queue, std::min(g->second, group_tiles[kind]), p_->sm_count, stream_));
+        for (int g = 0, first = 0; g < kGroups; first += group_slots[g], ++g) {
+            if (group_tiles[g] == 0) continue;
+            if (kind_of[g] == kLaunchSubset && uses_masks(group_shape[g]))
+                chk(launch_tc_mask_scatter(holos, sd + first, group_slots[g], group_maxP[g], p_->sm_count, stream_));
+            if (launch_uses_tc(group_shape[g], kind_of[g]))
+                chk(launch_tc_rw_tables(holos, sd + first, group_slots[g], p_->sm_count, stream_));
+            chk(shape_launch(group_shape[g], kind_of[g], holos, sd + first, group_slots[g], group_tiles[g],
+                             group_maxN[g], queue, std::min(grid_of(g), group_tiles[g]), p_->sm_count,
+                             stream_));
         }
         double *mh = met_h_ + (size_t)(serial & 1) * 2 * B;
         for (Req *r : finishing) {

@@ -44,6 +44,7 @@ private:
         size_t off = 0, bytes = 0;
         HoloDev dev{};
         int slot = -1;
+        bool tc_subset = false;          // compressed iterations on the tensor cores, whatever the shape's kernel
         int L = 0;                       // next launch index of this request's schedule
         int64_t last_launch = -1;        // serial of the last launch that used it
         bool cancelled = false;
@@ -51,7 +52,8 @@ private:
         std::vector<double> met;         // host copy of e, u
     };
     void loop();
-    size_t footprint(const HoloSpec &s) const;
+    bool tc_subset(const HoloSpec &s) const;
+    size_t footprint(const HoloSpec &s, bool masks) const;
     void place(Req &r);
     void finish(Req &r, cswgs_status st);
 
@@ -59,6 +61,12 @@ private:
     cudaStream_t stream_ = nullptr;
     Arena arena_;
     TileShape shape_{256, 4};
+    // strip length of each launch group's last composition (sizes in slot order)
+    struct StripChoice {
+        std::vector<int> P, N;
+        int strip = 0;
+    };
+    StripChoice strips_[3];
     bool shape_set_ = false;
     std::thread th_;
     std::mutex mu_;
