@@ -245,30 +245,125 @@ __device__ __forceinline__ void put8h(unsigned char *base, uint32_t stride, uint
     *reinterpret_cast<uint4 *>(base + stride + off) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
 }
 
+// Two FP32 values worked on by one instruction (fma.rn.f32x2 and its kin; each
+// half is rounded like the scalar instruction's result).
+__device__ __forceinline__ uint64_t pack2(float a, float b)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+__device__ __forceinline__ float2 unpack2(uint64_t v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ float rsqrt_approx(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // Eight complex values of u, split for GEMM 2 and packed (the four BF16
 // component rows, or the two FP16 ones), to be stored once their slot is free.
 struct Packed8 {
     uint32_t w[4][4];
 };
 
+// The two values of a BF16 pair as an FP32 pair (a BF16 is an FP32's upper half).
+__device__ __forceinline__ uint64_t bf16x2_floats(uint32_t h)
+{
+    return pack2(__uint_as_float(h << 16), __uint_as_float(h & 0xFFFF0000u));
+}
+
+// |S|^2 of 16 pixels, two by two, and whether every one is a normal FP32
+// number (false for a NaN: min.NaN keeps it).
+__device__ __forceinline__ bool norms16(const float *sr, const float *si, uint64_t *n2)
+{
+    float lo = 1.f, hi = 1.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const uint64_t a = pack2(sr[2 * q], sr[2 * q + 1]), b = pack2(si[2 * q], si[2 * q + 1]);
+        n2[q] = fma2(a, a, mul2(b, b));
+        const float2 n = unpack2(n2[q]);
+        asm("min.NaN.f32 %0, %0, %1;" : "+f"(lo) : "f"(n.x));
+        asm("min.NaN.f32 %0, %0, %1;" : "+f"(lo) : "f"(n.y));
+        hi = fmaxf(hi, fmaxf(n.x, n.y));
+    }
+    return lo >= 1.17549435e-38f && hi <= 3.0e38f;
+}
+
+// Pixels whose |S|^2 is no normal FP32 number: S is scaled by a power of two so
+// that it becomes one (u = S / |S| needs S up to a factor only).  S = 0 has
+// phase 0, and so has an S that is no finite number.
+__device__ __forceinline__ void rescale16(float *sr, float *si, uint64_t *n2)
+{
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        const float2 n = unpack2(n2[e >> 1]);
+        float v = (e & 1) ? n.y : n.x, a = sr[e], b = si[e];
+        if (!(v >= 1.17549435e-38f && v <= 3.0e38f)) {
+            const float f = fmaxf(fabsf(a), fabsf(b)) < 1.f ? 0x1p100f : 0x1p-100f;
+            a *= f;
+            b *= f;
+            v = fmaf(a, a, b * b);
+            if (!(v > 0.f && v <= 3.0e38f)) {
+                a = 1.f;
+                b = 0.f;
+                v = 1.f;
+            }
+        }
+        sr[e] = a;
+        si[e] = b;
+        n2[e >> 1] = (e & 1) ? pack2(n.x, v) : pack2(v, n.y);
+    }
+}
+
+// ur, ui: four pairs each, columns 2q and 2q + 1.
 template <bool F16>
-__device__ __forceinline__ Packed8 pack8(const float2 *v)
+__device__ __forceinline__ Packed8 pack8(const uint64_t *ur, const uint64_t *ui)
 {
     Packed8 p;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const float2 a = v[2 * q], b = v[2 * q + 1];
+        const float2 a = unpack2(ur[q]), b = unpack2(ui[q]);
         if (F16) {
-            p.w[0][q] = h2_bits(__floats2half2_rn(a.x, b.x));
-            p.w[1][q] = h2_bits(__floats2half2_rn(a.y, b.y));
+            p.w[0][q] = h2_bits(__floats2half2_rn(a.x, a.y));
+            p.w[1][q] = h2_bits(__floats2half2_rn(b.x, b.y));
             p.w[2][q] = p.w[3][q] = 0u;
         } else {
-            const __nv_bfloat162 rh = __floats2bfloat162_rn(a.x, b.x), ih = __floats2bfloat162_rn(a.y, b.y);
-            const float2 rf = __bfloat1622float2(rh), jf = __bfloat1622float2(ih);
-            p.w[0][q] = bf16x2_bits(rh);
-            p.w[1][q] = bf16x2_bits(__floats2bfloat162_rn(a.x - rf.x, b.x - rf.y));
-            p.w[2][q] = bf16x2_bits(ih);
-            p.w[3][q] = bf16x2_bits(__floats2bfloat162_rn(a.y - jf.x, b.y - jf.y));
+            const uint32_t rh = bf16x2_bits(__floats2bfloat162_rn(a.x, a.y));
+            const uint32_t ih = bf16x2_bits(__floats2bfloat162_rn(b.x, b.y));
+            const float2 rl = unpack2(sub2(ur[q], bf16x2_floats(rh))), il = unpack2(sub2(ui[q], bf16x2_floats(ih)));
+            p.w[0][q] = rh;
+            p.w[1][q] = bf16x2_bits(__floats2bfloat162_rn(rl.x, rl.y));
+            p.w[2][q] = ih;
+            p.w[3][q] = bf16x2_bits(__floats2bfloat162_rn(il.x, il.y));
         }
     }
     return p;
@@ -1000,12 +1095,14 @@ __device__ __noinline__ void control_load(const HoloDev *__restrict__ holos, con
 
 // The partial V_n = sum_y conj(R_n(y)) Z(n, y) of spot n of a closed Z
 // accumulation (a strip at row block y0) over the tile's 128 rows.  R_n(y)
-// along the rows by recurrence: its phase is quadratic in y, so R(y + 1) =
-// R(y) D(y) and D(y + 1) = D(y) E with the constant E = e^{i (2 pi 2 Gh / 2^32
-// + 2 gl)}; R and D are evaluated directly every 8 rows (the product's
-// rounding grows with the run length).  Every lane computes (a lane past N
-// uses spot N - 1's factors and stores nothing): no divergent branch in the
-// row loop.
+// along the rows by recurrence: its phase is quadratic in y, so R(y + 2) =
+// R(y) D(y) and D(y + 2) = D(y) E with the constant E = e^{i (2 pi 8 Gh / 2^32
+// + 8 gl)}, the even and the odd rows side by side in packed FP32 pairs; R and
+// D are evaluated directly every 16 rows (seven steps: the product's rounding
+// grows with the run length).  Every lane computes (a lane past N uses spot
+// N - 1's factors and stores nothing): no divergent branch in the row loop.
+// A latency-bound chain on one warp per SM quarter: for holograms of more than
+// 128 spots GEMM 2 waits for it, once per spot block.
 __device__ __forceinline__ float2 strip_dot(uint32_t z_re, uint32_t z_im, const int4 *coef, int n, int N, int y0,
                                             int half)
 {
@@ -1013,41 +1110,48 @@ __device__ __forceinline__ float2 strip_dot(uint32_t z_re, uint32_t z_im, const 
     const int32_t tilt = cf.y, Gh = cf.z;
     const float gl = __int_as_float(cf.w);
     float es, ec;
-    sincos_fix(kFixRound + 2u * (uint32_t)Gh, fmaf(2.f, gl, -kTwoPiF), es, ec);
-    float vr0 = 0.f, vi0 = 0.f, vr1 = 0.f, vi1 = 0.f;
+    sincos_fix(kFixRound + 8u * (uint32_t)Gh, fmaf(8.f, gl, -kTwoPiF), es, ec);
+    const uint64_t E_c = pack2(ec, ec), E_s = pack2(es, es), nE_s = pack2(-es, -es);
+    uint64_t vr = 0ull, vi = 0ull;   // even and odd rows; vi is the sum's negative imaginary part
 #pragma unroll 1
     for (int ys = 0; ys < kRows; ys += 16) {
         float zr[16], zi[16];
         ld16(z_re + ys, zr);
         ld16(z_im + ys, zi);
-        float2 r[16];
+        const int u0 = y0 + ys - half;
+        // R at rows u0, u0 + 1 and D there: phase of R(u + 2) / R(u), tilt 2 + Gh (4 u + 4)
+        const float2 p0 = spot_factor(tilt, Gh, gl, u0, kFixRound, 1.f);
+        const float2 p1 = spot_factor(tilt, Gh, gl, u0 + 1, kFixRound, 1.f);
+        float2 d0, d1;
+        sincos_fix(kFixRound + 2u * (uint32_t)tilt + (uint32_t)Gh * (uint32_t)(4 * u0 + 4),
+                   fmaf(gl, (float)(4 * u0 + 4), -kTwoPiF), d0.y, d0.x);
+        sincos_fix(kFixRound + 2u * (uint32_t)tilt + (uint32_t)Gh * (uint32_t)(4 * u0 + 8),
+                   fmaf(gl, (float)(4 * u0 + 8), -kTwoPiF), d1.y, d1.x);
+        uint64_t Rc[8], Rs[8];
+        Rc[0] = pack2(p0.x, p1.x);
+        Rs[0] = pack2(p0.y, p1.y);
+        uint64_t Dc = pack2(d0.x, d1.x), Ds = pack2(d0.y, d1.y);
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int u0 = y0 + ys + 8 * b - half, du = 2 * u0 + 1;
-            float2 pr = spot_factor(tilt, Gh, gl, u0, kFixRound, 1.f);
-            float ds, dc;
-            sincos_fix(kFixRound + (uint32_t)tilt + (uint32_t)Gh * (uint32_t)du, fmaf(gl, (float)du, -kTwoPiF), ds,
-                       dc);
-            float2 d = make_float2(dc, ds);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                r[8 * b + e] = pr;
-                if (e < 7) {
-                    pr = make_float2(fmaf(pr.x, d.x, -pr.y * d.y), fmaf(pr.x, d.y, pr.y * d.x));
-                    d = make_float2(fmaf(d.x, ec, -d.y * es), fmaf(d.x, es, d.y * ec));
-                }
+        for (int q = 0; q < 7; ++q) {
+            const uint64_t nDs = Ds ^ 0x8000000080000000ull;
+            Rc[q + 1] = fma2(Rc[q], Dc, mul2(Rs[q], nDs));
+            Rs[q + 1] = fma2(Rc[q], Ds, mul2(Rs[q], Dc));
+            if (q < 6) {
+                const uint64_t t = fma2(Dc, E_c, mul2(Ds, nE_s));
+                Ds = fma2(Dc, E_s, mul2(Ds, E_c));
+                Dc = t;
             }
         }
         ld_wait();
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            vr0 = fmaf(r[2 * e].x, zr[2 * e], fmaf(r[2 * e].y, zi[2 * e], vr0));
-            vi0 = fmaf(r[2 * e].x, zi[2 * e], fmaf(-r[2 * e].y, zr[2 * e], vi0));
-            vr1 = fmaf(r[2 * e + 1].x, zr[2 * e + 1], fmaf(r[2 * e + 1].y, zi[2 * e + 1], vr1));
-            vi1 = fmaf(r[2 * e + 1].x, zi[2 * e + 1], fmaf(-r[2 * e + 1].y, zr[2 * e + 1], vi1));
+        for (int q = 0; q < 8; ++q) {
+            const uint64_t a = pack2(zr[2 * q], zr[2 * q + 1]), b = pack2(zi[2 * q], zi[2 * q + 1]);
+            vr = fma2(Rc[q], a, fma2(Rs[q], b, vr));
+            vi = fma2(Rs[q], a, fma2(Rc[q] ^ 0x8000000080000000ull, b, vi));
         }
     }
-    return make_float2(vr0 + vr1, vi0 + vi1);
+    const float2 r = unpack2(vr), i = unpack2(vi);
+    return make_float2(r.x + r.y, -(i.x + i.y));
 }
 
 // The columns xl .. xr of grid row gy that lie in the pupil: the grid's, within
@@ -1234,29 +1338,33 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, G2
                     ld16(s_re + lanes + xs, sr);
                     ld16(s_im + lanes + xs, si);
                     ld_wait();
+                    uint64_t n2[8];
+                    const bool normal = norms16(sr, si, n2);
+                    if (!warp_and(normal)) rescale16(sr, si, n2);
                     Packed8 pk[2];
 #pragma unroll
                     for (int g = 0; g < 2; ++g) {
-                        float2 u[8];
+                        uint64_t ur[4], ui[4];
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
+                        for (int e = 0; e < 4; ++e) {
                             // branch-free: the lanes are rows, so a per-pixel branch
-                            // (subset membership, the pupil edge) would diverge
-                            const int jj = 8 * g + e;
-                            const bool valid = ((bits >> jj) & 1u) != 0u;
-                            const float a = sr[jj], b = si[jj];
-                            const float n2 = a * a + b * b;
-                            float amp = 1.f;   // Eq. 3's A
-                            if constexpr (kGauss) {
+                            // (subset membership, the pupil edge) would diverge; a
+                            // pixel without u takes the factor 0
+                            const int jj = 8 * g + 2 * e;
+                            const float2 n = unpack2(n2[jj >> 1]);
+                            float r0 = rsqrt_approx(n.x), r1 = rsqrt_approx(n.y);
+                            if constexpr (kGauss) {   // Eq. 3's A
                                 const int xq = gx0 + jj - half;
-                                amp = exp2f(-kA * (float)(xq * xq + yq2));
+                                r0 *= exp2f(-kA * (float)(xq * xq + yq2));
+                                r1 *= exp2f(-kA * (float)((xq + 1) * (xq + 1) + yq2));
                             }
-                            const bool lit = n2 > 0.f;
-                            const float rs = rsqrtf(n2) * amp;
-                            const float ur = lit ? a * rs : amp, ui = lit ? b * rs : 0.f;   // S = 0: phase 0
-                            u[e] = make_float2(valid ? ur : 0.f, valid ? ui : 0.f);
+                            r0 = ((bits >> jj) & 1u) ? r0 : 0.f;
+                            r1 = ((bits >> (jj + 1)) & 1u) ? r1 : 0.f;
+                            const uint64_t rs = pack2(r0, r1);
+                            ur[e] = mul2(pack2(sr[jj], sr[jj + 1]), rs);
+                            ui[e] = mul2(pack2(si[jj], si[jj + 1]), rs);
                         }
-                        pk[g] = pack8<F16>(u);
+                        pk[g] = pack8<F16>(ur, ui);
                     }
                     // u's slot of this K-step is free once GEMM 2 has read its last
                     // K-step (US earlier in GEMM 2's order: of this tile, or of the
