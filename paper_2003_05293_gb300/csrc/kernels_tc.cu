@@ -501,62 +501,121 @@ __global__ void __launch_bounds__(256) mask_scatter_kernel(const HoloDev *__rest
     if (sl.pass == kPassSubset && H.mask) scatter_subset(H, sl);
 }
 
-// The same masks drawn in shared memory: G CTAs per slot (grid G x slots),
-// each holding the slot's whole mask and taking 1 / G of the Mp draws, each
-// draw an OR in shared memory; the CTA's copy then goes out word by word (G =
-// 1: stored whole, zero words included; G > 1: the non-zero words ORed into
-// the mask, which is clear before).  P^2 / 8 bytes of shared memory: up to P
-// of about 1280.
+// The same masks drawn in shared memory: a cluster of G CTAs per slot (grid G x
+// slots), each holding the slot's whole mask and taking 1 / G of the Mp draws,
+// each draw an OR in shared memory; then each CTA ORs its 1 / G of the words
+// over the cluster (distributed shared memory) and stores them, zero words
+// included.  P^2 / 8 bytes of shared memory: up to P of about 1280.
+// A Feistel round adds F(R), a function of one half only, and a half takes at
+// most P values: the four rounds' F are tabled first (4 P hashes instead of
+// 4 Mp / G; 16 bits an entry, halves and entries carried doubled so that they
+// are byte offsets), and a draw is four table loads, four additions modulo a
+// half's range and the OR.  Bound by the shared-memory path (random 16-bit
+// loads and ORs, three to four lanes to a bank); with the hashes made per draw
+// it was bound by the ALU, and with G > 1 it ended in an OR of every word in
+// global memory: 46.7 us for 64 masks of P = 1152, c = 1/8. (A 64-hologram
+// batch of 31 launches: 11.70 ms with that form, 11.09 with this.)
 constexpr int kLocalThreads = 1024;
+
+// (L + F(R)) mod p with everything doubled: byte offsets into the round tables.
+__device__ __forceinline__ void table_round(uint32_t &L, uint32_t &R, const unsigned char *tab, uint32_t p2)
+{
+    const uint32_t s = L + *reinterpret_cast<const uint16_t *>(tab + R);
+    L = R;
+    R = min(s, s - p2);   // s < 2 p2: the difference wraps past every p2 when s < p2
+}
 
 __global__ void __launch_bounds__(kLocalThreads) mask_local_kernel(const HoloDev *__restrict__ holos,
                                                                    const LaunchSlot *__restrict__ slots)
 {
     extern __shared__ __align__(16) uint32_t s_words[];
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const LaunchSlot sl = slots[blockIdx.y];
-    const HoloDev H = holos[sl.holo];
-    if (sl.pass != kPassSubset || !H.mask) return;
+    const HoloDev &H = holos[sl.holo];
+    if (sl.pass != kPassSubset || !H.mask) return;   // the same in every CTA of the cluster
     const uint32_t G = gridDim.x, x = blockIdx.x;
     const int P = H.P, mw = H.mask_words, words = P * mw;
     const int tid = threadIdx.x;
-    for (int i = tid; i < words; i += kLocalThreads) s_words[i] = 0u;
-    __syncthreads();
+    const uint32_t a = H.fa, b = H.fb, D = (uint32_t)H.D;   // the permutation's rectangle, D <= a b
+    unsigned char *tab = reinterpret_cast<unsigned char *>(s_words + ((words + 3) & ~3));
+    unsigned char *t0 = tab, *t1 = t0 + 2 * b, *t2 = t1 + 2 * a, *t3 = t2 + 2 * b;   // entries: b, a, b, a
     const SubsetDraw d = subset_draw(H, sl.j);
-    const UDiv dP = udiv_of((uint32_t)P);
+    for (int i = tid; i < words; i += kLocalThreads) s_words[i] = 0u;
+    for (uint32_t v = tid; v < max(a, b); v += kLocalThreads) {
+        if (v < b) {
+            reinterpret_cast<uint16_t *>(t0)[v] = (uint16_t)(2u * __umulhi(fmix32(v ^ d.K.k0), a));
+            reinterpret_cast<uint16_t *>(t2)[v] = (uint16_t)(2u * __umulhi(fmix32(v ^ d.K.k2), a));
+        }
+        if (v < a) {
+            reinterpret_cast<uint16_t *>(t1)[v] = (uint16_t)(2u * __umulhi(fmix32(v ^ d.K.k1), b));
+            reinterpret_cast<uint16_t *>(t3)[v] = (uint16_t)(2u * __umulhi(fmix32(v ^ d.K.k3), b));
+        }
+    }
+    __syncthreads();
     const uint32_t k0 = (uint32_t)((uint64_t)H.Mp * x / G), k1 = (uint32_t)((uint64_t)H.Mp * (x + 1) / G);
-    if (H.aperture == 0 && H.fa == (uint32_t)P && H.fb == (uint32_t)P && H.D == P * P) {
-        // the square grid: the permutation's rectangle is the grid, so its
-        // final halves (L, R) are the pixel's row and column (subset_pixel
-        // without the cycle walk, the pupil map and the division by P)
-        const uint32_t D = (uint32_t)H.D;
+    const bool grid = H.aperture == 0 && a == (uint32_t)P && b == (uint32_t)P && D == (uint32_t)P * (uint32_t)P;
+    // this thread's draws, kLocalThreads apart: the halves of each kk = (k + off)
+    // mod D step by a fixed pair (the square grid's D is a multiple of b: the
+    // wrap around D leaves R as it is)
+    if (grid) {
+        const uint32_t p2 = 2u * (uint32_t)P;
+        uint32_t kk = k0 + tid + d.off, r0;
+        kk = kk >= D ? kk - D : kk;
+        uint32_t l0 = 2u * udiv(kk, d.fb, r0);
+        r0 *= 2u;
+        const uint32_t dl = 2u * (kLocalThreads / (uint32_t)P % (uint32_t)P), dr = 2u * (kLocalThreads % (uint32_t)P);
+#pragma unroll 4
         for (uint32_t k = k0 + tid; k < k1; k += kLocalThreads) {
-            uint32_t kk = k + d.off;
-            kk = kk >= D ? kk - D : kk;
-            uint32_t R;
-            uint32_t L = udiv(kk, dP, R);
-            feistel_round(L, R, d.K.k0, (uint32_t)P);
-            feistel_round(L, R, d.K.k1, (uint32_t)P);
-            feistel_round(L, R, d.K.k2, (uint32_t)P);
-            feistel_round(L, R, d.K.k3, (uint32_t)P);
-            atomicOr(s_words + L * (uint32_t)mw + (R >> 5), 1u << (R & 31));
+            uint32_t L = l0, R = r0;
+            table_round(L, R, t0, p2);
+            table_round(L, R, t1, p2);
+            table_round(L, R, t2, p2);
+            table_round(L, R, t3, p2);
+            atomicOr(s_words + (L >> 1) * (uint32_t)mw + (R >> 6), 1u << ((R >> 1) & 31));
+            r0 += dr;
+            l0 += dl;
+            if (r0 >= p2) {
+                r0 -= p2;
+                l0 += 2u;
+            }
+            l0 = l0 >= p2 ? l0 - p2 : l0;
         }
     } else {
+        const UDiv dP = udiv_of((uint32_t)P);
+        const uint32_t a2 = 2u * a, b2 = 2u * b, extra = a * b - D;
+        auto permute_tab = [&](uint32_t y) {
+            uint32_t R;
+            uint32_t L = 2u * udiv(y, d.fb, R);
+            R *= 2u;
+            table_round(L, R, t0, a2);
+            table_round(L, R, t1, b2);
+            table_round(L, R, t2, a2);
+            table_round(L, R, t3, b2);
+            return (L >> 1) * b + (R >> 1);
+        };
         for (uint32_t k = k0 + tid; k < k1; k += kLocalThreads) {
-            const uint32_t m = subset_pixel(H, d, k);
+            uint32_t y = k + d.off;
+            y = permute_tab(y >= D ? y - D : y);
+            for (uint32_t w = 0; y >= D && w < extra; ++w) y = permute_tab(y);   // cycle walk (permute_domain)
+            const uint32_t m = pupil_pixel(H, y < D ? y : 0u);
             uint32_t c;
             const uint32_t r = udiv(m, dP, c);
             atomicOr(s_words + r * (uint32_t)mw + (c >> 5), 1u << (c & 31));
         }
     }
-    __syncthreads();
     uint32_t *g = subset_mask(H, sl.j);
     if (G == 1) {
+        __syncthreads();
         for (int i = tid; i < words; i += kLocalThreads) g[i] = s_words[i];
     } else {
-        for (int i = tid; i < words; i += kLocalThreads) {
-            const uint32_t v = s_words[i];
-            if (v) atomicOr(g + i, v);
+        cluster.sync();
+        const int i1 = (int)((int64_t)words * (x + 1) / G);
+        for (int i = (int)((int64_t)words * x / G) + tid; i < i1; i += kLocalThreads) {
+            uint32_t v = 0u;
+            for (uint32_t q = 0; q < G; ++q) v |= cluster.map_shared_rank(s_words, q)[i];
+            g[i] = v;
         }
+        cluster.sync();   // every CTA's words are read before it leaves
     }
 }
 
@@ -1942,18 +2001,20 @@ cudaError_t launch_tc_rw_tables(const HoloDev *holos, const LaunchSlot *slots, i
 }
 
 // The shared-memory form of the mask draw for a launch whose holograms are
-// at most maxP pixels a side: the CTAs per slot (about one wave over the
-// SMs), or 0 when the mask does not fit a CTA's shared memory or the launch
-// has too few holograms for it: every CTA also clears and writes out a whole
-// mask, so past 8 CTAs per hologram the global bit sets of
-// mask_scatter_kernel (a few hundred thousand draws spread over every SM)
-// cost less.
+// at most maxP pixels a side: the CTAs per slot (a cluster: 1, 2, 4 or 8, about
+// one wave over the SMs), or 0 when the mask and the round tables do not fit a
+// CTA's shared memory or the launch has too few holograms for it: every CTA
+// clears a whole mask, and 8 of them per hologram must still fill half the
+// SMs; below that the global bit sets of mask_scatter_kernel (a few hundred
+// thousand draws spread over every SM) cost less.
 static int mask_local_shape(int maxP, int nslots, int sm_count, size_t *smem)
 {
-    const int G = std::max(1, sm_count / std::max(1, nslots));
-    if (G > 8) return 0;
-    *smem = (size_t)maxP * (size_t)mask_words_of(maxP) * 4;
-    if (*smem > 200 * 1024) return 0;
+    if (16 * nslots < sm_count) return 0;
+    int G = 8;
+    while (G > 1 && G * nslots > sm_count) G >>= 1;
+    // the mask, and four tables of at most maxP 16-bit entries (doubled: below 2^16)
+    *smem = (((size_t)maxP * (size_t)mask_words_of(maxP) + 3) & ~(size_t)3) * 4 + 4 * 2 * (size_t)(maxP + 1);
+    if (*smem > 220 * 1024) return 0;
     if (cudaFuncSetAttribute(tc::mask_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem) !=
         cudaSuccess) {
         (void)cudaGetLastError();
@@ -1969,8 +2030,18 @@ cudaError_t launch_tc_mask_scatter(const HoloDev *holos, const LaunchSlot *slots
     (void)cudaGetLastError();
     size_t smem = 0;
     if (const int G = mask_local_shape(maxP, nslots, sm_count, &smem)) {
-        tc::mask_local_kernel<<<dim3((unsigned)G, (unsigned)nslots), tc::kLocalThreads, smem, s>>>(holos, slots);
-        return cudaGetLastError();
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)G;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)G, (unsigned)nslots);
+        cfg.blockDim = dim3(tc::kLocalThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, tc::mask_local_kernel, holos, slots);
     }
     // a launch of few holograms (or holograms too large for the shared-memory
     // form): four blocks per SM over the launch, the draws' latency spread wide

@@ -49,3 +49,27 @@ def test_update_and_metrics(plan, P, N, full):
     assert math.sqrt(np.mean((r["w"] / ref["w"] - 1) ** 2)) < TOL_PHASE_RMS
     assert abs(r["e"] - ref["e"]) < TOL_EU and abs(r["u"] - ref["u"]) < TOL_EU
     assert abs(float(np.sum(r["I"])) - r["e"]) < 1e-12 * N
+
+
+@pytest.mark.parametrize("count", [3, 20, 80])
+def test_batch_tails_and_masks(plan, count):
+    """Batches that take clusters of 8, 4 and 1 blocks, and subset masks drawn
+    in global memory or in the shared memory of 4 and 1 blocks: each hologram
+    of uneven size against the oracle."""
+    rng = np.random.default_rng(count)
+    pbs = []
+    for i in range(count):
+        pb = workloads.problem(int(rng.choice([64, 98, 160, 258])), int(rng.integers(1, 40)), 5.0, 0.25, 4,
+                               seed=900 + i)
+        if i % 3 == 1:
+            pb.extra = dict(aperture="round", waist=0.6 * pb.P, subset_mode="windows" if i % 2 else "fresh")
+        pbs.append(pb)
+    b = plan.batch(pbs, None)
+    b.run()
+    got = b.results()
+    for pb, g in zip(pbs, got):
+        ex = getattr(pb, "extra", None) or {}
+        ref = oracle.solve(pb.P, pb.xyz, c=pb.c, iterations=pb.iterations, seed=pb.seed, **(
+            dict(aperture=ex["aperture"], waist=ex["waist"], subset_mode=ex["subset_mode"]) if ex else {}))
+        assert abs(g["e"] - ref["e"]) < TOL_EU and abs(g["u"] - ref["u"]) < TOL_EU
+    b.close()
