@@ -497,7 +497,8 @@ void Server::loop()
             if (kind_of[g] == kLaunchSubset && uses_masks(group_shape[g]))
                 chk(launch_tc_mask_scatter(holos, sd + first, group_slots[g], group_maxP[g], p_->sm_count, stream_));
             if (launch_uses_tc(group_shape[g], kind_of[g]))
-                chk(launch_tc_rw_tables(holos, sd + first, group_slots[g], p_->sm_count, stream_));
+                chk(launch_tc_rw_tables(holos, sd + first, group_slots[g], group_maxP[g], group_maxN[g], p_->sm_count,
+                                        stream_));
             chk(shape_launch(group_shape[g], kind_of[g], holos, sd + first, group_slots[g], group_tiles[g],
                              group_maxN[g], queue, std::min(grid_of(g), group_tiles[g]), p_->sm_count,
                              stream_));

@@ -67,9 +67,26 @@ def test_batch_tails_and_masks(plan, count):
     b = plan.batch(pbs, None)
     b.run()
     got = b.results()
+    b.close()
     for pb, g in zip(pbs, got):
         ex = getattr(pb, "extra", None) or {}
         ref = oracle.solve(pb.P, pb.xyz, c=pb.c, iterations=pb.iterations, seed=pb.seed, **(
             dict(aperture=ex["aperture"], waist=ex["waist"], subset_mode=ex["subset_mode"]) if ex else {}))
         assert abs(g["e"] - ref["e"]) < TOL_EU and abs(g["u"] - ref["u"]) < TOL_EU
-    b.close()
+
+
+@pytest.mark.parametrize("scale", [1e-25, 1e-12, 1.0, 1e18])
+def test_amplitude_scale(plan, scale):
+    """u = S / |S| and the phase map do not depend on the amplitudes' scale, also
+    where |S|^2 leaves FP32's normal range; a weak spot among strong ones keeps
+    its phase."""
+    P, N = 192, 20
+    pb = workloads.problem(P, N, 5.0, 0.25, 3, seed=77)
+    amp = np.linspace(0.5, 1.5, N) * scale
+    amp[3] *= 1e-3
+    out = torch.empty(pb.M, dtype=torch.float32, device="cuda")
+    r = plan.solve(pb.xyz, P, pb.c, 3, pb.seed, amp=amp, out=out, state=True)
+    ref = oracle.solve(P, pb.xyz, amp / scale, c=pb.c, iterations=3, seed=pb.seed)
+    assert rms_wrapped(r["theta"], ref["theta"]) < TOL_PHASE_RMS
+    assert rms_wrapped(out.cpu().numpy(), ref["phase"]) < TOL_PHASE_RMS
+    assert abs(r["e"] - ref["e"]) < TOL_EU and abs(r["u"] - ref["u"]) < TOL_EU
