@@ -828,7 +828,7 @@ def main():
                                         TRAFFIC_SUB, args),
             "roofline_full_passes": full_roofline(tile, fma_achieved, fma_peak, sm_count, max_mhz, TRAFFIC_FULL,
                                                   n_full_launches, full_ms),
-            "gpu_launches": args.steps * launches_per_step(tile, n_sub, n_full_launches),
+            "gpu_launches": args.steps * (launches_per_step(tile, n_sub, n_full_launches) + 1),   # and the results kernel
             "kernel_times_from": "CUDA events recorded inside the graph around each launch, last timed step",
             "clocks": clk}
 

@@ -151,7 +151,10 @@ static cswgs_status copy_maps(cswgs_plan_s *p, DevBuf &buf, const std::vector<Ma
     return CSWGS_OK;
 }
 
-// FP32 solver: one hologram through a cached single-hologram batch.
+// FP32 solver: one hologram through a cached single-hologram batch.  The
+// inputs go up at the start of the batch's graph and the results come back
+// through its pinned block, so that a call is one graph launch and one
+// synchronisation.
 static cswgs_status solve_fp32(cswgs_plan_s *p, HoloSpec h, float *phase_out, int out_on_host,
                                double *e, double *u, double *final_w, double *final_theta,
                                double *spot_intensity)
@@ -166,6 +169,7 @@ static cswgs_status solve_fp32(cswgs_plan_s *p, HoloSpec h, float *phase_out, in
         std::unique_ptr<Fp32Batch> nb;
         CSWGS_TRY(batch_build_host(p, v, false, host_out, &nb));
         b = nb.get();
+        b->upload_in_graph = true;
         p->solve_cache[key] = std::move(nb);
     } else {
         b = it->second.get();
@@ -173,39 +177,29 @@ static cswgs_status solve_fp32(cswgs_plan_s *p, HoloSpec h, float *phase_out, in
         b->holos[0].seed = b->specs[0].seed;
         fill_pupil(b->holos[0], b->specs[0]);
         batch_restage(b, 0);
-        // the seed, the beam and the SLM frame live in the device hologram record
-        CSWGS_CUDA_TRY(cudaMemcpyAsync(b->holos_d.p, b->holos.data(), sizeof(HoloDev), cudaMemcpyHostToDevice,
-                                       p->stream));
     }
     cudaStream_t s = p->stream;
-    CSWGS_TRY(batch_upload_inputs(b, s));
-    std::vector<float *> outs{host_out ? nullptr : phase_out};
-    CSWGS_TRY(batch_set_outputs(b, outs, s));
+    // the seed, the beam, the SLM frame and the output live in the hologram record
+    b->holos[0].phase_out = host_out || !phase_out ? b->own_phase[0] : phase_out;
+    std::memcpy(static_cast<char *>(b->staging) + b->in_bytes, b->holos.data(), sizeof(HoloDev));
     CSWGS_TRY(batch_enqueue(b, s));
-    const HoloDev &H = b->holos[0];
-    std::vector<double> met(2 + N);
-    std::vector<SpotState> st(N);
-    if (b->specs[0].final_pass) {
-        CSWGS_CUDA_TRY(cudaMemcpyAsync(met.data(), H.metrics, sizeof(double) * (2 + N), cudaMemcpyDeviceToHost, s));
-        if (host_out) {
-            const size_t n = (size_t)H.P * H.P;
-            if (float *d = host_direct(p, phase_out))
-                CSWGS_TRY(copy_maps(p, b->copy_jobs, {MapCopy{b->own_phase[0], d, n}}, s));
-            else
-                CSWGS_CUDA_TRY(cudaMemcpyAsync(phase_out, b->own_phase[0], sizeof(float) * n, cudaMemcpyDeviceToHost, s));
-        }
+    if (b->specs[0].final_pass && host_out) {
+        const size_t n = (size_t)b->holos[0].P * b->holos[0].P;
+        if (float *d = host_direct(p, phase_out))
+            CSWGS_TRY(copy_maps(p, b->copy_jobs, {MapCopy{b->own_phase[0], d, n}}, s));
+        else
+            CSWGS_CUDA_TRY(cudaMemcpyAsync(phase_out, b->own_phase[0], sizeof(float) * n, cudaMemcpyDeviceToHost, s));
     }
-    if (final_w || final_theta)
-        CSWGS_CUDA_TRY(cudaMemcpyAsync(st.data(), H.state, sizeof(SpotState) * N, cudaMemcpyDeviceToHost, s));
     CSWGS_TRY(batch_status(b, s));
+    const SpotState *st = b->result_state();
     for (int n = 0; n < N; ++n) {
         if (final_w) final_w[n] = (double)st[n].w;
         if (final_theta) final_theta[n] = (double)(int32_t)st[n].theta * (2.0 * M_PI / 4294967296.0);
     }
     if (b->specs[0].final_pass) {
-        if (e) *e = met[0];
-        if (u) *u = met[1];
-        if (spot_intensity) std::memcpy(spot_intensity, met.data() + 2, sizeof(double) * N);
+        if (e) *e = b->result_eu(0)[0];
+        if (u) *u = b->result_eu(0)[1];
+        if (spot_intensity) std::memcpy(spot_intensity, b->result_intensity(), sizeof(double) * N);
     }
     return CSWGS_OK;
 }
@@ -214,17 +208,6 @@ static cswgs_status set_device(cswgs_plan_s *p)
 {
     CSWGS_CUDA_TRY(cudaSetDevice(p->device));
     return CSWGS_OK;
-}
-
-// e and u of every hologram of a batch into one host block (pinned memory,
-// written through its device address): one launch instead of a copy per
-// hologram.
-__global__ void eu_gather_kernel(const HoloDev *__restrict__ holos, int count, double *dst)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-        dst[2 * i] = holos[i].metrics[0];
-        dst[2 * i + 1] = holos[i].metrics[1];
-    }
 }
 
 // A request of a host-buffer batch's update must keep the batch's shape.
@@ -242,7 +225,6 @@ cswgs_batch_s::~cswgs_batch_s()
     if (stream) cudaStreamSynchronize(stream);
     b.reset();
     if (ev_in) cudaEventDestroy(ev_in);
-    if (eu_host) cudaFreeHost(eu_host);
     if (stream) cudaStreamDestroy(stream);
 }
 
@@ -533,15 +515,13 @@ cswgs_status cswgs_batch_run(cswgs_batch b)
     std::lock_guard<std::mutex> lk(p->mu);
     CSWGS_TRY(set_device(p));
     if (!b->host) return batch_enqueue(b->b.get(), p->stream);
-    // host-buffer batch, all on its own stream: staged inputs in, the graph,
-    // e and u out, the phase maps out
+    // host-buffer batch, all on its own stream: staged inputs in, the graph
+    // (e and u out with it), the phase maps out
     Fp32Batch *fb = b->b.get();
     cudaStream_t s = b->stream;
     CSWGS_TRY(batch_upload_inputs(fb, s));
     CSWGS_CUDA_TRY(cudaEventRecord(b->ev_in, s));
     CSWGS_TRY(batch_enqueue(fb, s));
-    eu_gather_kernel<<<1, 128, 0, s>>>(fb->holos_d.as<HoloDev>(), b->count, b->eu_host);
-    CSWGS_CUDA_TRY(cudaGetLastError());
     // pinned maps go out on the copy engines: host batches are meant to
     // alternate, and the engines leave the SMs to the other batch's
     // iterations (the copy kernel would share them); pageable maps the GPU can
@@ -581,10 +561,7 @@ static cswgs_status host_batch_fill(cswgs_batch b, const cswgs_request *reqs, st
         }
         b->host_out[i] = reqs[i].phase_out;
     }
-    if (changed)
-        CSWGS_CUDA_TRY(cudaMemcpyAsync(fb->holos_d.p, fb->holos.data(), sizeof(HoloDev) * b->count,
-                                       cudaMemcpyHostToDevice, b->stream));
-    return CSWGS_OK;
+    return changed ? batch_upload_records(fb, b->stream) : CSWGS_OK;
 }
 
 cswgs_status cswgs_batch_create_host(cswgs_plan p, const cswgs_request *reqs, int count, cswgs_batch *out)
@@ -614,8 +591,6 @@ cswgs_status cswgs_batch_create_host(cswgs_plan p, const cswgs_request *reqs, in
     };
     if (st == CSWGS_OK) cuda(cudaStreamCreateWithFlags(&bb->stream, cudaStreamNonBlocking), "stream");
     if (st == CSWGS_OK) cuda(cudaEventCreateWithFlags(&bb->ev_in, cudaEventDisableTiming), "event");
-    if (st == CSWGS_OK)
-        cuda(cudaMallocHost(reinterpret_cast<void **>(&bb->eu_host), sizeof(double) * 2 * count), "pinned e, u");
     if (st == CSWGS_OK) st = host_batch_fill(bb, reqs, specs, true);
     if (st == CSWGS_OK) st = batch_set_outputs(bb->b.get(), std::vector<float *>(count, nullptr), bb->stream);
     if (st == CSWGS_OK) cuda(cudaStreamSynchronize(bb->stream), "set-up");
@@ -649,30 +624,13 @@ cswgs_status cswgs_batch_results(cswgs_batch b, cswgs_result *results)
     std::lock_guard<std::mutex> lk(p->mu);
     CSWGS_TRY(set_device(p));
     Fp32Batch *fb = b->b.get();
-    if (b->host) {
-        CSWGS_TRY(batch_status(fb, b->stream));   // synchronises the batch's stream
-        float ms = 0.f;
-        if (fb->timing) cudaEventElapsedTime(&ms, fb->events.front(), fb->events.back());
-        for (int i = 0; i < b->count; ++i) {
-            results[i].status = CSWGS_OK;
-            results[i].e = b->eu_host[2 * i];
-            results[i].u = b->eu_host[2 * i + 1];
-            results[i].latency_ms = ms;
-            results[i].queue_ms = 0.0;
-        }
-        return CSWGS_OK;
-    }
-    std::vector<double> eu(2 * b->count);
-    for (int i = 0; i < b->count; ++i)
-        CSWGS_CUDA_TRY(cudaMemcpyAsync(&eu[2 * i], fb->holos[i].metrics, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                                       p->stream));
-    CSWGS_TRY(batch_status(fb, p->stream));
+    CSWGS_TRY(batch_status(fb, b->host ? b->stream : p->stream));   // synchronises the batch's stream
     float ms = 0.f;
     if (fb->timing) cudaEventElapsedTime(&ms, fb->events.front(), fb->events.back());
     for (int i = 0; i < b->count; ++i) {
         results[i].status = CSWGS_OK;
-        results[i].e = eu[2 * i];
-        results[i].u = eu[2 * i + 1];
+        results[i].e = fb->result_eu(i)[0];
+        results[i].u = fb->result_eu(i)[1];
         results[i].latency_ms = ms;
         results[i].queue_ms = 0.0;
     }
@@ -786,9 +744,7 @@ cswgs_status cswgs_solve_batch(cswgs_plan p, const cswgs_request *reqs, int coun
             }
             batch_restage(b, i);
         }
-        if (changed)
-            CSWGS_CUDA_TRY(cudaMemcpyAsync(b->holos_d.p, b->holos.data(), sizeof(HoloDev) * count,
-                                           cudaMemcpyHostToDevice, p->stream));
+        if (changed) CSWGS_TRY(batch_upload_records(b, p->stream));
     }
     cudaStream_t s = p->stream;
     CSWGS_TRY(batch_upload_inputs(b, s));
@@ -796,10 +752,8 @@ cswgs_status cswgs_solve_batch(cswgs_plan p, const cswgs_request *reqs, int coun
     for (int i = 0; i < count; ++i) outs[i] = (reqs[i].out_on_host ? nullptr : reqs[i].phase_out);
     CSWGS_TRY(batch_set_outputs(b, outs, s));
     CSWGS_TRY(batch_enqueue(b, s));
-    std::vector<double> eu(2 * count);
     std::vector<MapCopy> jobs;
     for (int i = 0; i < count; ++i) {
-        CSWGS_CUDA_TRY(cudaMemcpyAsync(&eu[2 * i], b->holos[i].metrics, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
         if (reqs[i].out_on_host && reqs[i].phase_out) {
             const size_t n = (size_t)specs[i].P * specs[i].P;
             if (float *d = host_direct(p, reqs[i].phase_out))
@@ -815,8 +769,8 @@ cswgs_status cswgs_solve_batch(cswgs_plan p, const cswgs_request *reqs, int coun
     cudaEventElapsedTime(&ms, b->events.front(), b->events.back());
     for (int i = 0; i < count; ++i) {
         results[i].status = CSWGS_OK;
-        results[i].e = eu[2 * i];
-        results[i].u = eu[2 * i + 1];
+        results[i].e = b->result_eu(i)[0];
+        results[i].u = b->result_eu(i)[1];
         results[i].latency_ms = ms;
         results[i].queue_ms = 0.0;
     }

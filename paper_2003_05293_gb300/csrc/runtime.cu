@@ -303,8 +303,10 @@ static cswgs_status batch_build_shape(cswgs_plan_s *p, std::vector<HoloSpec> spe
         if (s.has_init_th) in += align256(sizeof(double) * s.N);
     }
     b->in_bytes = in;
+    const size_t holos_off = in;
+    b->up_bytes = in + align256(sizeof(HoloDev) * count);
     // work buffers
-    size_t work = in;
+    size_t work = b->up_bytes;
     std::vector<size_t> w_off(count);
     b->maxN = 0;
     for (int h = 0; h < count; ++h) {
@@ -339,7 +341,12 @@ static cswgs_status batch_build_shape(cswgs_plan_s *p, std::vector<HoloSpec> spe
         }
     b->mask_bytes = work - b->mask_begin;
     CSWGS_TRY(b->mem.ensure(work));
-    CSWGS_CUDA_TRY(cudaMallocHost(&b->staging, std::max<size_t>(in, 256)));
+    size_t res = 1 + 2 * (size_t)count;   // doubles: status, e and u, a single hologram's I_n and states
+    if (count == 1) res += (size_t)b->maxN * (1 + sizeof(SpotState) / sizeof(double));
+    CSWGS_CUDA_TRY(cudaMallocHost(&b->staging, b->up_bytes + sizeof(double) * res));
+    b->results = reinterpret_cast<double *>(static_cast<char *>(b->staging) + b->up_bytes);
+    std::memset(b->results, 0, sizeof(double) * res);
+    b->holos_d = reinterpret_cast<HoloDev *>(b->mem.as<char>() + holos_off);
 
     char *base = b->mem.as<char>();
     char *stg = static_cast<char *>(b->staging);
@@ -482,15 +489,14 @@ static cswgs_status batch_build_shape(cswgs_plan_s *p, std::vector<HoloSpec> spe
     }
     b->pairs_total = pairs_total;
     b->pairs_iter = pairs_iter;
-    CSWGS_TRY(b->holos_d.ensure(sizeof(HoloDev) * count));
     CSWGS_TRY(b->slots_d.ensure(sizeof(LaunchSlot) * std::max<size_t>(1, slots.size())));
     CSWGS_TRY(b->queue_d.ensure(256));
-    CSWGS_CUDA_TRY(cudaMemcpy(b->holos_d.p, b->holos.data(), sizeof(HoloDev) * count, cudaMemcpyHostToDevice));
     if (!slots.empty())
         CSWGS_CUDA_TRY(cudaMemcpy(b->slots_d.p, slots.data(), sizeof(LaunchSlot) * slots.size(),
                                   cudaMemcpyHostToDevice));
     CSWGS_CUDA_TRY(cudaMemset(b->queue_d.p, 0, 256));
     CSWGS_CUDA_TRY(cudaMemset(b->mem.p, 0, work));
+    CSWGS_CUDA_TRY(cudaMemcpy(b->holos_d, b->holos.data(), sizeof(HoloDev) * count, cudaMemcpyHostToDevice));
     if (timing) {
         b->events.resize(L_max + 2);   // before the preparation, before each step, after the last
         for (auto &e : b->events) CSWGS_CUDA_TRY(cudaEventCreate(&e));
@@ -550,9 +556,8 @@ void batch_restage(Fp32Batch *b, int h)
 
 cswgs_status batch_status(Fp32Batch *b, cudaStream_t s)
 {
-    unsigned st = 0;
-    CSWGS_CUDA_TRY(cudaMemcpyAsync(&st, b->queue_d.as<unsigned>() + 2, sizeof st, cudaMemcpyDeviceToHost, s));
     CSWGS_CUDA_TRY(cudaStreamSynchronize(s));
+    const unsigned st = *reinterpret_cast<const unsigned *>(b->results);
     if (st) return set_error(CSWGS_ETIMEOUT, "a bounded wait inside the tensor-core kernel ran out (status %u)", st);
     return CSWGS_OK;
 }
@@ -564,6 +569,28 @@ cswgs_status batch_upload_inputs(Fp32Batch *b, cudaStream_t s)
     return CSWGS_OK;
 }
 
+cswgs_status batch_upload_records(Fp32Batch *b, cudaStream_t s)
+{
+    CSWGS_CUDA_TRY(cudaMemcpyAsync(b->holos_d, b->holos.data(), sizeof(HoloDev) * b->holos.size(),
+                                   cudaMemcpyHostToDevice, s));
+    return CSWGS_OK;
+}
+
+// The last kernel of a run: its results into pinned host memory (a single
+// hologram's I_n and spot states too).
+__global__ void __launch_bounds__(256) results_kernel(const HoloDev *__restrict__ holos, int count,
+                                                      const unsigned *status, double *dst)
+{
+    if (threadIdx.x == 0) *reinterpret_cast<unsigned *>(dst) = *status;
+    for (int i = threadIdx.x; i < 2 * count; i += 256) dst[1 + i] = holos[i >> 1].metrics[i & 1];
+    if (count != 1) return;
+    const int N = holos[0].N;
+    const double *state = reinterpret_cast<const double *>(holos[0].state);
+    for (int n = threadIdx.x; n < N; n += 256) dst[3 + n] = holos[0].metrics[2 + n];
+    for (int n = threadIdx.x; n < 2 * N; n += 256) dst[3 + N + n] = state[n];
+}
+static_assert(sizeof(SpotState) == 2 * sizeof(double), "states are copied as pairs of 8 bytes");
+
 cswgs_status batch_set_outputs(Fp32Batch *b, const std::vector<float *> &dev_phase, cudaStream_t s)
 {
     bool changed = false;
@@ -574,20 +601,19 @@ cswgs_status batch_set_outputs(Fp32Batch *b, const std::vector<float *> &dev_pha
             changed = true;
         }
     }
-    if (changed)
-        CSWGS_CUDA_TRY(cudaMemcpyAsync(b->holos_d.p, b->holos.data(), sizeof(HoloDev) * b->holos.size(),
-                                       cudaMemcpyHostToDevice, s));
-    return CSWGS_OK;
+    return changed ? batch_upload_records(b, s) : CSWGS_OK;
 }
 
 cswgs_status batch_enqueue_direct(Fp32Batch *b, cudaStream_t s, bool capturing)
 {
     // inside a stream capture the timing events become event-record nodes
     const unsigned evflag = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
-    const HoloDev *holos = b->holos_d.as<HoloDev>();
+    const HoloDev *holos = b->holos_d;
     const LaunchSlot *slots = b->slots_d.as<LaunchSlot>();
     unsigned *queue = b->queue_d.as<unsigned>();
     const int count = (int)b->holos.size();
+    if (b->upload_in_graph)
+        CSWGS_CUDA_TRY(cudaMemcpyAsync(b->mem.p, b->staging, b->up_bytes, cudaMemcpyHostToDevice, s));
     // work queue, blocks done, status word (a bounded wait inside a kernel that ran out)
     CSWGS_CUDA_TRY(cudaMemsetAsync(queue, 0, 3 * sizeof(unsigned), s));
     if (b->mask_bytes) CSWGS_CUDA_TRY(cudaMemsetAsync(b->mem.as<char>() + b->mask_begin, 0, b->mask_bytes, s));
@@ -642,6 +668,8 @@ cswgs_status batch_enqueue_direct(Fp32Batch *b, cudaStream_t s, bool capturing)
         }
     }
     if (b->timing) CSWGS_CUDA_TRY(cudaEventRecordWithFlags(b->events[steps + 1], s, evflag));
+    results_kernel<<<1, 256, 0, s>>>(holos, count, queue + 2, b->results);
+    CSWGS_CUDA_TRY(cudaGetLastError());
     return CSWGS_OK;
 }
 

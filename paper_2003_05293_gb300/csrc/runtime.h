@@ -110,8 +110,23 @@ struct Fp32Batch {
     std::vector<size_t> in_off;           // per hologram: offset of its inputs in the staging block
     size_t in_bytes = 0;                  // size of the input block (device + pinned staging)
     DevBuf mem;                           // all per-hologram buffers
-    DevBuf holos_d, slots_d, queue_d;
-    void *staging = nullptr;              // pinned host copy of the inputs
+    HoloDev *holos_d = nullptr;           // device hologram records, behind the inputs in mem
+    size_t up_bytes = 0;                  // the inputs and the records (device + pinned staging)
+    DevBuf slots_d, queue_d;
+    void *staging = nullptr;              // pinned: the inputs, the records, the results
+    // Results of the last run, written by its last kernel into the pinned
+    // block: the status word, {e, u} per hologram, and for a batch of one
+    // hologram I_n and the spot states.  One synchronisation hands them all
+    // over (a copy from device memory per value took ~14 us of host time each:
+    // a 64-hologram batch spent 0.5 ms of 11.9 on its e and u).
+    double *results = nullptr;
+    const double *result_eu(int h) const { return results + 1 + 2 * h; }
+    const double *result_intensity() const { return results + 1 + 2 * holos.size(); }
+    const SpotState *result_state() const
+    {
+        return reinterpret_cast<const SpotState *>(result_intensity() + holos[0].N);
+    }
+    bool upload_in_graph = false;         // every run starts with the upload of inputs and records
     std::vector<float *> own_phase;       // internal phase buffers (host outputs), per hologram
     std::vector<int> l_slot0, l_nslots, l_tiles, l_maxN, l_maxP;   // per (step, kernel kind)
     TileShape shape{256, 4, 256};
@@ -138,6 +153,7 @@ struct Fp32Batch {
 cswgs_status batch_build(cswgs_plan_s *p, std::vector<HoloSpec> specs, bool timing,
                          std::unique_ptr<Fp32Batch> *out);
 cswgs_status batch_upload_inputs(Fp32Batch *b, cudaStream_t s);
+cswgs_status batch_upload_records(Fp32Batch *b, cudaStream_t s);   // the hologram records, from their host mirror
 // CSWGS_ETIMEOUT when a bounded wait inside a kernel of the batch ran out (synchronises s)
 cswgs_status batch_status(Fp32Batch *b, cudaStream_t s);
 cswgs_status batch_set_outputs(Fp32Batch *b, const std::vector<float *> &dev_phase, cudaStream_t s);
@@ -183,7 +199,6 @@ struct cswgs_batch_s {
     bool host = false;
     cudaStream_t stream = nullptr;
     cudaEvent_t ev_in = nullptr;          // the last run has read the staged inputs
-    double *eu_host = nullptr;            // pinned, 2 per hologram
     std::vector<float *> host_out;        // per hologram: host phase map of the next run, or NULL
     cswgs::DevBuf jobs;                   // map copies of the last run
     ~cswgs_batch_s();
