@@ -140,9 +140,7 @@ struct Fp32Batch {
     size_t mask_begin = 0, mask_bytes = 0;   // subset masks (cleared at the start of every run)
     // the next compressed launch's subset masks are drawn on a side stream
     // (two masks per hologram, by the parity of j), beside the tails and the
-    // R' tables between launches, when every hologram has the square
-    // aperture; a round pupil's draws (a row search each) run on the main
-    // stream before the launch
+    // R' tables between launches
     cudaStream_t side = nullptr;
     cudaEvent_t ev_start = nullptr, ev_tail[2] = {nullptr, nullptr}, ev_scat[2] = {nullptr, nullptr};
     DevBuf copy_jobs;   // host phase maps written out by the copy kernel (cswgs_solve_batch)
