@@ -1695,13 +1695,8 @@ __device__ __forceinline__ float4 tail_warp_sum(const HoloDev &H, int n, int g, 
 
 __device__ __forceinline__ double2 tail_warp_sum64(const HoloDev &H, int n, int g, int G, int tiles)
 {
-    double vr = 0.0, vi = 0.0;
-#pragma unroll 4
-    for (int t = g; t < tiles; t += G) {
-        const double2 p = __ldcg(&H.part64[(size_t)t * H.N + n]);
-        vr += p.x;
-        vi += p.y;
-    }
+    const double2 v = tile_sum64(H.part64 + n, H.N, g, G, tiles);
+    double vr = v.x, vi = v.y;
 #pragma unroll
     for (int o = 4; o < 32; o <<= 1) {
         vr += __shfl_xor_sync(0xffffffffu, vr, o);

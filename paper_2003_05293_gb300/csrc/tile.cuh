@@ -62,21 +62,57 @@ __device__ __forceinline__ double block_min_f64(double v, double *s_red)
 // Weighted update (Eqs. 4-6) from the per-tile partial fields of one pass:
 // V_n = (1/count) sum_tiles part; w_n <- w_n <|V|> / |V_n|; theta_n <- arg V_n.
 // The tile partials are summed with Kahan compensation.
-// Compensated sum of spot n's tile partials t = t0, t0 + dt, ... (8 loads in flight).
+// Compensated sum of spot n's tile partials t = t0, t0 + dt, ..., 8 loads in
+// flight at a time: the last ones too, with zeros past the end (a remainder
+// loop would wait for each of up to 7 loads on its own, ~0.4 us apiece; of a
+// mixed batch's 27 us of tails per launch that was most).
 __device__ __forceinline__ float4 tile_sum(const HoloDev &H, int n, int t0, int dt, int tiles)
 {
+    constexpr int B = 8;
+    const float2 *part = H.part + n;
+    const int N = H.N;
     float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;
-#pragma unroll 8   // loads issued ahead of the compensated sum's chain
-    for (int t = t0; t < tiles; t += dt) {
-        float2 p = __ldcg(&H.part[(size_t)t * H.N + n]);
-        float yr = p.x - cr, tr = sr + yr;
-        cr = (tr - sr) - yr;
-        sr = tr;
-        float yi = p.y - ci, ti = si + yi;
-        ci = (ti - si) - yi;
-        si = ti;
+    for (int t = t0; t < tiles; t += B * dt) {
+        float2 p[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            const int tk = t + k * dt;
+            p[k] = tk < tiles ? __ldcg(part + (size_t)tk * N) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            float yr = p[k].x - cr, tr = sr + yr;
+            cr = (tr - sr) - yr;
+            sr = tr;
+            float yi = p[k].y - ci, ti = si + yi;
+            ci = (ti - si) - yi;
+            si = ti;
+        }
     }
     return make_float4(sr, cr, si, ci);
+}
+
+// Sum of FP64 partials part[t N], t = t0, t0 + dt, ... < tiles, the same way.
+__device__ __forceinline__ double2 tile_sum64(const double2 *part, int N, int t0, int dt, int tiles)
+{
+    constexpr int B = 8;
+    double vr = 0.0, vi = 0.0;
+    for (int t = t0; t < tiles; t += B * dt) {
+        double2 p[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            const int tk = t + k * dt;
+            p[k] = tk < tiles ? __ldcg(part + (size_t)tk * N) : make_double2(0.0, 0.0);
+        }
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            if (t + k * dt < tiles) {   // FP64 additions are dear: none of the zeros
+                vr += p[k].x;
+                vi += p[k].y;
+            }
+        }
+    }
+    return make_double2(vr, vi);
 }
 
 // (s, c) += (t, d), two compensated sums (each stands for s - c): the rounding
@@ -99,15 +135,37 @@ __device__ __forceinline__ void update_spot(const HoloDev &H, int n, float2 v, d
     H.state[n] = st;
 }
 
+//
+// The last block of a hologram runs this alone, bound by the latency of its
+// loads: where it has threads to spare, G of them share a spot's tiles (t = g,
+// g + G, ...), their sums meeting in `scratch` (16 bytes per thread).  With one
+// thread per spot, 81 tiles of 10 spots took a third of a 14.6 us iteration.
 template <int THREADS>
-__device__ void tail_update(const HoloDev &H, const LaunchSlot &sl, float2 *s_v, double *s_red)
+__device__ void tail_update(const HoloDev &H, const LaunchSlot &sl, float2 *s_v, void *scratch, double *s_red)
 {
     const int N = H.N;
     const float inv = 1.0f / (float)sl.count;
+    const int G = max(1, min(min(THREADS / N, 32), sl.tiles));
+    float4 *s_grp = static_cast<float4 *>(scratch);
+    if (G > 1) {
+        const int n = threadIdx.x % N, g = threadIdx.x / N;
+        if (g < G) s_grp[g * N + n] = tile_sum(H, n, g, G, sl.tiles);
+        __syncthreads();
+    }
     double local = 0.0;
     for (int n = threadIdx.x; n < N; n += THREADS) {
-        const float4 q = tile_sum(H, n, 0, 1, sl.tiles);
-        float2 v = make_float2(q.x * inv, q.z * inv);
+        float4 q;
+        if (G > 1) {
+            q = s_grp[n];
+            for (int g = 1; g < G; ++g) {
+                const float4 p = s_grp[g * N + n];
+                add_comp(q.x, q.y, p.x, p.y);
+                add_comp(q.z, q.w, p.z, p.w);
+            }
+        } else {
+            q = tile_sum(H, n, 0, 1, sl.tiles);
+        }
+        float2 v = make_float2((q.x - q.y) * inv, (q.z - q.w) * inv);
         s_v[n] = v;
         local += (double)hypotf(v.x, v.y);
     }
@@ -119,18 +177,25 @@ __device__ void tail_update(const HoloDev &H, const LaunchSlot &sl, float2 *s_v,
 // (FP64 partials) divided by the pupil's sum of A, I_n = |V_n|^2,
 // e = sum_n I_n, u by Eq. 7.
 template <int THREADS>
-__device__ void tail_metrics(const HoloDev &H, const LaunchSlot &sl, double *s_red)
+__device__ void tail_metrics(const HoloDev &H, const LaunchSlot &sl, void *scratch, double *s_red)
 {
     const int N = H.N;
     const double inv = 1.0 / H.norm;   // sum of A over the pupil (P^2 for the square uniform grid)
     double e = 0.0, imax = -1.0, imin = 1e300;
+    const int G = max(1, min(min(THREADS / N, 32), sl.tiles));   // threads per spot, as in tail_update
+    double2 *s_grp = static_cast<double2 *>(scratch);
+    auto sum = [&](int n, int g) { return tile_sum64(H.part64 + n, N, g, G, sl.tiles); };
+    if (G > 1) {
+        const int n = threadIdx.x % N, g = threadIdx.x / N;
+        if (g < G) s_grp[g * N + n] = sum(n, g);
+        __syncthreads();
+    }
     for (int n = threadIdx.x; n < N; n += THREADS) {
-        double vr = 0.0, vi = 0.0;
-#pragma unroll 8
-        for (int t = 0; t < sl.tiles; ++t) {
-            double2 p = __ldcg(&H.part64[(size_t)t * N + n]);
-            vr += p.x;
-            vi += p.y;
+        const double2 v = G > 1 ? s_grp[n] : sum(n, 0);
+        double vr = v.x, vi = v.y;
+        for (int g = 1; g < G; ++g) {
+            vr += s_grp[g * N + n].x;
+            vi += s_grp[g * N + n].y;
         }
         vr *= inv;
         vi *= inv;
@@ -260,8 +325,8 @@ __device__ __forceinline__ void store_tile_partials(const HoloDev &H, int pass, 
 // After a tile's partials are written: the last tile of this hologram's pass
 // (arrival counter) runs the update or the metrics, then resets the counter.
 template <int THREADS>
-__device__ __forceinline__ void finish_tile(const HoloDev &H, const LaunchSlot &sl, float2 *s_v, double *s_red,
-                                            int *s_last)
+__device__ __forceinline__ void finish_tile(const HoloDev &H, const LaunchSlot &sl, float2 *s_v, void *scratch,
+                                            double *s_red, int *s_last)
 {
     __threadfence();
     __syncthreads();
@@ -272,8 +337,8 @@ __device__ __forceinline__ void finish_tile(const HoloDev &H, const LaunchSlot &
     __syncthreads();
     if (*s_last) {
         __threadfence();
-        if (sl.pass == kPassFinal) tail_metrics<THREADS>(H, sl, s_red);
-        else tail_update<THREADS>(H, sl, s_v, s_red);
+        if (sl.pass == kPassFinal) tail_metrics<THREADS>(H, sl, scratch, s_red);
+        else tail_update<THREADS>(H, sl, s_v, scratch, s_red);
         __syncthreads();
         if (threadIdx.x == 0) *H.counter = 0u;
     }
@@ -434,7 +499,7 @@ __device__ void process_tile(const HoloDev &H, const LaunchSlot &sl, int t, int 
         store_tile_partials<THREADS>(H, pass, t, n0, nc, m.part);
         __syncthreads();
     }
-    finish_tile<THREADS>(H, sl, m.v, s_red, s_last);
+    finish_tile<THREADS>(H, sl, m.v, m.part, s_red, s_last);
 }
 
 // A tile of a compressed iteration with the half-precision sincos option
@@ -549,7 +614,7 @@ __device__ void process_tile_h2(const HoloDev &H, const LaunchSlot &sl, int t, i
         store_tile_partials<THREADS>(H, sl.pass, t, n0, nc, m.part);
         __syncthreads();
     }
-    finish_tile<THREADS>(H, sl, m.v, s_red, s_last);
+    finish_tile<THREADS>(H, sl, m.v, m.part, s_red, s_last);
 }
 
 // One spot factor of a separable tile: e^{i 2 pi (c u + G u^2)} for pixel
@@ -635,7 +700,7 @@ __device__ void process_full_tile(const HoloDev &H, const LaunchSlot &sl, int t,
                     if (H.slm) H.slm[(size_t)r * H.slm_pitch + c] = g0;
                 }
             }
-            finish_tile<THREADS>(H, sl, m.v, s_red, s_last);
+            finish_tile<THREADS>(H, sl, m.v, m.part, s_red, s_last);
             return;
         }
     }
@@ -774,7 +839,7 @@ __device__ void process_full_tile(const HoloDev &H, const LaunchSlot &sl, int t,
         store_tile_partials<THREADS>(H, pass, t, w0, wc, m.part);
         __syncthreads();
     }
-    finish_tile<THREADS>(H, sl, m.v, s_red, s_last);
+    finish_tile<THREADS>(H, sl, m.v, m.part, s_red, s_last);
 }
 
 // Spot preparation (step 1 of the path) for spot n of hologram H: fixed-point
