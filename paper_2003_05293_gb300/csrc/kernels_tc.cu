@@ -708,6 +708,7 @@ __global__ void __launch_bounds__(256) rw_tables_kernel(const HoloDev *__restric
 //   cs_free           the MMAs that read it are done (its buffer is free)
 //   z_full            a Z accumulation is done: a strip, or one spot block of a tile
 //   z_empty           the V warps have read Z
+//   dot[2]            the second V warps' half of a dot is in shared memory
 //   drain             both issuing warps' last commits, before tensor memory is freed
 // Every wait is bounded; a timeout ends the loop of the side that saw it and
 // sets the status word, and the other side's waits then run out in turn.
@@ -730,7 +731,8 @@ enum Bar {
     kCsFree,                      // the MMAs that read it are done
     kZFull,                       // a Z accumulation is done
     kZEmpty,
-    kG2Info,    // the u warps have published the next tile's GEMM 2 operands
+    kDot0,      // the second V warps' half sums are in shared memory, by parity of the accumulation
+    kG2Info = kDot0 + 2,    // the u warps have published the next tile's GEMM 2 operands
     kDrain,     // both issuing warps' last commits (2 arrivals)
     kBarsWs
 };
@@ -757,12 +759,13 @@ struct Info {
 };
 
 
-// The epilogue warps: 4 u warps (epilogue 1, warps 0 .. 3) and 4 V warps
-// (epilogue 2, warps 4 .. 7), each group one warp per TMEM lane quadrant.
-// (Eight warps sharing both epilogues were measured: 5 % slower, and 12 % at
-// more than one GEMM 2 spot block, where epilogue 2 of every tile no longer
-// overlaps epilogue 1 of the next.)
-constexpr int kUWarps = 4, kVWarps = 4;
+// The epilogue warps: 4 u warps (epilogue 1, warps 0 .. 3), one per TMEM lane
+// quadrant, and 8 V warps (epilogue 2, warps 4 .. 11), two per quadrant: each
+// takes half the rows of a strip's dot and half the columns of the final
+// pass's phase map.  GEMM 2 of the next strip (N > 128: of the next spot block)
+// waits for the dot to have read Z, a latency-bound chain: with 4 V warps a
+// batch of N = 100 spent 5 % and one of N up to 300 14 % of its time on it.
+constexpr int kUWarps = 4, kVWarps = 8;
 
 template <int W>
 struct Cfg {
@@ -1181,7 +1184,7 @@ __device__ __noinline__ void control_load(const HoloDev *__restrict__ holos, con
 }
 
 // The partial V_n = sum_y conj(R_n(y)) Z(n, y) of spot n of a closed Z
-// accumulation (a strip at row block y0) over the tile's 128 rows.  R_n(y)
+// accumulation (a strip at row block y0) over the tile's rows ys0 .. ys1 - 1.  R_n(y)
 // along the rows by recurrence: its phase is quadratic in y, so R(y + 2) =
 // R(y) D(y) and D(y + 2) = D(y) E with the constant E = e^{i (2 pi 8 Gh / 2^32
 // + 8 gl)}, the even and the odd rows side by side in packed FP32 pairs; R and
@@ -1191,7 +1194,7 @@ __device__ __noinline__ void control_load(const HoloDev *__restrict__ holos, con
 // A latency-bound chain on one warp per SM quarter: for holograms of more than
 // 128 spots GEMM 2 waits for it, once per spot block.
 __device__ __forceinline__ float2 strip_dot(uint32_t z_re, uint32_t z_im, const int4 *coef, int n, int N, int y0,
-                                            int half)
+                                            int half, int ys0, int ys1)
 {
     const int4 cf = coef[min(n, N - 1)];
     const int32_t tilt = cf.y, Gh = cf.z;
@@ -1201,7 +1204,7 @@ __device__ __forceinline__ float2 strip_dot(uint32_t z_re, uint32_t z_im, const 
     const uint64_t E_c = pack2(ec, ec), E_s = pack2(es, es), nE_s = pack2(-es, -es);
     uint64_t vr = 0ull, vi = 0ull;   // even and odd rows; vi is the sum's negative imaginary part
 #pragma unroll 1
-    for (int ys = 0; ys < kRows; ys += 16) {
+    for (int ys = ys0; ys < ys1; ys += 16) {
         float zr[16], zi[16];
         ld16(z_re + ys, zr);
         ld16(z_im + ys, zi);
@@ -1299,16 +1302,17 @@ __device__ __forceinline__ float arg_turn(float y, float x)
 }
 
 // The final pass's phase map Phi = arg S (Eq. 1) and SLM gray levels of one
-// tile row (grid row gy, columns x0 .. x0 + 63), from S in tensor memory, K-step
-// by K-step: 0 outside the pupil.  Every lane of the warp runs the tensor-memory
+// tile row (grid row gy, K-steps ks0 .. ks1 - 1 of the 64 columns from x0 on), from
+// S in tensor memory, K-step by K-step: 0 outside the pupil.  Every lane of the warp runs the tensor-memory
 // loads (they are warp-collective); a row past the grid stores nothing.
-__device__ __forceinline__ void final_phases(const HoloDev &H, uint32_t s_re, uint32_t s_im, int gy, int x0)
+__device__ __forceinline__ void final_phases(const HoloDev &H, uint32_t s_re, uint32_t s_im, int gy, int x0, int ks0,
+                                             int ks1)
 {
     const int P = H.P;
     int xl, xr;
     row_span(P, H.aperture, gy, xl, xr);
 #pragma unroll 1
-    for (int ks = 0; ks < kKSteps; ++ks) {
+    for (int ks = ks0; ks < ks1; ++ks) {
         const int gx0 = x0 + 16 * ks;
         float sr[16], si[16], o[16];
         __syncwarp();   // converged for the warp-collective loads
@@ -1525,9 +1529,11 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, G2
 // Z(n, y), one spot per thread over all 128 rows, while the u warps go on with
 // the next tiles.  In the final pass they also write each tile's phase map
 // (and gray levels) from S, beside the u warps' work on u.
-__device__ __forceinline__ void epilogue_v(const Info *info, uint32_t mb, uint32_t tmem, unsigned *status)
+__device__ __forceinline__ void epilogue_v(const Info *info, float2 (*s_half)[kSpotBlock], uint32_t mb, uint32_t tmem,
+                                           unsigned *status)
 {
-    const int tid = threadIdx.x - 32 * kUWarps, lane = tid & 31, q = tid >> 5;   // TMEM lane quadrant q
+    const int tid = threadIdx.x - 32 * kUWarps, lane = tid & 31, q = (tid >> 5) & 3;   // TMEM lane quadrant q
+    const int hv = tid >> 7;                                                           // half of the rows
     const uint32_t lanes = (uint32_t)(32 * q) << 16;
     uint32_t n_z = 0u;   // Z accumulations reduced
     uint32_t n_s = 0u;   // tiles with products seen, per S buffer (low half: j = 0, high half: j = 1)
@@ -1553,7 +1559,8 @@ __device__ __forceinline__ void epilogue_v(const Info *info, uint32_t mb, uint32
             if (!ok) break;
             fence_after();
             const uint32_t s_re = tmem + kS0 + 2 * kCols * j + lanes;
-            final_phases(H, s_re, s_re + kCols, y0 + 32 * q + lane, (t % ((P + kCols - 1) / kCols)) * kCols);
+            final_phases(H, s_re, s_re + kCols, y0 + 32 * q + lane, (t % ((P + kCols - 1) / kCols)) * kCols,
+                         hv * (kKSteps / 2), (hv + 1) * (kKSteps / 2));
             fence_before();
         }
         // the info slot (and S buffer) is read: it goes back with this group's arrival
@@ -1567,10 +1574,24 @@ __device__ __forceinline__ void epilogue_v(const Info *info, uint32_t mb, uint32
             if (!ok) break;
             fence_after();
             const int n = sb * kSpotBlock + 32 * q + lane;
-            const float2 v = strip_dot(tmem + lanes, tmem + kRows + lanes, coef, n, N, y0, half);
+            float2 v = strip_dot(tmem + lanes, tmem + kRows + lanes, coef, n, N, y0, half, hv * (kRows / 2),
+                                       (hv + 1) * (kRows / 2));
             fence_before();
+            const uint32_t buf = n_z & 1u;
+            if (hv) s_half[buf][32 * q + lane] = v;
             __syncwarp();
-            if (lane == 0) arrive(mbar_at(mb, kZEmpty));
+            if (lane == 0) {
+                arrive(mbar_at(mb, kZEmpty));
+                if (hv) arrive(mbar_at(mb, kDot0 + buf));
+            }
+            if (hv) continue;
+            // the first V warps add the second ones' halves (the second ones write
+            // a buffer again only after Z has been released twice more)
+            ok = warp_and(wait_newest(mbar_at(mb, kDot0 + buf), (n_z + 1u) >> 1));
+            if (!ok) break;
+            const float2 w = s_half[buf][32 * q + lane];
+            v.x += w.x;
+            v.y += w.y;
             if (n < N) {
                 const size_t off = (size_t)s_loc * N + n;
                 if (pass == kPassFinal) part64[off] = make_double2((double)v.x, (double)v.y);
@@ -1596,6 +1617,7 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
     __shared__ __align__(8) uint64_t s_mbar[kBarsWs];
     __shared__ Info s_info[2];
     __shared__ G2Info s_g2;
+    __shared__ float2 s_half[2][tc::kSpotBlock];
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, warp = tid >> 5;
     // queue[3] != 0 (a test of the bounded waits): the producer publishes no
@@ -1609,6 +1631,7 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
             // S buffers and info slots go back from the epilogue and the GEMM 1 warp
             const uint32_t cnt = (b == kSEmpty0 || b == kSEmpty0 + 1) ? W + 1
                                  : b == kZEmpty                               ? kVWarps
+                                 : (b == kDot0 || b == kDot0 + 1)             ? kVWarps / 2
                                  : (b >= kUStep0 && b < kUStep0 + kKSteps)    ? kUWarps
                                  : b == kDrain                                ? 2
                                                                               : 1;
@@ -1646,7 +1669,7 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
     } else if (warp < kUWarps) {
         epilogue_u<F16, US>(m, s_info, &s_g2, mb, s_tmem, status);
     } else {
-        epilogue_v(s_info, mb, s_tmem, status);
+        epilogue_v(s_info, s_half, mb, s_tmem, status);
     }
     tc::fence_before();
     __syncthreads();
@@ -1896,7 +1919,7 @@ static cudaError_t tcws_launch(const HoloDev *holos, const LaunchSlot *slots, in
 }
 
 // epilogue warps of the warp-specialised kernel
-constexpr int kWsWarps = 8;
+constexpr int kWsWarps = 12;
 
 int full_tc_tiles(int P) { return tc::tiles(P); }
 
