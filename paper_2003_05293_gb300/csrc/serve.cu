@@ -153,21 +153,21 @@ bool Server::tc_subset(const HoloSpec &s) const
     return c * s.N > 4.0 * full_tc_spot_blocks(s.N);
 }
 
-size_t Server::footprint(const HoloSpec &s, bool masks) const
+size_t Server::footprint(const HoloSpec &s, TileShape shape, bool masks) const
 {
     const size_t M = (size_t)s.P * s.P;
-    const size_t tiles = (size_t)max_pass_tiles(s, shape_);
+    const size_t tiles = (size_t)max_pass_tiles(s, shape);
     size_t b = 0;
     b += al256(sizeof(double) * 3 * s.N) + (s.has_amp ? al256(sizeof(double) * s.N) : 0);
     b += al256(sizeof(int4) * s.N) + al256(sizeof(SpotState) * s.N);
     b += al256(sizeof(float2) * tiles * s.N) + al256(sizeof(double2) * tiles * s.N);
     b += 256 + al256(sizeof(double) * (2 + s.N));
     b += al256(sizeof(float) * M);   // phase map (the caller's device buffer is used when given)
-    if (uses_tc(shape_)) {
+    if (uses_tc(shape)) {
         size_t rw, c, cs;
         full_tc_table_bytes(s.P, s.N, &rw, &c, &cs);
         b += al256(rw) + al256(c) + al256(cs);
-        if (shape_.fp16 && shape_.threads == kSubsetTc) b += al256(cs / 2);
+        if (shape.fp16 && shape.threads == kSubsetTc) b += al256(cs / 2);
     }
     if (masks) b += al256(sizeof(uint32_t) * (size_t)s.P * mask_words_of(s.P));
     return b;
@@ -177,7 +177,8 @@ size_t Server::footprint(const HoloSpec &s, bool masks) const
 void Server::place(Req &r)
 {
     const HoloSpec &s = r.spec;
-    const size_t tiles = (size_t)max_pass_tiles(s, shape_);
+    const TileShape shape = r.lean ? lean_shape() : shape_;
+    const size_t tiles = (size_t)max_pass_tiles(s, shape);
     char *b = arena_.base() + r.off;
     size_t o = 0;
     HoloDev &H = r.dev;
@@ -217,7 +218,7 @@ void Server::place(Req &r)
     float *own = reinterpret_cast<float *>(b + o);
     o += al256(sizeof(float) * (size_t)s.P * s.P);
     H.phase_out = r.phase_dev ? r.phase_dev : own;
-    if (uses_tc(shape_)) {
+    if (uses_tc(shape)) {
         size_t rw, c, cs;
         full_tc_table_bytes(s.P, s.N, &rw, &c, &cs);
         H.rwtab = reinterpret_cast<unsigned char *>(b + o);
@@ -226,12 +227,12 @@ void Server::place(Req &r)
         o += al256(c);
         H.cstab = reinterpret_cast<unsigned char *>(b + o);
         o += al256(cs);
-        if (shape_.fp16 && shape_.threads == kSubsetTc) {
+        if (shape.fp16 && shape.threads == kSubsetTc) {
             H.cstab16 = reinterpret_cast<unsigned char *>(b + o);
             o += al256(cs / 2);
         }
     }
-    if (uses_masks(shape_) || r.tc_subset) {
+    if (uses_masks(shape) || r.tc_subset) {
         // the subset mask starts clear (each compressed launch's tails clear it again)
         H.mask = reinterpret_cast<uint32_t *>(b + o);
         H.mask_words = mask_words_of(s.P);
@@ -269,10 +270,14 @@ cswgs_status Server::submit(const cswgs_request &q, uint64_t *ticket)
         CSWGS_TRY(start());
     }
     r->tc_subset = tc_subset(r->spec);
-    size_t need = footprint(r->spec, uses_masks(shape_) || r->tc_subset);
+    size_t need = footprint(r->spec, shape_, uses_masks(shape_) || r->tc_subset);
     if (r->tc_subset && need > arena_.capacity()) {   // no room for the mask: the shape's own kernel needs none
         r->tc_subset = false;
-        need = footprint(r->spec, false);
+        need = footprint(r->spec, shape_, uses_masks(shape_));
+    }
+    if (need > arena_.capacity()) {   // no room for the shape's tables: the CUDA-core kernels need none
+        r->lean = true;
+        need = footprint(r->spec, lean_shape(), false);
     }
     if (need > arena_.capacity()) {
         st_.rejected++;
@@ -425,20 +430,21 @@ void Server::loop()
             if (a && !a->cancelled && pass_of(a->spec, a->L) >= 0) order.push_back(a.get());
         std::stable_sort(order.begin(), order.end(), [](Req *a, Req *b) { return a->spec.N > b->spec.N; });
         // groups: compressed iterations on the shape's kernel, the same on the
-        // tensor cores, full passes
-        constexpr int kGroups = 3;
-        const int kind_of[kGroups] = {kLaunchSubset, kLaunchSubset, kLaunchFull};
+        // tensor cores, full passes; both kinds of the lean requests
+        constexpr int kGroups = 5;
+        const int kind_of[kGroups] = {kLaunchSubset, kLaunchSubset, kLaunchFull, kLaunchSubset, kLaunchFull};
         TileShape tc_shape = shape_;
         tc_shape.threads = kSubsetTc;
         tc_shape.ppt = 1;
-        const TileShape group_shape[kGroups] = {shape_, tc_shape, shape_};
+        const TileShape group_shape[kGroups] = {shape_, tc_shape, shape_, lean_shape(), lean_shape()};
         int nslots = 0, group_slots[kGroups] = {}, group_tiles[kGroups] = {}, group_maxN[kGroups] = {},
             group_maxP[kGroups] = {};
         std::vector<Req *> finishing;
         for (int g = 0; g < kGroups; ++g) {
             for (Req *r : order) {
                 const int pass = pass_of(r->spec, r->L);
-                if ((pass == kPassSubset ? (r->tc_subset ? 1 : 0) : 2) != g) continue;
+                const int sub = r->tc_subset ? 1 : 0;
+                if ((pass == kPassSubset ? (r->lean ? 3 : sub) : (r->lean ? 4 : 2)) != g) continue;
                 LaunchSlot &sl = sbuf[nslots++];
                 sl.holo = r->slot;
                 sl.pass = pass;

@@ -44,6 +44,7 @@ private:
         size_t off = 0, bytes = 0;
         HoloDev dev{};
         int slot = -1;
+        bool lean = false;               // on the CUDA-core kernels: no room for the shape's tables and masks
         bool tc_subset = false;          // compressed iterations on the tensor cores, whatever the shape's kernel
         int L = 0;                       // next launch index of this request's schedule
         int64_t last_launch = -1;        // serial of the last launch that used it
@@ -53,7 +54,8 @@ private:
     };
     void loop();
     bool tc_subset(const HoloSpec &s) const;
-    size_t footprint(const HoloSpec &s, bool masks) const;
+    size_t footprint(const HoloSpec &s, TileShape shape, bool masks) const;
+    TileShape lean_shape() const { return TileShape{256, 4, 256, shape_.fp16}; }
     void place(Req &r);
     void finish(Req &r, cswgs_status st);
 
@@ -66,7 +68,7 @@ private:
         std::vector<int> P, N;
         int strip = 0;
     };
-    StripChoice strips_[3];
+    StripChoice strips_[5];
     bool shape_set_ = false;
     std::thread th_;
     std::mutex mu_;
