@@ -64,3 +64,21 @@ def test_no_room_for_the_mask(tmp_path):
             lo = mid
     r = taken(hi)
     assert abs(r["e"] - ref["e"]) < TOL_EU and abs(r["u"] - ref["u"]) < TOL_EU
+
+
+def test_no_room_for_the_tables(tmp_path):
+    """A loop whose shape runs everything on the tensor cores takes a request
+    whose factor tables do not fit its memory on the CUDA-core kernels, beside
+    one that fits, and refuses one that fits neither way."""
+    from paper_2003_05293_gb300 import CswgsError, Plan
+    cache = write_pinned_tune_cache(tmp_path / "t.json", 1, 1, FULL_WS)
+    fits = workloads.problem(64, 8, 2.0, 0.25, 4, seed=5)
+    lean = workloads.problem(256, 8, 2.0, 0.25, 4, seed=6)     # 384 KiB without tables, 600 KiB with them
+    never = workloads.problem(1024, 8, 2.0, 0.25, 4, seed=7)   # its phase map alone is 4 MiB
+    with Plan(precision="fp32", max_batch=8, mem_cap_bytes=500 << 10, tune_cache=cache) as p:
+        for pb in (fits, lean, fits):
+            g = p.wait(p.submit(pb, None), 60.0)
+            r = p.solve(pb.xyz, pb.P, pb.c, pb.iterations, pb.seed)
+            assert abs(g["e"] - r["e"]) < TOL_EU and abs(g["u"] - r["u"]) < TOL_EU
+        with pytest.raises(CswgsError):
+            p.submit(never, None)
