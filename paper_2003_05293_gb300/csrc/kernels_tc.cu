@@ -694,16 +694,13 @@ __global__ void __launch_bounds__(256) rw_tables_kernel(const HoloDev *__restric
 // metrics) run in a small kernel right after the launch, so tiles neither
 // fence nor count arrivals.
 // Hand-overs, all mbarriers:
-//   ready[2]          producer -> GEMM 1, u and V warps: tile k in info slot k & 1
+//   ready[2]          producer -> GEMM 1, GEMM 2, u and V warps: tile k in info slot k & 1
 //   full[r], empty[r] GEMM 1 operand ring: copies landed / MMAs done
 //   s_full[2]         GEMM 1 of the tile in that S buffer is done
-//   s_empty[2]        the u warps have read that S buffer and info slot, the V and
-//                     GEMM 1 warps that info slot
-//   g2_info           u warps -> GEMM 2 warp: the tile's C blocks and its place in
-//                     its strip (or done)
+//   s_empty[2]        the tile's u warps have read that S buffer and info slot, the
+//                     V and GEMM warps that info slot
 //   u_step[4]         the u warps have written u's columns of one K-step of GEMM 2
-//   u_free[4]         GEMM 2 has read them (one phase per tile with products, so
-//                     that no wait is two phases short)
+//   u_free[2][4]      GEMM 2 has read them, per S buffer
 //   cs_full           GEMM 2's C block has landed
 //   cs_free           the MMAs that read it are done (its buffer is free)
 //   z_full            a Z accumulation is done: a strip, or one spot block of a tile
@@ -726,23 +723,20 @@ enum Bar {
     kSFull0 = kEmpty0 + kRingMax,
     kSEmpty0 = kSFull0 + 2,
     kUStep0 = kSEmpty0 + 2,       // u's columns of GEMM 2's K-step 0 .. 3 are written
-    kUFree0 = kUStep0 + kKSteps,  // ... and GEMM 2 has read them
-    kCsFull = kUFree0 + kKSteps,  // GEMM 2's C block has landed
+    kUFree0 = kUStep0 + kKSteps,  // ... and GEMM 2 has read them, per S buffer
+    kCsFull = kUFree0 + 2 * kKSteps,  // GEMM 2's C block has landed
     kCsFree,                      // the MMAs that read it are done
     kZFull,                       // a Z accumulation is done
     kZEmpty,
     kDot0,      // the second V warps' half sums are in shared memory, by parity of the accumulation
-    kG2Info = kDot0 + 2,    // the u warps have published the next tile's GEMM 2 operands
-    kDrain,     // both issuing warps' last commits (2 arrivals)
+    kDrain = kDot0 + 2,     // both issuing warps' last commits (2 arrivals)
     kBarsWs
 };
 
-// The GEMM 2 warp's work item, published by the u warps when they take up a
-// tile with products (a single slot: the next one is written only after the
-// GEMM 2 warp has issued that tile's first K-step, so it has read it).
+// The GEMM 2 warp's work item: a published tile with products.
 struct G2Info {
     const unsigned char *cstab;   // GEMM 2's C blocks in the launch's format
-    int nsb, cb, done, f16;
+    int nsb, cb, j;               // j: the tile's S buffer
     int first, last;              // the tile opens / closes its strip's Z accumulation
 };
 
@@ -753,19 +747,22 @@ struct G2Info {
 struct Info {
     int item, empty, done, tile;
     int first, last;   // the first / last tile with products of the strip
-    int zero, pad;     // zero: the strip's last tile, and the strip has no products
+    int zero;          // the strip's last tile, and the strip has no products
+    uint32_t before;   // tiles with products published before this one
     LaunchSlot sl;
     HoloDev H;
 };
 
 
-// The epilogue warps: 4 u warps (epilogue 1, warps 0 .. 3), one per TMEM lane
-// quadrant, and 8 V warps (epilogue 2, warps 4 .. 11), two per quadrant: each
-// takes half the rows of a strip's dot and half the columns of the final
-// pass's phase map.  GEMM 2 of the next strip (N > 128: of the next spot block)
-// waits for the dot to have read Z, a latency-bound chain: with 4 V warps a
-// batch of N = 100 spent 5 % and one of N up to 300 14 % of its time on it.
-constexpr int kUWarps = 4, kVWarps = 8;
+// The epilogue warps: two groups of 4 u warps (epilogue 1), one warp per TMEM
+// lane quadrant, group g taking the tiles of S buffer g, so that one tile's mask
+// loads, tensor-memory latency and waits pass while the other group works; and
+// 8 V warps (epilogue 2), two per quadrant: each takes half the rows of a
+// strip's dot and half the columns of the final pass's phase map.  GEMM 2 of
+// the next strip (N > 128: of the next spot block) waits for the dot to have
+// read Z, a latency-bound chain: with 4 V warps a batch of N = 100 spent 5 %
+// and one of N up to 300 14 % of its time on it.
+constexpr int kUWarps = 8, kVWarps = 8;   // kUWarps: both groups
 
 template <int W>
 struct Cfg {
@@ -929,11 +926,10 @@ __device__ __forceinline__ bool gemm1(Ctl &C, int nc, int j)
 // has read the last one; the last tile of a strip (and each spot block but the
 // last) closes it.  After each K-step of the last spot block, u's columns of
 // that K-step go back to the epilogue warps.
-template <int US>
+template <bool F16, int US>
 __device__ __forceinline__ bool gemm2(Ctl &C, const G2Info &g)
 {
-    const int f16 = g.f16;
-    const uint32_t comps = f16 ? 2u : 4u, kbytes = comps * kCk;
+    const uint32_t comps = F16 ? 2u : 4u, kbytes = comps * kCk;
     const uint32_t id = idesc(kSpotBlock, kRows, 0), idn = idesc(kSpotBlock, kRows, 1);
     const uint32_t z_re = C.tmem, z_im = C.tmem + kRows;
     const uint64_t cs0 = desc(C.cs, 128, 256);                       // [128 spots][16 columns] per component
@@ -961,7 +957,7 @@ __device__ __forceinline__ bool gemm2(Ctl &C, const G2Info &g)
             const uint32_t acc = (opens && ks == 0) ? 0u : 1u;
             const uint64_t cs = cs0 + ((uint64_t)(ks * kbytes) >> 4);
             const uint64_t us = u0 + ((uint64_t)((ks % US) * kUSlot) >> 4);   // u's slot of this K-step
-            if (f16) {
+            if (F16) {
                 // conj(C) u: Z_re = C_re u_re + C_im u_im, Z_im = C_re u_im - C_im u_re
                 const uint64_t cr = cs, ci = cs + ((uint64_t)kCk >> 4);
                 const uint64_t ur = us, ui = us + ((uint64_t)kUc >> 4);
@@ -970,7 +966,7 @@ __device__ __forceinline__ bool gemm2(Ctl &C, const G2Info &g)
                     mma(z_re, ci, ui, id, 1u);
                     mma(z_im, cr, ui, id, acc);
                     mma(z_im, ci, ur, idn, 1u);
-                    if (sb == g.nsb - 1) commit(mbar_at(C.mb, kUFree0 + ks));
+                    if (sb == g.nsb - 1) commit(mbar_at(C.mb, kUFree0 + kKSteps * g.j + ks));
                 }
             } else {
                 uint64_t a[4], b[4];
@@ -980,7 +976,7 @@ __device__ __forceinline__ bool gemm2(Ctl &C, const G2Info &g)
                 }
                 if (elect_one()) {
                     complex_mma(z_re, z_im, a, b, id, idn, acc, 1);
-                    if (sb == g.nsb - 1) commit(mbar_at(C.mb, kUFree0 + ks));
+                    if (sb == g.nsb - 1) commit(mbar_at(C.mb, kUFree0 + kKSteps * g.j + ks));
                 }
             }
             __syncwarp();
@@ -1027,20 +1023,30 @@ __device__ __forceinline__ Ctl ctl_init(const SmemWs &m, uint32_t mb, uint32_t t
     return C;
 }
 
-// The GEMM 2 warp: per tile with products, its operands as the epilogue
-// publishes them, then GEMM 2 once u is ready.
-template <int US>
-__device__ __noinline__ void control_gemm2(const SmemWs &m, const G2Info *g2, uint32_t mb, uint32_t tmem,
+// The GEMM 2 warp: per published tile with products, GEMM 2 as u's K-steps
+// come in; the info slot goes back as soon as it is read.
+template <bool F16, int US>
+__device__ __noinline__ void control_gemm2(const SmemWs &m, const Info *info, uint32_t mb, uint32_t tmem,
                                            unsigned *status)
 {
     Ctl C = ctl_init(m, mb, tmem);
     bool ok = true;
-    for (uint32_t n = 0;; ++n) {
-        ok = warp_wait(mbar_at(mb, kG2Info), n);
-        if (!ok) break;
-        const G2Info g = *g2;
-        if (g.done) break;
-        ok = gemm2<US>(C, g);
+    for (uint32_t k = 0;; ++k) {
+        const int j = k & 1;
+        ok = warp_wait(mbar_at(mb, kReady0 + j), (k >> 1) & 1u);
+        if (!ok || info[j].done) break;
+        const int empty = info[j].empty, P = info[j].H.P;
+        G2Info g;
+        g.cstab = F16 ? info[j].H.cstab16 : info[j].H.cstab;
+        g.nsb = nspotblocks(info[j].H.N);
+        g.cb = info[j].tile % ((P + kCols - 1) / kCols);
+        g.j = j;
+        g.first = info[j].first;
+        g.last = info[j].last;
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) arrive(mbar_at(mb, kSEmpty0 + j));
+        if (empty) continue;
+        ok = gemm2<F16, US>(C, g);
         if (!ok) break;
     }
     const bool drained = drain<Lay<US>::kRing>(C, true);
@@ -1103,7 +1109,8 @@ __device__ __noinline__ void control_load(const HoloDev *__restrict__ holos, con
     bool ok = true;
     int slot = 0;   // a block's items only rise, so their slots are found by scanning forward
     int item = blockIdx.x;   // the first items go to the blocks in order, the rest through the queue
-    uint32_t k = 0;   // tiles published
+    uint32_t k = 0;        // tiles published
+    uint32_t before = 0;   // those with products
     for (bool stop = false; !stop;) {
         const bool fin = item >= total_tiles || !ok;
         // the next item's pop is in flight while this one is published and multiplied
@@ -1155,6 +1162,7 @@ __device__ __noinline__ void control_load(const HoloDev *__restrict__ holos, con
                     info[j].first = c == cf ? 1 : 0;
                     info[j].last = c == cl ? 1 : 0;
                     info[j].zero = (cf < 0 && c == c1 - 1) ? 1 : 0;
+                    info[j].before = before;
                     info[j].sl = sl;
                 }
                 uint32_t *dst = reinterpret_cast<uint32_t *>(&info[j].H);
@@ -1167,7 +1175,16 @@ __device__ __noinline__ void control_load(const HoloDev *__restrict__ holos, con
             __syncwarp();
             if (lane0) arrive(mbar_at(mb, kReady0 + j));
             ++k;
-            if (stop) break;
+            if (stop) {
+                // the end goes to both u groups: into the other slot too
+                if (k >= 2 && ok) ok = warp_wait(mbar_at(mb, kSEmpty0 + (j ^ 1)), (k >> 1) - 1u);
+                if (lane0) {
+                    info[j ^ 1].done = 1;
+                    arrive(mbar_at(mb, kReady0 + (j ^ 1)));
+                }
+                break;
+            }
+            if (!empty) before++;
             if (!empty) ok = load_gemm1<R>(C, *Hp, rb, c);
         }
         item = __shfl_sync(0xffffffffu, next, 0);
@@ -1346,39 +1363,28 @@ __device__ __forceinline__ void final_phases(const HoloDev &H, uint32_t s_re, ui
     }
 }
 
-// The u warps (epilogue 1): per tile, u = A S / |S| into GEMM 2's B operand,
-// K-step by K-step: K-step ks goes to u's slot ks % US once GEMM 2 has read
-// that slot's last K-step (computed first, stored after the wait).  A tile outside the pupil gets, in
-// the final pass, phase 0 and gray lut[0] here, and a strip with no tile
-// inside the pupil its zero partials.
+// A group of u warps (epilogue 1): per tile of its S buffer, u = A S / |S| into
+// GEMM 2's B operand, K-step by K-step: K-step ks goes to u's slot ks once
+// GEMM 2 has read the slot's last K-step, the previous tile's (computed first,
+// stored after the wait).  A tile outside the pupil gets, in the final pass,
+// phase 0 and gray lut[0] here, and a strip with no tile inside the pupil its
+// zero partials.
 template <bool F16, int US>
-__device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, G2Info *g2, uint32_t mb, uint32_t tmem,
+__device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, uint32_t mb, uint32_t tmem,
                                            unsigned *status)
 {
-    constexpr int kT = 32 * kUWarps;
-    const int tid = threadIdx.x, lane = tid & 31, q = tid >> 5;   // warps 0 .. 3: TMEM lane quadrant q
+    static_assert(US == kKSteps, "a slot per K-step");
+    constexpr int kT = 32 * kUWarps / 2;
+    const int tid = threadIdx.x & (kT - 1), lane = tid & 31, q = tid >> 5;   // TMEM lane quadrant q
+    const int j = threadIdx.x / kT;                                          // group, S buffer and info slot
     const uint32_t lanes = (uint32_t)(32 * q) << 16;
-    // phases seen: s_full[j] once per tile with products (low half: j = 0,
-    // high half: j = 1); n_p: tiles with products taken up (u_free[ks]
-    // completes once per such tile)
-    uint32_t n_s = 0u, n_p = 0u;
+    uint32_t n_s = 0u;   // this group's tiles with products (s_full[j] completes once per such tile)
     bool ok = true;
-    for (uint32_t k = 0;; ++k) {
-        const int j = k & 1;
+    for (uint32_t k = j;; k += 2) {
         ok = warp_and(wait(mbar_at(mb, kReady0 + j), (k >> 1) & 1u));
-        if (!ok) break;
-        if (info[j].done) {
-            // the GEMM 2 warp has read the last published operands once it has
-            // issued that tile's first K-step
-            if (n_p > 0u) ok = warp_and(wait_newest(mbar_at(mb, kUFree0), n_p));
-            if (ok && tid == 0) {
-                g2->done = 1;
-                arrive(mbar_at(mb, kG2Info));
-            }
-            break;
-        }
-        const int item = info[j].item, empty = info[j].empty, t = info[j].tile;
-        const int first = info[j].first, last = info[j].last, zero = info[j].zero;
+        if (!ok || info[j].done) break;
+        const int item = info[j].item, empty = info[j].empty, t = info[j].tile, zero = info[j].zero;
+        const uint32_t before = info[j].before;
         const LaunchSlot sl = info[j].sl;
         const HoloDev H = info[j].H;   // by value: global stores below cannot alias it
         const int P = H.P, N = H.N, half = P >> 1, pass = sl.pass;
@@ -1406,6 +1412,11 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, G2
                     if (H.slm) H.slm[(size_t)r * H.slm_pitch + c] = g0;
                 }
             }
+            // the other group's phases are looked at here as well (see below)
+            if (before > n_s)
+                for (int ks = 0; ks < kKSteps && ok; ++ks)
+                    ok = warp_and(wait_newest(mbar_at(mb, kUFree0 + kKSteps * (j ^ 1) + ks), before - n_s));
+            if (!ok) break;
             continue;
         }
 
@@ -1422,25 +1433,9 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, G2
                 mword = 0ull;
             }
         }
-        // the single GEMM 2 operand slot is free once GEMM 2 has issued the
-        // previous tile's first K-step
-        if (n_p > 0u) {
-            ok = warp_and(wait_newest(mbar_at(mb, kUFree0), n_p));
-            if (!ok) break;
-        }
-        if (tid == 0) {
-            g2->cstab = F16 ? H.cstab16 : H.cstab;
-            g2->nsb = nspotblocks(N);
-            g2->cb = t % col_tiles;
-            g2->done = 0;
-            g2->f16 = F16 ? 1 : 0;
-            g2->first = first;
-            g2->last = last;
-            arrive(mbar_at(mb, kG2Info));
-        }
-        n_p++;
-        n_s += 1u << (16 * j);
-        ok = warp_and(wait_newest(mbar_at(mb, kSFull0 + j), (n_s >> (16 * j)) & 0xFFFFu));
+        const uint32_t other = before - n_s;   // the other group's tiles with products before this one
+        n_s++;
+        ok = warp_and(wait_newest(mbar_at(mb, kSFull0 + j), n_s));
         if (!ok) break;
         fence_after();
         {
@@ -1494,15 +1489,15 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, G2
                         }
                         pk[g] = pack8<F16>(ur, ui);
                     }
-                    // u's slot of this K-step is free once GEMM 2 has read its last
-                    // K-step (US earlier in GEMM 2's order: of this tile, or of the
-                    // previous tile with products); K-step 0's was waited for above
-                    // (the condition is the same in every lane of the warp, so
-                    // the warp's vote stays matched)
-                    const int pks = (ks + kKSteps - US) % kKSteps;
-                    const uint32_t pcount = ks >= US ? n_p : n_p - 1u;
-                    if (pcount > 0u && !(ks == 0 && US == kKSteps) &&
-                        !warp_and(wait_newest(mbar_at(mb, kUFree0 + pks), pcount)))
+                    // u's slot of this K-step is free once GEMM 2 has read the
+                    // last u in it: the other group's last tile's or this one's.
+                    // Each group has its own phases, and since a group looks at the
+                    // other's at every tile (an empty one too) no wait is more than
+                    // one phase short.  (The conditions are the same in every lane,
+                    // so the warp's votes stay matched.)
+                    if (other > 0u && !warp_and(wait_newest(mbar_at(mb, kUFree0 + kKSteps * (j ^ 1) + ks), other)))
+                        return false;
+                    if (n_s > 1u && !warp_and(wait_newest(mbar_at(mb, kUFree0 + kKSteps * j + ks), n_s - 1u)))
                         return false;
                     unsigned char *slot = m.u + (ks % US) * kUSlot;
                     store8<F16>(slot, kUc, core_off(row, 0, 16), pk[0]);
@@ -1616,7 +1611,6 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t s_mbar[kBarsWs];
     __shared__ Info s_info[2];
-    __shared__ G2Info s_g2;
     __shared__ float2 s_half[2][tc::kSpotBlock];
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -1628,11 +1622,11 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
         tc::s_wait_polls = queue[4] != 0u ? queue[4] : tc::kWaitPolls;
         for (int b = 0; b < kBarsWs; ++b) {
             // the epilogue's releases arrive once per warp
-            // S buffers and info slots go back from the epilogue and the GEMM 1 warp
-            const uint32_t cnt = (b == kSEmpty0 || b == kSEmpty0 + 1) ? W + 1
+            // S buffers and info slots go back from a u group, the V warps and both GEMM warps
+            const uint32_t cnt = (b == kSEmpty0 || b == kSEmpty0 + 1) ? kUWarps / 2 + kVWarps + 2
                                  : b == kZEmpty                               ? kVWarps
                                  : (b == kDot0 || b == kDot0 + 1)             ? kVWarps / 2
-                                 : (b >= kUStep0 && b < kUStep0 + kKSteps)    ? kUWarps
+                                 : (b >= kUStep0 && b < kUStep0 + kKSteps)    ? kUWarps / 2
                                  : b == kDrain                                ? 2
                                                                               : 1;
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(tc::saddr(&s_mbar[b])), "r"(cnt));
@@ -1665,9 +1659,9 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
     } else if (warp == W + 1) {
         control_gemm1<R>(m, s_info, mb, s_tmem, status);
     } else if (warp == W + 2) {
-        control_gemm2<US>(m, &s_g2, mb, s_tmem, status);
+        control_gemm2<F16, US>(m, s_info, mb, s_tmem, status);
     } else if (warp < kUWarps) {
-        epilogue_u<F16, US>(m, s_info, &s_g2, mb, s_tmem, status);
+        epilogue_u<F16, US>(m, s_info, mb, s_tmem, status);
     } else {
         epilogue_v(s_info, s_half, mb, s_tmem, status);
     }
@@ -1919,7 +1913,7 @@ static cudaError_t tcws_launch(const HoloDev *holos, const LaunchSlot *slots, in
 }
 
 // epilogue warps of the warp-specialised kernel
-constexpr int kWsWarps = 12;
+constexpr int kWsWarps = 16;
 
 int full_tc_tiles(int P) { return tc::tiles(P); }
 
