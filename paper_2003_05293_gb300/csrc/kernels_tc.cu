@@ -23,10 +23,10 @@
 // with the two B operands as two 128-row windows of one 192-row tile
 // [-C_im | C_re | C_im]: 6 instructions per spot chunk.
 // GEMM 2 (the forward projection) is M = 128 spots x N = 128 rows x K = 16
-// columns per instruction, real and imaginary parts apart, with split FP16
-// operands too (12 instructions per K-step).  The half-precision option
-// (compressed launches only) takes the operands' FP16 roundings alone (|u|,
-// |C| <= 1; 4 instructions per K-step): the sums run over many pixels whose
+// columns per instruction (N = 256 where real and imaginary parts share an A
+// operand), with split FP16 operands too (9 instructions per K-step).  The
+// half-precision option (compressed launches only) takes the operands' FP16
+// roundings alone (|u|, |C| <= 1; 3 instructions per K-step): the sums run over many pixels whose
 // rounding errors (2^-12 relative) do not add up coherently.
 //
 // The operands are factor tables in global memory, laid out block by block
@@ -216,29 +216,6 @@ __device__ __forceinline__ void put8(unsigned char *base, uint32_t stride, uint3
         *reinterpret_cast<uint4 *>(base + c * stride + off) = make_uint4(w[c][0], w[c][1], w[c][2], w[c][3]);
 }
 
-// Issues the 12 MMAs of a complex product with split operands:
-//   D_re += Ar Br - Ai Bi,  D_im += Ar Bi + Ai Br   (conj_a = 0)
-//   D_re += Ar Br + Ai Bi,  D_im += Ar Bi - Ai Br   (conj_a = 1)
-// a[c], b[c]: descriptors of the components re hi, re lo, im hi, im lo.
-__device__ __forceinline__ void complex_mma(uint32_t d_re, uint32_t d_im, const uint64_t a[4], const uint64_t b[4],
-                                            uint32_t id, uint32_t id_neg, uint32_t acc, int conj_a)
-{
-    const uint32_t id_ii = conj_a ? id : id_neg;     // the Ai Bi term of D_re
-    const uint32_t id_ir = conj_a ? id_neg : id;     // the Ai Br term of D_im
-    mma(d_re, a[0], b[0], id, acc);
-    mma(d_re, a[0], b[1], id, 1u);
-    mma(d_re, a[1], b[0], id, 1u);
-    mma(d_re, a[2], b[2], id_ii, 1u);
-    mma(d_re, a[2], b[3], id_ii, 1u);
-    mma(d_re, a[3], b[2], id_ii, 1u);
-    mma(d_im, a[0], b[2], id, acc);
-    mma(d_im, a[0], b[3], id, 1u);
-    mma(d_im, a[1], b[2], id, 1u);
-    mma(d_im, a[2], b[0], id_ir, 1u);
-    mma(d_im, a[2], b[1], id_ir, 1u);
-    mma(d_im, a[3], b[0], id_ir, 1u);
-}
-
 // Eight complex values -> FP16 rows of the re and im component tiles
 // (`stride` bytes apart), one 16-byte store each (round to nearest).
 __device__ __forceinline__ void put8h(unsigned char *base, uint32_t stride, uint32_t off, const float2 *v)
@@ -372,20 +349,16 @@ __device__ __forceinline__ Packed8 pack8(const uint64_t *ur, const uint64_t *ui)
 }
 
 // The rows of a Packed8 at byte offset `off` of the component tiles `stride`
-// bytes apart: re hi, re lo, im hi, im lo; or re hi, im hi alone.
+// bytes apart: re hi, im hi, re lo, im lo; or re hi, im hi alone.
 template <bool F16>
 __device__ __forceinline__ void store8(unsigned char *base, uint32_t stride, uint32_t off, const Packed8 &p)
 {
-    if (F16) {
-        *reinterpret_cast<uint4 *>(base + off) = make_uint4(p.w[0][0], p.w[0][1], p.w[0][2], p.w[0][3]);
-        *reinterpret_cast<uint4 *>(base + stride + off) = make_uint4(p.w[1][0], p.w[1][1], p.w[1][2], p.w[1][3]);
-    } else {
+    constexpr int at[4] = {0, F16 ? 1 : 2, 1, 3};   // tile of p.w[c]
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-            *reinterpret_cast<uint4 *>(base + c * stride + off) = make_uint4(p.w[c][0], p.w[c][1], p.w[c][2], p.w[c][3]);
-    }
+    for (int c = 0; c < (F16 ? 2 : 4); ++c)
+        *reinterpret_cast<uint4 *>(base + at[c] * stride + off) =
+            make_uint4(p.w[c][0], p.w[c][1], p.w[c][2], p.w[c][3]);
 }
-
 
 // ------------------------------------------------------------- factor tables --
 // Items of eight phasors; consecutive threads take consecutive rows of one
@@ -930,7 +903,8 @@ template <bool F16, int US>
 __device__ __forceinline__ bool gemm2(Ctl &C, const G2Info &g)
 {
     const uint32_t comps = F16 ? 2u : 4u, kbytes = comps * kCk;
-    const uint32_t id = idesc(kSpotBlock, kRows, 0), idn = idesc(kSpotBlock, kRows, 1);
+    const uint32_t id2 = idesc(kSpotBlock, 2 * kRows, 0), id = idesc(kSpotBlock, kRows, 0),
+                   idn = idesc(kSpotBlock, kRows, 1);
     const uint32_t z_re = C.tmem, z_im = C.tmem + kRows;
     const uint64_t cs0 = desc(C.cs, 128, 256);                       // [128 spots][16 columns] per component
     const uint64_t u0 = desc(C.u, 128, 256);                         // [128 rows][16 columns] per component
@@ -957,27 +931,26 @@ __device__ __forceinline__ bool gemm2(Ctl &C, const G2Info &g)
             const uint32_t acc = (opens && ks == 0) ? 0u : 1u;
             const uint64_t cs = cs0 + ((uint64_t)(ks * kbytes) >> 4);
             const uint64_t us = u0 + ((uint64_t)((ks % US) * kUSlot) >> 4);   // u's slot of this K-step
-            if (F16) {
-                // conj(C) u: Z_re = C_re u_re + C_im u_im, Z_im = C_re u_im - C_im u_re
-                const uint64_t cr = cs, ci = cs + ((uint64_t)kCk >> 4);
-                const uint64_t ur = us, ui = us + ((uint64_t)kUc >> 4);
-                if (elect_one()) {
-                    mma(z_re, cr, ur, id, acc);
-                    mma(z_re, ci, ui, id, 1u);
-                    mma(z_im, cr, ui, id, acc);
-                    mma(z_im, ci, ur, idn, 1u);
-                    if (sb == g.nsb - 1) commit(mbar_at(C.mb, kUFree0 + kKSteps * g.j + ks));
+            // conj(C) u: [Z_re | Z_im] += C_re [u_re | u_im], both halves of u as one
+            // operand of N = 256 (12 KB of shared memory read for its 128 cycles;
+            // two of N = 128 read 16 KB); Z_re += C_im u_im, Z_im -= C_im u_re
+            const uint64_t crh = cs, cih = cs + ((uint64_t)((F16 ? 1 : 2) * kCk) >> 4);
+            const uint64_t crl = cs + ((uint64_t)kCk >> 4), cil = cs + ((uint64_t)(3 * kCk) >> 4);
+            const uint64_t urh = us, uih = us + ((uint64_t)kUc >> 4);
+            const uint64_t url = us + ((uint64_t)(2 * kUc) >> 4), uil = us + ((uint64_t)(3 * kUc) >> 4);
+            if (elect_one()) {
+                mma(z_re, crh, urh, id2, acc);
+                mma(z_re, cih, uih, id, 1u);
+                mma(z_im, cih, urh, idn, 1u);
+                if (!F16) {
+                    mma(z_re, crh, url, id2, 1u);
+                    mma(z_re, crl, urh, id2, 1u);
+                    mma(z_re, cih, uil, id, 1u);
+                    mma(z_re, cil, uih, id, 1u);
+                    mma(z_im, cih, url, idn, 1u);
+                    mma(z_im, cil, urh, idn, 1u);
                 }
-            } else {
-                uint64_t a[4], b[4];
-                for (int q = 0; q < 4; ++q) {
-                    a[q] = cs + ((uint64_t)(q * kCk) >> 4);
-                    b[q] = us + ((uint64_t)(q * kUc) >> 4);
-                }
-                if (elect_one()) {
-                    complex_mma(z_re, z_im, a, b, id, idn, acc, 1);
-                    if (sb == g.nsb - 1) commit(mbar_at(C.mb, kUFree0 + kKSteps * g.j + ks));
-                }
+                if (sb == g.nsb - 1) commit(mbar_at(C.mb, kUFree0 + kKSteps * g.j + ks));
             }
             __syncwarp();
         }
