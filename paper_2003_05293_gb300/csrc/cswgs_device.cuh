@@ -9,6 +9,11 @@
 
 namespace cswgs {
 
+// A chained kernel's start (its successor may be launched) and the wait for its
+// predecessor's completion and memory (launch_chained).
+__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 constexpr float kTwoPiF = 6.28318530717958647692f;
 

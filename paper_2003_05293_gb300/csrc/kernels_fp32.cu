@@ -77,6 +77,8 @@ iter_subset_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__restri
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double s_red[THREADS / 32];
     __shared__ int s_last;
+    chain_start();
+    chain_wait();
     persistent_tiles(holos, slots, nslots, total_tiles, queue, [&](const HoloDev &H, const LaunchSlot &sl, int t) {
         process_tile<THREADS, PPT>(H, sl, t, maxN, smem, s_red, &s_last);
     });
@@ -226,7 +228,7 @@ int iter_fp32_max_grid(TileShape shape, int kind, int maxN, int sm_count)
 
 cudaError_t launch_iter_fp32(TileShape shape, int kind, const HoloDev *holos, const LaunchSlot *slots,
                              int nslots, int total_tiles, int maxN, unsigned *queue, int grid,
-                             cudaStream_t s)
+                             int sm_count, cudaStream_t s)
 {
     // the smem attribute is set by iter_fp32_max_grid, which every batch calls first
     const size_t smem = iter_fp32_smem(shape, kind, maxN);
@@ -239,8 +241,8 @@ cudaError_t launch_iter_fp32(TileShape shape, int kind, const HoloDev *holos, co
 #undef X
     } else if (kind == kLaunchSubset) {
 #define X(T, K) if (shape.threads == T && shape.ppt == K) { \
-            iter_subset_kernel<T, K><<<grid, T, smem, s>>>(holos, slots, nslots, total_tiles, maxN, queue); \
-            return cudaGetLastError(); }
+            return launch_chained(iter_subset_kernel<T, K>, dim3(grid), dim3(T), smem, chain_launch(nslots, sm_count), s, \
+                                  holos, slots, nslots, total_tiles, maxN, queue); }
         CSWGS_SUBSET_SHAPES(X)
 #undef X
     } else {

@@ -598,8 +598,10 @@ __global__ void __launch_bounds__(256) rw_tables_kernel(const HoloDev *__restric
     __shared__ int4 s_cf[kChunk];      // {B, Gh, gl, theta + rounding}
     __shared__ float s_wa[kChunk];     // w a, scaled
     __shared__ uint32_t s_max[8];
+    chain_start();
     const LaunchSlot sl = slots[blockIdx.y];
     const HoloDev H = holos[sl.holo];
+    chain_wait();
     if (!H.rwtab) return;
     const int P = H.P, N = H.N, half = P >> 1, nc = nchunks(N);
     const int blocks = ((P + kRows - 1) / kRows) * nc;   // (128 rows, 16 spots) blocks, 256 threads each
@@ -727,21 +729,25 @@ struct Info {
 };
 
 
-// The epilogue warps: two groups of 4 u warps (epilogue 1), one warp per TMEM
-// lane quadrant, group g taking the tiles of S buffer g, so that one tile's mask
-// loads, tensor-memory latency and waits pass while the other group works; and
-// 8 V warps (epilogue 2), two per quadrant: each takes half the rows of a
-// strip's dot and half the columns of the final pass's phase map.  GEMM 2 of
-// the next strip (N > 128: of the next spot block) waits for the dot to have
-// read Z, a latency-bound chain: with 4 V warps a batch of N = 100 spent 5 %
-// and one of N up to 300 14 % of its time on it.
-constexpr int kUWarps = 8, kVWarps = 8;   // kUWarps: both groups
+// The epilogue warps: UG groups of 4 u warps (epilogue 1), one warp per TMEM
+// lane quadrant, and 8 V warps (epilogue 2), two per quadrant: each takes half
+// the rows of a strip's dot and half the columns of the final pass's phase map.
+// GEMM 2 of the next strip (N > 128: of the next spot block) waits for the dot
+// to have read Z, a latency-bound chain: with 4 V warps a batch of N = 100 spent
+// 5 % and one of N up to 300 14 % of its time on it.
+// With UG = 2, group g takes the tiles of S buffer g, and one tile's mask loads,
+// tensor-memory latency and waits pass while the other group works; the kernel
+// then has 96 registers a thread instead of 127.  At more than one spot block
+// and in launches of few holograms that is worth it (64 holograms of N up to
+// 300: 12.51 -> 12.29 ms; 16 of N = 100: 4.15 -> 4.07), at N <= 128, where the
+// shared-memory pipe bounds a long launch, it is not (64 of N = 100: 10.73 ->
+// 10.88, FP16 9.14 -> 9.25).
+constexpr int kVWarps = 8;
 
-template <int W>
+template <int UG>
 struct Cfg {
-    static_assert(W == kUWarps + kVWarps, "epilogue warps: the u and the V group");
-    static constexpr int kEpi = 32 * W;               // epilogue threads
-    static constexpr int kThreads = kEpi + 96;        // and the producer, GEMM 1 and GEMM 2 warps
+    static constexpr int kU = 4 * UG, kEpi = kU + kVWarps;   // u warps, epilogue warps
+    static constexpr int kThreads = 32 * (kEpi + 3);         // and the producer, GEMM 1 and GEMM 2 warps
 };
 
 // Shared-memory layout of the kernel with US slots of u (one K-step each;
@@ -1336,24 +1342,24 @@ __device__ __forceinline__ void final_phases(const HoloDev &H, uint32_t s_re, ui
     }
 }
 
-// A group of u warps (epilogue 1): per tile of its S buffer, u = A S / |S| into
+// A group of u warps (epilogue 1): per tile (UG = 2: of its S buffer), u = A S / |S| into
 // GEMM 2's B operand, K-step by K-step: K-step ks goes to u's slot ks once
 // GEMM 2 has read the slot's last K-step, the previous tile's (computed first,
 // stored after the wait).  A tile outside the pupil gets, in the final pass,
 // phase 0 and gray lut[0] here, and a strip with no tile inside the pupil its
 // zero partials.
-template <bool F16, int US>
+template <int UG, bool F16, int US>
 __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, uint32_t mb, uint32_t tmem,
                                            unsigned *status)
 {
     static_assert(US == kKSteps, "a slot per K-step");
-    constexpr int kT = 32 * kUWarps / 2;
+    constexpr int kT = 128;
     const int tid = threadIdx.x & (kT - 1), lane = tid & 31, q = tid >> 5;   // TMEM lane quadrant q
-    const int j = threadIdx.x / kT;                                          // group, S buffer and info slot
     const uint32_t lanes = (uint32_t)(32 * q) << 16;
-    uint32_t n_s = 0u;   // this group's tiles with products (s_full[j] completes once per such tile)
+    uint32_t n_seen = 0u;   // this group's tiles with products, per S buffer (low half: j = 0, high half: j = 1)
     bool ok = true;
-    for (uint32_t k = j;; k += 2) {
+    for (uint32_t k = threadIdx.x / kT;; k += UG) {
+        const int j = k & 1;   // S buffer and info slot
         ok = warp_and(wait(mbar_at(mb, kReady0 + j), (k >> 1) & 1u));
         if (!ok || info[j].done) break;
         const int item = info[j].item, empty = info[j].empty, t = info[j].tile, zero = info[j].zero;
@@ -1385,10 +1391,11 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, ui
                     if (H.slm) H.slm[(size_t)r * H.slm_pitch + c] = g0;
                 }
             }
-            // the other group's phases are looked at here as well (see below)
-            if (before > n_s)
+            // the other buffer's phases are looked at here as well (see below)
+            const uint32_t other = before - ((n_seen >> (16 * j)) & 0xFFFFu);
+            if (UG == 2 && other > 0u)
                 for (int ks = 0; ks < kKSteps && ok; ++ks)
-                    ok = warp_and(wait_newest(mbar_at(mb, kUFree0 + kKSteps * (j ^ 1) + ks), before - n_s));
+                    ok = warp_and(wait_newest(mbar_at(mb, kUFree0 + kKSteps * (j ^ 1) + ks), other));
             if (!ok) break;
             continue;
         }
@@ -1406,8 +1413,10 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, ui
                 mword = 0ull;
             }
         }
-        const uint32_t other = before - n_s;   // the other group's tiles with products before this one
-        n_s++;
+        // tiles with products on this S buffer up to this one (s_full[j] completes
+        // once per such tile), and on the other one before it
+        n_seen += 1u << (16 * j);
+        const uint32_t n_s = (n_seen >> (16 * j)) & 0xFFFFu, other = before + 1u - n_s;
         ok = warp_and(wait_newest(mbar_at(mb, kSFull0 + j), n_s));
         if (!ok) break;
         fence_after();
@@ -1463,10 +1472,10 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, ui
                         pk[g] = pack8<F16>(ur, ui);
                     }
                     // u's slot of this K-step is free once GEMM 2 has read the
-                    // last u in it: the other group's last tile's or this one's.
-                    // Each group has its own phases, and since a group looks at the
-                    // other's at every tile (an empty one too) no wait is more than
-                    // one phase short.  (The conditions are the same in every lane,
+                    // last u in it: that of the last tile on the other S buffer or on
+                    // this one.  Each buffer has its own phases, and since a group
+                    // looks at both at every tile (UG = 2: at an empty one too) no
+                    // wait is more than one phase short.  (The conditions are the same in every lane,
                     // so the warp's votes stay matched.)
                     if (other > 0u && !warp_and(wait_newest(mbar_at(mb, kUFree0 + kKSteps * (j ^ 1) + ks), other)))
                         return false;
@@ -1497,10 +1506,11 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, ui
 // Z(n, y), one spot per thread over all 128 rows, while the u warps go on with
 // the next tiles.  In the final pass they also write each tile's phase map
 // (and gray levels) from S, beside the u warps' work on u.
+template <int UG>
 __device__ __forceinline__ void epilogue_v(const Info *info, float2 (*s_half)[kSpotBlock], uint32_t mb, uint32_t tmem,
                                            unsigned *status)
 {
-    const int tid = threadIdx.x - 32 * kUWarps, lane = tid & 31, q = (tid >> 5) & 3;   // TMEM lane quadrant q
+    const int tid = threadIdx.x - 128 * UG, lane = tid & 31, q = (tid >> 5) & 3;       // TMEM lane quadrant q
     const int hv = tid >> 7;                                                           // half of the rows
     const uint32_t lanes = (uint32_t)(32 * q) << 16;
     uint32_t n_z = 0u;   // Z accumulations reduced
@@ -1575,8 +1585,8 @@ __device__ __forceinline__ void epilogue_v(const Info *info, float2 (*s_half)[kS
 
 }  // namespace tc
 
-template <int W, bool F16, int US>
-__global__ void __launch_bounds__(tc::ws::Cfg<W>::kThreads, 1)
+template <int UG, bool F16, int US>
+__global__ void __launch_bounds__(tc::ws::Cfg<UG>::kThreads, 1)
 iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__restrict__ slots, int nslots,
                       int total_tiles, unsigned *queue)
 {
@@ -1586,20 +1596,22 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
     __shared__ Info s_info[2];
     __shared__ float2 s_half[2][tc::kSpotBlock];
     __shared__ uint32_t s_tmem;
+    constexpr int W = Cfg<UG>::kEpi;   // the producer's warp
     const int tid = threadIdx.x, warp = tid >> 5;
     // queue[3] != 0 (a test of the bounded waits): the producer publishes no
     // work item, so every other role's first wait runs out, before any copy
     // or MMA is issued; queue[4] != 0: the poll limit of every wait
+    chain_start();
     const bool withhold = queue[3] != 0u;
     if (tid == 0) {
         tc::s_wait_polls = queue[4] != 0u ? queue[4] : tc::kWaitPolls;
         for (int b = 0; b < kBarsWs; ++b) {
             // the epilogue's releases arrive once per warp
             // S buffers and info slots go back from a u group, the V warps and both GEMM warps
-            const uint32_t cnt = (b == kSEmpty0 || b == kSEmpty0 + 1) ? kUWarps / 2 + kVWarps + 2
+            const uint32_t cnt = (b == kSEmpty0 || b == kSEmpty0 + 1) ? 4 + kVWarps + 2
                                  : b == kZEmpty                               ? kVWarps
                                  : (b == kDot0 || b == kDot0 + 1)             ? kVWarps / 2
-                                 : (b >= kUStep0 && b < kUStep0 + kKSteps)    ? kUWarps / 2
+                                 : (b >= kUStep0 && b < kUStep0 + kKSteps)    ? 4
                                  : b == kDrain                                ? 2
                                                                               : 1;
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(tc::saddr(&s_mbar[b])), "r"(cnt));
@@ -1620,6 +1632,7 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
                      :: "r"(tc::saddr(&s_tmem)), "r"(kTmemColsWs));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
+    chain_wait();   // the R' tables, the masks, and the last launch's queue
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -1633,10 +1646,10 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
         control_gemm1<R>(m, s_info, mb, s_tmem, status);
     } else if (warp == W + 2) {
         control_gemm2<F16, US>(m, s_info, mb, s_tmem, status);
-    } else if (warp < kUWarps) {
-        epilogue_u<F16, US>(m, s_info, mb, s_tmem, status);
+    } else if (warp < Cfg<UG>::kU) {
+        epilogue_u<UG, F16, US>(m, s_info, mb, s_tmem, status);
     } else {
-        epilogue_v(s_info, s_half, mb, s_tmem, status);
+        epilogue_v<UG>(s_info, s_half, mb, s_tmem, status);
     }
     tc::fence_before();
     __syncthreads();
@@ -1707,6 +1720,9 @@ tcws_tails_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__restric
     const LaunchSlot sl = slots[blockIdx.x / CL];
     const HoloDev &H = holos[sl.holo];
     const int rank = blockIdx.x % CL, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    chain_start();
+    if (tid < 32) asm volatile("prefetch.global.L1 [%0];" :: "l"(reinterpret_cast<const char *>(&H) + 8 * tid));
+    chain_wait();
     if (blockIdx.y > 0) {   // a whole cluster of its own
         if (sl.pass == kPassSubset && H.mask) {
             uint32_t *mask = subset_mask(H, sl.j);
@@ -1810,38 +1826,39 @@ tcws_tails_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__restric
     cluster.sync();   // s_out is read before any block of the cluster leaves
 }
 
-template <int W, bool F16, int US>
+template <int UG, bool F16, int US>
 static int tcws_max_grid_of(int maxN, int sm_count)
 {
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, iter_full_tcws_kernel<W, F16, US>) != cudaSuccess) return 0;
+    if (cudaFuncGetAttributes(&fa, iter_full_tcws_kernel<UG, F16, US>) != cudaSuccess) return 0;
     const size_t limit = 227 * 1024 - fa.sharedSizeBytes;
     const size_t smem = tc::ws::Lay<US>::kSmem;
     if (smem > limit || maxN > kTailMaxN) return 0;
-    if (cudaFuncSetAttribute(iter_full_tcws_kernel<W, F16, US>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(iter_full_tcws_kernel<UG, F16, US>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)limit) != cudaSuccess)
         return 0;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, iter_full_tcws_kernel<W, F16, US>,
-                                                      tc::ws::Cfg<W>::kThreads, smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, iter_full_tcws_kernel<UG, F16, US>,
+                                                      tc::ws::Cfg<UG>::kThreads, smem) != cudaSuccess)
         return 0;
     return std::min(per_sm, 1) * sm_count;   // a block holds all 512 tensor-memory columns
 }
 
-// Resident blocks of the kernel (both precisions; sets their shared-memory limit).
-template <int W>
+// Resident blocks of the kernel (all forms; sets their shared-memory limits).
 static int tcws_max_grid(int maxN, int sm_count)
 {
     constexpr int K4 = tc::ws::kKSteps;
-    return std::min(tcws_max_grid_of<W, false, K4>(maxN, sm_count), tcws_max_grid_of<W, true, K4>(maxN, sm_count));
+    return std::min({tcws_max_grid_of<1, false, K4>(maxN, sm_count), tcws_max_grid_of<1, true, K4>(maxN, sm_count),
+                     tcws_max_grid_of<2, false, K4>(maxN, sm_count), tcws_max_grid_of<2, true, K4>(maxN, sm_count)});
 }
 
-template <int W, bool F16, int US>
-static void tcws_launch_one(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles,
-                            unsigned *queue, int grid, cudaStream_t s)
+template <int UG, bool F16>
+static cudaError_t tcws_launch_one(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles,
+                                   unsigned *queue, int grid, bool chain, cudaStream_t s)
 {
-    iter_full_tcws_kernel<W, F16, US><<<grid, tc::ws::Cfg<W>::kThreads, tc::ws::Lay<US>::kSmem, s>>>(
-        holos, slots, nslots, total_tiles, queue);
+    constexpr int K4 = tc::ws::kKSteps;
+    return launch_chained(iter_full_tcws_kernel<UG, F16, K4>, dim3(grid), dim3(tc::ws::Cfg<UG>::kThreads),
+                          tc::ws::Lay<K4>::kSmem, chain, s, holos, slots, nslots, total_tiles, queue);
 }
 
 // The tails of a launch of `items` work items: clusters of as many blocks (up to
@@ -1861,8 +1878,7 @@ cudaError_t launch_tc_tails(const HoloDev *holos, const LaunchSlot *slots, int n
             const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kernel<<<grid, kTailThreads, smem, s>>>(holos, slots);
-        return cudaGetLastError();
+        return launch_chained(kernel, grid, dim3(kTailThreads), smem, chain_launch(nslots, sm_count), s, holos, slots);
     };
     switch (cl) {
     case 8: return go(tcws_tails_kernel<8>);
@@ -1872,21 +1888,21 @@ cudaError_t launch_tc_tails(const HoloDev *holos, const LaunchSlot *slots, int n
     }
 }
 
-template <int W>
 static cudaError_t tcws_launch(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles, int maxN,
                                unsigned *queue, int grid, bool subset, int f16, int sm_count, cudaStream_t s)
 {
-    constexpr int K4 = tc::ws::kKSteps;
     (void)cudaGetLastError();
-    if (f16) tcws_launch_one<W, true, K4>(holos, slots, nslots, total_tiles, queue, grid, s);
-    else tcws_launch_one<W, false, K4>(holos, slots, nslots, total_tiles, queue, grid, s);
-    const cudaError_t e = cudaGetLastError();
+    // two groups of u warps where they pay (kVWarps' comment): more than one
+    // spot block, or less than about 20 holograms' worth of work items (a
+    // block's few tiles, where latency counts)
+    const bool ug2 = tc::nspotblocks(maxN) > 1 || total_tiles < 8 * grid;
+    const bool chain = chain_launch(nslots, sm_count);
+    const auto one = f16 ? (ug2 ? tcws_launch_one<2, true> : tcws_launch_one<1, true>)
+                         : (ug2 ? tcws_launch_one<2, false> : tcws_launch_one<1, false>);
+    const cudaError_t e = one(holos, slots, nslots, total_tiles, queue, grid, chain, s);
     if (e != cudaSuccess) return e;
     return launch_tc_tails(holos, slots, nslots, total_tiles, maxN, subset, sm_count, s);
 }
-
-// epilogue warps of the warp-specialised kernel
-constexpr int kWsWarps = 16;
 
 int full_tc_tiles(int P) { return tc::tiles(P); }
 
@@ -1971,7 +1987,7 @@ int full_tc_assign_strips(LaunchSlot *slots, int nslots, const int *P, const int
 
 int full_tc_max_grid(int variant, int maxN, int sm_count)
 {
-    return variant == kFullTcWs ? tcws_max_grid<kWsWarps>(maxN, sm_count) : 0;
+    return variant == kFullTcWs ? tcws_max_grid(maxN, sm_count) : 0;
 }
 
 void full_tc_table_bytes(int P, int N, size_t *rw, size_t *c, size_t *cs)
@@ -1998,8 +2014,7 @@ cudaError_t launch_tc_rw_tables(const HoloDev *holos, const LaunchSlot *slots, i
     // at most a block of threads per table block of the largest hologram
     const int need = ((maxP + tc::kRows - 1) / tc::kRows) * tc::nchunks(maxN);
     dim3 grid((unsigned)std::max(1, std::min(need, 16 * sm_count / nslots)), (unsigned)nslots);
-    tc::rw_tables_kernel<<<grid, 256, 0, s>>>(holos, slots);
-    return cudaGetLastError();
+    return launch_chained(tc::rw_tables_kernel, grid, dim3(256), 0, chain_launch(nslots, sm_count), s, holos, slots);
 }
 
 // The shared-memory form of the mask draw for a launch whose holograms are
@@ -2055,14 +2070,14 @@ cudaError_t launch_tc_mask_scatter(const HoloDev *holos, const LaunchSlot *slots
 cudaError_t launch_subset_tc(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles, int maxN,
                              unsigned *queue, int grid, int f16, int sm_count, cudaStream_t s)
 {
-    return tcws_launch<kWsWarps>(holos, slots, nslots, total_tiles, maxN, queue, grid, true, f16, sm_count, s);
+    return tcws_launch(holos, slots, nslots, total_tiles, maxN, queue, grid, true, f16, sm_count, s);
 }
 
 cudaError_t launch_full_tc(int variant, const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles,
                            int maxN, unsigned *queue, int grid, int sm_count, cudaStream_t s)
 {
     if (variant != kFullTcWs) return cudaErrorInvalidValue;
-    return tcws_launch<kWsWarps>(holos, slots, nslots, total_tiles, maxN, queue, grid, false, 0, sm_count, s);
+    return tcws_launch(holos, slots, nslots, total_tiles, maxN, queue, grid, false, 0, sm_count, s);
 }
 
 }  // namespace cswgs

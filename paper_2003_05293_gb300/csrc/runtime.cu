@@ -232,7 +232,7 @@ cudaError_t shape_launch(TileShape shape, int kind, const HoloDev *holos, const 
         return launch_subset_tc(holos, slots, nslots, total_tiles, maxN, queue, grid, shape.fp16, sm_count, s);
     if (kind == kLaunchSubset && shape.threads == kSubsetGather)
         return launch_subset_gather(holos, slots, nslots, total_tiles, maxN, queue, grid, sm_count, s);
-    return launch_iter_fp32(shape, kind, holos, slots, nslots, total_tiles, maxN, queue, grid, s);
+    return launch_iter_fp32(shape, kind, holos, slots, nslots, total_tiles, maxN, queue, grid, sm_count, s);
 }
 
 TileShape full_fallback(TileShape shape, int maxN, int sm_count)
