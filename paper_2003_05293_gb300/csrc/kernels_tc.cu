@@ -1179,53 +1179,69 @@ __device__ __noinline__ void control_load(const HoloDev *__restrict__ holos, con
     if ((!ok || !drained) && lane0) atomicOr(status, 1u);
 }
 
+// sin and cos of 2 pi T / 2^32 + corr to FP32 rounding (corr small): the top 24
+// bits of T through sincospi, the rest and corr to first order.
+__device__ __forceinline__ float2 phasor_exact(int32_t T, float corr)
+{
+    const int32_t hi = T & ~0xFF;
+    float s, c;
+    sincospif((float)hi * 0x1p-31f, &s, &c);   // hi has 24 significant bits: exact
+    const float r = fmaf((float)(T & 0xFF), kTwoPiF * 0x1p-32f, corr);
+    return make_float2(fmaf(-s, r, c), fmaf(c, r, s));
+}
+
 // The partial V_n = sum_y conj(R_n(y)) Z(n, y) of spot n of a closed Z
 // accumulation (a strip at row block y0) over the tile's rows ys0 .. ys1 - 1.  R_n(y)
 // along the rows by recurrence: its phase is quadratic in y, so R(y + 2) =
 // R(y) D(y) and D(y + 2) = D(y) E with the constant E = e^{i (2 pi 8 Gh / 2^32
 // + 8 gl)}, the even and the odd rows side by side in packed FP32 pairs; R and
-// D are evaluated directly every 16 rows (seven steps: the product's rounding
-// grows with the run length).  Every lane computes (a lane past N uses spot
-// N - 1's factors and stores nothing): no divergent branch in the row loop.
-// A latency-bound chain on one warp per SM quarter: for holograms of more than
-// 128 spots GEMM 2 waits for it, once per spot block.
+// D are evaluated directly every 8 rows (three steps).  An error of E or D is
+// the same way round in every run and grows with its length: with hardware
+// sine and cosine for E and runs of seven steps every theta_n was off by 2e-6
+// rad rms per iteration, whatever the products' precision; E to FP32 rounding
+// and runs of three leave 2e-7 to 3e-7, as much as phasors of each pixel's own.
+// Every lane computes (a lane past N uses spot N - 1's factors and stores
+// nothing): no divergent branch in the row loop.  A latency-bound chain: for
+// holograms of more than 128 spots GEMM 2 waits for it, once per spot block.
 __device__ __forceinline__ float2 strip_dot(uint32_t z_re, uint32_t z_im, const int4 *coef, int n, int N, int y0,
                                             int half, int ys0, int ys1)
 {
     const int4 cf = coef[min(n, N - 1)];
     const int32_t tilt = cf.y, Gh = cf.z;
     const float gl = __int_as_float(cf.w);
-    float es, ec;
-    sincos_fix(kFixRound + 8u * (uint32_t)Gh, fmaf(8.f, gl, -kTwoPiF), es, ec);
-    const uint64_t E_c = pack2(ec, ec), E_s = pack2(es, es), nE_s = pack2(-es, -es);
+    const float2 E = phasor_exact((int32_t)(8u * (uint32_t)Gh), 8.f * gl);
+    const uint64_t E_c = pack2(E.x, E.x), E_s = pack2(E.y, E.y), nE_s = pack2(-E.y, -E.y);
     uint64_t vr = 0ull, vi = 0ull;   // even and odd rows; vi is the sum's negative imaginary part
 #pragma unroll 1
     for (int ys = ys0; ys < ys1; ys += 16) {
         float zr[16], zi[16];
         ld16(z_re + ys, zr);
         ld16(z_im + ys, zi);
-        const int u0 = y0 + ys - half;
-        // R at rows u0, u0 + 1 and D there: phase of R(u + 2) / R(u), tilt 2 + Gh (4 u + 4)
-        const float2 p0 = spot_factor(tilt, Gh, gl, u0, kFixRound, 1.f);
-        const float2 p1 = spot_factor(tilt, Gh, gl, u0 + 1, kFixRound, 1.f);
-        float2 d0, d1;
-        sincos_fix(kFixRound + 2u * (uint32_t)tilt + (uint32_t)Gh * (uint32_t)(4 * u0 + 4),
-                   fmaf(gl, (float)(4 * u0 + 4), -kTwoPiF), d0.y, d0.x);
-        sincos_fix(kFixRound + 2u * (uint32_t)tilt + (uint32_t)Gh * (uint32_t)(4 * u0 + 8),
-                   fmaf(gl, (float)(4 * u0 + 8), -kTwoPiF), d1.y, d1.x);
         uint64_t Rc[8], Rs[8];
-        Rc[0] = pack2(p0.x, p1.x);
-        Rs[0] = pack2(p0.y, p1.y);
-        uint64_t Dc = pack2(d0.x, d1.x), Ds = pack2(d0.y, d1.y);
 #pragma unroll
-        for (int q = 0; q < 7; ++q) {
-            const uint64_t nDs = Ds ^ 0x8000000080000000ull;
-            Rc[q + 1] = fma2(Rc[q], Dc, mul2(Rs[q], nDs));
-            Rs[q + 1] = fma2(Rc[q], Ds, mul2(Rs[q], Dc));
-            if (q < 6) {
-                const uint64_t t = fma2(Dc, E_c, mul2(Ds, nE_s));
-                Ds = fma2(Dc, E_s, mul2(Ds, E_c));
-                Dc = t;
+        for (int b = 0; b < 2; ++b) {
+            const int u0 = y0 + ys + 8 * b - half;
+            // R at rows u0, u0 + 1 and D there: phase of R(u + 2) / R(u), tilt 2 + Gh (4 u + 4)
+            const float2 p0 = spot_factor(tilt, Gh, gl, u0, kFixRound, 1.f);
+            const float2 p1 = spot_factor(tilt, Gh, gl, u0 + 1, kFixRound, 1.f);
+            float2 d0, d1;
+            sincos_fix(kFixRound + 2u * (uint32_t)tilt + (uint32_t)Gh * (uint32_t)(4 * u0 + 4),
+                       fmaf(gl, (float)(4 * u0 + 4), -kTwoPiF), d0.y, d0.x);
+            sincos_fix(kFixRound + 2u * (uint32_t)tilt + (uint32_t)Gh * (uint32_t)(4 * u0 + 8),
+                       fmaf(gl, (float)(4 * u0 + 8), -kTwoPiF), d1.y, d1.x);
+            Rc[4 * b] = pack2(p0.x, p1.x);
+            Rs[4 * b] = pack2(p0.y, p1.y);
+            uint64_t Dc = pack2(d0.x, d1.x), Ds = pack2(d0.y, d1.y);
+#pragma unroll
+            for (int q = 4 * b; q < 4 * b + 3; ++q) {
+                const uint64_t nDs = Ds ^ 0x8000000080000000ull;
+                Rc[q + 1] = fma2(Rc[q], Dc, mul2(Rs[q], nDs));
+                Rs[q + 1] = fma2(Rc[q], Ds, mul2(Rs[q], Dc));
+                if (q < 4 * b + 2) {
+                    const uint64_t t = fma2(Dc, E_c, mul2(Ds, nE_s));
+                    Ds = fma2(Dc, E_s, mul2(Ds, E_c));
+                    Dc = t;
+                }
             }
         }
         ld_wait();
