@@ -642,7 +642,8 @@ cswgs_status batch_enqueue_direct(Fp32Batch *b, cudaStream_t s, bool capturing)
         if (masked(0)) CSWGS_TRY(draw(0));
     }
     for (size_t L = 0; L < steps; ++L) {
-        if (b->timing) CSWGS_CUDA_TRY(cudaEventRecordWithFlags(b->events[L + 1], s, evflag));
+        if (b->timing && (L == 0 || L >= b->joined_steps))
+            CSWGS_CUDA_TRY(cudaEventRecordWithFlags(b->events[L + 1], s, evflag));
         for (int kind = 0; kind < 2; ++kind) {
             const size_t i = 2 * L + kind;
             const int tiles = b->l_tiles[i];

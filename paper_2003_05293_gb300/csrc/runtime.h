@@ -133,6 +133,7 @@ struct Fp32Batch {
     int grid[2] = {0, 0};                                     // resident blocks per kernel kind
     int maxN = 0;
     bool timing = false;
+    size_t joined_steps = 1;              // the first steps, timed as one (no event between them)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     std::vector<cudaEvent_t> events;      // launch boundaries (timing)

@@ -5,8 +5,8 @@
 // two, subset fraction c as the nearest power of two: a compressed launch on
 // the CUDA cores costs c times a full one, on the tensor cores about as much
 // as a full one, so the winner changes with c).  Each candidate runs a
-// synthetic batch of that key's size (one compressed iteration, one full
-// iteration, the final pass); the fastest compressed-iteration shape and the
+// synthetic batch of that key's size (three compressed iterations in a row, one
+// full iteration, the final pass; as a graph, like a user's run); the fastest compressed-iteration shape and the
 // fastest full-pass shape win.  Results live in the plan and, when the plan
 // names a cache file, in a small JSON file.
 #include <algorithm>
@@ -87,6 +87,12 @@ static const int kSubCandidates[][2] = {{128, 2}, {128, 4}, {128, 8}, {256, 2}, 
                                         {kSubsetGather, 1}};
 static const int kFullCandidates[] = {128, 256, 512, kFullTcWs};
 
+// Compressed iterations of a timed run: in a row, since a chain's launches
+// overlap and the next mask is drawn beside them (a single iteration launched
+// kernel by kernel timed the launches of small work, not the work, and the
+// choice changed from run to run: one optics' solves took 680 or 870 us).
+constexpr int kTuneSub = 3;
+
 static std::vector<HoloSpec> synthetic(const TuneKey &k, double c)
 {
     std::vector<HoloSpec> v;
@@ -98,7 +104,7 @@ static std::vector<HoloSpec> synthetic(const TuneKey &k, double c)
         s.D = s.P * s.P;   // the square uniform pupil
         s.fa = s.fb = (uint32_t)s.P;
         s.norm = (double)s.D;
-        s.iterations = 2;
+        s.iterations = kTuneSub + 1;
         s.n_full = 1;
         s.first_j = 1;
         s.final_pass = 1;
@@ -114,23 +120,33 @@ static std::vector<HoloSpec> synthetic(const TuneKey &k, double c)
     return v;
 }
 
-// Best-of-two device times of the synthetic schedule's three steps: a
-// compressed iteration, a full iteration and the final pass.
-static cswgs_status time_steps(cswgs_plan_s *p, const std::vector<HoloSpec> &specs, TileShape sh, double t[3])
+// Device times of the synthetic schedule's parts: a compressed iteration, a
+// full iteration and the final pass, each the best of three runs after a
+// warm-up; a candidate that takes half as long again as `best` (three times as
+// long in the warm-up), by which(t), is not run again.
+template <class Which>
+static cswgs_status time_steps(cswgs_plan_s *p, const std::vector<HoloSpec> &specs, TileShape sh, double best,
+                               Which which, double t[3])
 {
     std::unique_ptr<Fp32Batch> b;
     CSWGS_TRY(batch_build_with(p, specs, sh, &b));
+    b->joined_steps = kTuneSub;
     CSWGS_TRY(batch_upload_inputs(b.get(), p->stream));
     for (int i = 0; i < 3; ++i) t[i] = 1e30;
-    for (int rep = 0; rep < 3; ++rep) {
-        CSWGS_TRY(batch_enqueue_direct(b.get(), p->stream));
+    for (int rep = 0; rep < 4; ++rep) {
+        CSWGS_TRY(batch_enqueue(b.get(), p->stream));
         CSWGS_CUDA_TRY(cudaStreamSynchronize(p->stream));
-        if (rep == 0) continue;   // warm-up
+        const int first[4] = {1, 1 + kTuneSub, 2 + kTuneSub, 3 + kTuneSub};
+        double r[3];
         for (int i = 0; i < 3; ++i) {
             float ms = 0.f;
-            CSWGS_CUDA_TRY(cudaEventElapsedTime(&ms, b->events[1 + i], b->events[2 + i]));
-            t[i] = std::min(t[i], (double)ms);
+            CSWGS_CUDA_TRY(cudaEventElapsedTime(&ms, b->events[first[i]], b->events[first[i + 1]]));
+            r[i] = i == 0 ? ms / kTuneSub : ms;
         }
+        const bool slow = which(r) > (rep == 0 ? 3.0 : 1.5) * best;   // a first run is a cold one
+        if (rep == 0 && !slow) continue;
+        for (int i = 0; i < 3; ++i) t[i] = std::min(t[i], r[i]);
+        if (slow) break;
     }
     return CSWGS_OK;
 }
@@ -146,7 +162,7 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
         TileShape sh{cand[0], cand[1], best.full_threads, fp16};
         if (!shape_supported(sh)) continue;
         if (shape_max_grid(sh, kLaunchSubset, k.N, p->sm_count) <= 0) continue;
-        CSWGS_TRY(time_steps(p, specs, sh, t));
+        CSWGS_TRY(time_steps(p, specs, sh, best_sub, [](const double *r) { return r[0]; }, t));
         if (t[0] < best_sub) {
             best_sub = t[0];
             best.threads = cand[0];
@@ -156,8 +172,9 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
     for (int ft : kFullCandidates) {
         TileShape sh{best.threads, best.ppt, ft, fp16};
         if (shape_max_grid(sh, kLaunchFull, k.N, p->sm_count) <= 0) continue;
-        CSWGS_TRY(time_steps(p, specs, sh, t));
-        const double tf = wfull * t[1] + t[2];
+        const auto full_ms = [&](const double *r) { return wfull * r[1] + r[2]; };
+        CSWGS_TRY(time_steps(p, specs, sh, best_full, full_ms, t));
+        const double tf = full_ms(t);
         if (tf < best_full) {
             best_full = tf;
             best.full_threads = ft;
