@@ -37,10 +37,12 @@
 // theta and is remade before every launch.  A tile streams its blocks into shared memory
 // with bulk copies (cp.async.bulk, completion counted on an mbarrier) through
 // a ring; a producer warp issues GEMM 1's copies, two issuing warps (GEMM 1,
-// GEMM 2) issue the MMAs and commit them to mbarriers, and eight epilogue
-// warps run the CUDA-core stages: four turn S into u (epilogue 1), four reduce
-// Z to the spot fields (epilogue 2) once per strip of tiles along a row block
-// and, in the final pass, write the phase map from S.  Every wait is bounded
+// GEMM 2) issue the MMAs and commit them to mbarriers, and 12 or 16 epilogue
+// warps run the CUDA-core stages: one or two groups of four turn S into u
+// (epilogue 1), eight reduce Z to the spot fields (epilogue 2) once per strip of
+// tiles along a row block and, in the final pass, write the phase map from S.
+// The shared-memory pipe bounds a long launch of N <= 128: a tile's operand
+// reads, copies and stores of u take 8.0 k of its ~8.8 k cycles (N = 100).  Every wait is bounded
 // and a timeout is recorded in the launch's status word instead of hanging.
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
@@ -1526,7 +1528,7 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, ui
 
 // The V warps (epilogue 2): per strip (after the GEMM 2 of its last tile with
 // products) and spot block, the strip's partial V_n = sum_y conj(R_n(y))
-// Z(n, y), one spot per thread over all 128 rows, while the u warps go on with
+// Z(n, y), one spot per thread over half the 128 rows, while the u warps go on with
 // the next tiles.  In the final pass they also write each tile's phase map
 // (and gray levels) from S, beside the u warps' work on u.
 //
