@@ -16,7 +16,7 @@
 // Bound by the FP64 pipe (about 2 lanes a clock and SM): 4 FP64 multiply-adds
 // per pair and pass, against ~45 for a phasor of its own.  A 10-iteration
 // solve at P = 512, N = 100, c = 1/8 took 15.4 ms with one sincos per pair and
-// pass and takes 2.42 ms in this form.
+// pass and takes 2.32 ms in this form.
 // Phases are evaluated in FP64 with the range reduction done in turns
 // (t - rint(t)) before the double-precision sincospi.
 #include <cooperative_groups.h>
@@ -208,7 +208,9 @@ __global__ void __launch_bounds__(kF64Threads) fp64_pass(int P, int N, int rows_
 // V_n = (1 / count) sum of the items' partials, then the update or the
 // metrics, by one cluster of 8 blocks (the items' sums are FP64 additions,
 // which 8 SMs' pipes take 8 times as fast as one's).  Spots are dealt out to
-// the cluster's warps in fours: lanes are 4 spots x 8 groups of items.
+// the blocks in fours: lanes are 4 spots x 8 groups of items, and where a block
+// has warps to spare 2 to 16 of them share four spots (one warp each took 23 us
+// a pass at N = 100, 512 items, waiting for 16 loads one after another).
 constexpr int kF64Cluster = 8;
 constexpr int kF64TailThreads = 512;
 
@@ -219,17 +221,19 @@ fp64_tail(int N, int items, int64_t count, const double2 *__restrict__ part, con
     constexpr int W = kF64TailThreads / 32;
     __shared__ double s_red[3][W];
     __shared__ double s_out[3];
-    extern __shared__ double2 s_field[];   // this block's spots: V_n, four by four
+    extern __shared__ double2 s_field[];   // this block's spots: V_n, four by four; then the warps' sums
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const int rank = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int quads = (N + 3) / 4, nq = (quads - rank + kF64Cluster - 1) / kF64Cluster;
-    double sum = 0.0, imax = -1.0, imin = 1e300;
-    for (int i = warp; i < nq; i += W) {
+    int wq = W;   // warps per four spots: a power of two
+    while (wq > 1 && wq * nq > W) wq >>= 1;
+    double2 *s_sum = s_field + 4 * nq;   // [nq wq][4]
+    for (int i = warp / wq; i < nq; i += W / wq) {
         const int n = 4 * (rank + kF64Cluster * i) + (lane & 3);
         double vr = 0.0, vi = 0.0;
         if (n < N) {
-#pragma unroll 4
-            for (int t = lane >> 2; t < items; t += 8) {
+#pragma unroll 8
+            for (int t = (lane >> 2) + 8 * (warp % wq); t < items; t += 8 * wq) {
                 const double2 p = part[(size_t)t * N + n];
                 vr += p.x;
                 vi += p.y;
@@ -239,26 +243,38 @@ fp64_tail(int N, int items, int64_t count, const double2 *__restrict__ part, con
             vr += __shfl_xor_sync(0xffffffffu, vr, o);
             vi += __shfl_xor_sync(0xffffffffu, vi, o);
         }
-        if (lane < 4 && n < N) {
-            vr /= (double)count;
-            vi /= (double)count;
-            s_field[4 * i + lane] = make_double2(vr, vi);
-            if (final_pass) {
-                const double in = vr * vr + vi * vi;
-                metrics[2 + n] = in;
-                sum += in;
-                imax = fmax(imax, in);
-                imin = fmin(imin, in);
-            } else {
-                sum += hypot(vr, vi);
-            }
+        if (lane < 4) s_sum[(i * wq + warp % wq) * 4 + lane] = make_double2(vr, vi);
+    }
+    __syncthreads();
+    double sum = 0.0, imax = -1.0, imin = 1e300;
+    for (int k = tid; k < 4 * nq; k += kF64TailThreads) {   // a thread per spot
+        const int n = 4 * (rank + kF64Cluster * (k >> 2)) + (k & 3);
+        if (n >= N) continue;
+        double vr = 0.0, vi = 0.0;
+        for (int g = 0; g < wq; ++g) {
+            const double2 p = s_sum[((k >> 2) * wq + g) * 4 + (k & 3)];
+            vr += p.x;
+            vi += p.y;
+        }
+        vr /= (double)count;
+        vi /= (double)count;
+        s_field[k] = make_double2(vr, vi);
+        if (final_pass) {
+            const double in = vr * vr + vi * vi;
+            metrics[2 + n] = in;
+            sum += in;
+            imax = fmax(imax, in);
+            imin = fmin(imin, in);
+        } else {
+            sum += hypot(vr, vi);
         }
     }
-    for (int o = 1; o < 4; o <<= 1) {   // lanes 0 to 3 hold the warp's spots
-        sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        imax = fmax(imax, __shfl_xor_sync(0xffffffffu, imax, o));
-        imin = fmin(imin, __shfl_xor_sync(0xffffffffu, imin, o));
-    }
+    if (32 * warp < 4 * nq)   // the other warps hold no spot
+        for (int o = 16; o > 0; o >>= 1) {
+            sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            imax = fmax(imax, __shfl_xor_sync(0xffffffffu, imax, o));
+            imin = fmin(imin, __shfl_xor_sync(0xffffffffu, imin, o));
+        }
     if (lane == 0) {
         s_red[0][warp] = sum;
         s_red[1][warp] = imax;
@@ -266,7 +282,7 @@ fp64_tail(int N, int items, int64_t count, const double2 *__restrict__ part, con
     }
     __syncthreads();
     if (tid == 0) {
-        for (int q = 1; q < W; ++q) {
+        for (int q = 1; q < W && 32 * q < 4 * nq; ++q) {
             sum += s_red[0][q];
             imax = fmax(imax, s_red[1][q]);
             imin = fmin(imin, s_red[2][q]);
@@ -331,7 +347,9 @@ cudaError_t fp64_solve(const Fp64Work &wk, int P, int N, int Mp, int iterations,
     fp64_factors<<<dim3(blocks_for(P, 128), (unsigned)N, 2), 128, 0, s>>>(wk.xyz, N, P, wk.C, wk.R);
     const int G = N < kF64Threads ? kF64Threads / N : 1;
     const size_t smem = sizeof(double2) * ((size_t)N + (size_t)G * N + kF64Seg + kF64Threads) + sizeof(int) * kF64Seg;
-    const size_t tail_smem = sizeof(double2) * 4 * (size_t)((N + 31) / 32);
+    // V_n of a block's fours, and the warps' sums (at least W entries of four, or one per four)
+    const size_t nq = (size_t)((N + 31) / 32);
+    const size_t tail_smem = sizeof(double2) * 4 * (nq + std::max<size_t>(nq, kF64TailThreads / 32));
     cudaError_t e = cudaFuncSetAttribute(fp64_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     auto tail = [&](int64_t count, int fin) {
