@@ -35,6 +35,10 @@ constexpr int kF64Threads = 512;
 constexpr int kF64Seg = 1024;       // listed pixels of a row held in shared memory at a time
 constexpr int kF64MaskSeg = 1024;   // columns listed at a time (32 mask words: one warp scan)
 static_assert(kF64MaskSeg <= kF64Seg, "a column segment's pixels fit the list");
+// The pass's limit of dynamic shared memory, the same at every launch: it belongs
+// to the function, so a solve that set it to its own need would take it from
+// another thread's solve in the middle of its launches.  (N = 4096 needs 156 KB.)
+constexpr size_t kF64MaxSmem = 200 * 1024;
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b)
 {
@@ -350,7 +354,8 @@ cudaError_t fp64_solve(const Fp64Work &wk, int P, int N, int Mp, int iterations,
     // V_n of a block's fours, and the warps' sums (at least W entries of four, or one per four)
     const size_t nq = (size_t)((N + 31) / 32);
     const size_t tail_smem = sizeof(double2) * 4 * (nq + std::max<size_t>(nq, kF64TailThreads / 32));
-    cudaError_t e = cudaFuncSetAttribute(fp64_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > kF64MaxSmem) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(fp64_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF64MaxSmem);
     if (e != cudaSuccess) return e;
     auto tail = [&](int64_t count, int fin) {
         fp64_tail<<<kF64Cluster, kF64TailThreads, tail_smem, s>>>(N, items, count, wk.part, wk.amp, wk.w, wk.theta,

@@ -1909,8 +1909,9 @@ cudaError_t launch_tc_tails(const HoloDev *holos, const LaunchSlot *slots, int n
     const dim3 grid((unsigned)(cl * nslots), 1u + (subset ? (unsigned)(kTailClear / cl) : 0u));
     const size_t smem = tail_smem((maxN + 4 * cl - 1) / (4 * cl));
     auto go = [&](auto kernel) {
-        if (smem > 48 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (smem > 48 * 1024) {   // a limit for every launch, not this one's need: other threads launch it too
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)tail_smem(kTailMaxN / 4));
             if (e != cudaSuccess) return e;
         }
         return launch_chained(kernel, grid, dim3(kTailThreads), smem, chain_launch(nslots, sm_count), s, holos, slots);
@@ -2066,8 +2067,9 @@ static int mask_local_shape(int maxP, int nslots, int sm_count, size_t *smem)
     while (G > 1 && G * nslots > sm_count) G >>= 1;
     // the mask, and four tables of at most maxP 16-bit entries (doubled: below 2^16)
     *smem = (((size_t)maxP * (size_t)mask_words_of(maxP) + 3) & ~(size_t)3) * 4 + 4 * 2 * (size_t)(maxP + 1);
-    if (*smem > 220 * 1024) return 0;
-    if (cudaFuncSetAttribute(tc::mask_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem) !=
+    constexpr size_t kMaxSmem = 220 * 1024;   // the function's limit, which other threads' launches share
+    if (*smem > kMaxSmem) return 0;
+    if (cudaFuncSetAttribute(tc::mask_local_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) !=
         cudaSuccess) {
         (void)cudaGetLastError();
         return 0;
