@@ -695,7 +695,7 @@ cswgs_status batch_enqueue(Fp32Batch *b, cudaStream_t s)
         CSWGS_CUDA_TRY(cudaGraphInstantiate(&b->exec, g, 0));
     }
     // the plan's bounded-wait test words (queue[3], queue[4]), when they changed
-    const unsigned want[2] = {b->plan->test_withhold, b->plan->test_polls};
+    const unsigned want[2] = {b->test_hook ? b->plan->test_withhold : 0u, b->test_hook ? b->plan->test_polls : 0u};
     if (want[0] != b->test_words[0] || want[1] != b->test_words[1]) {
         CSWGS_CUDA_TRY(cudaMemcpyAsync(b->queue_d.as<unsigned>() + 3, want, sizeof want, cudaMemcpyHostToDevice, s));
         CSWGS_CUDA_TRY(cudaStreamSynchronize(s));   // `want` lives on this stack frame

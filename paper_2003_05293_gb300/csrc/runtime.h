@@ -134,6 +134,7 @@ struct Fp32Batch {
     int maxN = 0;
     bool timing = false;
     size_t joined_steps = 1;              // the first steps, timed as one (no event between them)
+    bool test_hook = true;                // runs under the plan's bounded-wait test (the autotuner's do not)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     std::vector<cudaEvent_t> events;      // launch boundaries (timing)

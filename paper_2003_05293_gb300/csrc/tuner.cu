@@ -131,6 +131,7 @@ static cswgs_status time_steps(cswgs_plan_s *p, const std::vector<HoloSpec> &spe
     std::unique_ptr<Fp32Batch> b;
     CSWGS_TRY(batch_build_with(p, specs, sh, &b));
     b->joined_steps = kTuneSub;
+    b->test_hook = false;
     CSWGS_TRY(batch_upload_inputs(b.get(), p->stream));
     for (int i = 0; i < 3; ++i) t[i] = 1e30;
     for (int rep = 0; rep < 4; ++rep) {
