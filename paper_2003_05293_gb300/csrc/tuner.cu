@@ -5,10 +5,11 @@
 // two, subset fraction c as the nearest power of two: a compressed launch on
 // the CUDA cores costs c times a full one, on the tensor cores about as much
 // as a full one, so the winner changes with c).  Each candidate runs a
-// synthetic batch of that key's size (three compressed iterations in a row, one
-// full iteration, the final pass; as a graph, like a user's run); the fastest compressed-iteration shape and the
-// fastest full-pass shape win.  Results live in the plan and, when the plan
-// names a cache file, in a small JSON file.
+// synthetic batch of that key's size (three compressed iterations in a row, or
+// one full iteration and the final pass; as a graph, like a user's run); the
+// fastest compressed-iteration shape and the fastest full-pass shape win.
+// Results live in the plan and, when the plan names a cache file, in a small
+// JSON file.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -93,7 +94,9 @@ static const int kFullCandidates[] = {128, 256, 512, kFullTcWs};
 // choice changed from run to run: one optics' solves took 680 or 870 us).
 constexpr int kTuneSub = 3;
 
-static std::vector<HoloSpec> synthetic(const TuneKey &k, double c)
+// A synthetic batch of the key's size: kTuneSub compressed iterations, or a full
+// iteration and the final pass.
+static std::vector<HoloSpec> synthetic(const TuneKey &k, double c, bool full)
 {
     std::vector<HoloSpec> v;
     for (int b = 0; b < k.B; ++b) {
@@ -104,10 +107,10 @@ static std::vector<HoloSpec> synthetic(const TuneKey &k, double c)
         s.D = s.P * s.P;   // the square uniform pupil
         s.fa = s.fb = (uint32_t)s.P;
         s.norm = (double)s.D;
-        s.iterations = kTuneSub + 1;
-        s.n_full = 1;
+        s.iterations = full ? 1 : kTuneSub;
+        s.n_full = full ? 1 : 0;
         s.first_j = 1;
-        s.final_pass = 1;
+        s.final_pass = full ? 1 : 0;
         s.seed = 0x5EEDull + (uint64_t)b;
         s.xyz.resize(3 * (size_t)s.N);
         uint64_t x = 12345 + (uint64_t)b;
@@ -120,33 +123,32 @@ static std::vector<HoloSpec> synthetic(const TuneKey &k, double c)
     return v;
 }
 
-// Device times of the synthetic schedule's parts: a compressed iteration, a
-// full iteration and the final pass, each the best of three runs after a
+// Device times (ms) of the synthetic schedule's parts: a compressed iteration,
+// or a full iteration and the final pass, each the best of three runs after a
 // warm-up; a candidate that takes half as long again as `best` (three times as
-// long in the warm-up), by which(t), is not run again.
-template <class Which>
-static cswgs_status time_steps(cswgs_plan_s *p, const std::vector<HoloSpec> &specs, TileShape sh, double best,
-                               Which which, double t[3])
+// long in the warm-up), by cost(t), is not run again.
+template <class Cost>
+static cswgs_status time_steps(cswgs_plan_s *p, const std::vector<HoloSpec> &specs, TileShape sh, bool full,
+                               double best, Cost cost, double t[2])
 {
     std::unique_ptr<Fp32Batch> b;
     CSWGS_TRY(batch_build_with(p, specs, sh, &b));
-    b->joined_steps = kTuneSub;
+    b->joined_steps = full ? 1 : kTuneSub;
     b->test_hook = false;
     CSWGS_TRY(batch_upload_inputs(b.get(), p->stream));
-    for (int i = 0; i < 3; ++i) t[i] = 1e30;
+    t[0] = t[1] = 1e30;
     for (int rep = 0; rep < 4; ++rep) {
         CSWGS_TRY(batch_enqueue(b.get(), p->stream));
         CSWGS_CUDA_TRY(cudaStreamSynchronize(p->stream));
-        const int first[4] = {1, 1 + kTuneSub, 2 + kTuneSub, 3 + kTuneSub};
-        double r[3];
-        for (int i = 0; i < 3; ++i) {
+        double r[2] = {0.0, 0.0};
+        for (int i = 0; i < (full ? 2 : 1); ++i) {
             float ms = 0.f;
-            CSWGS_CUDA_TRY(cudaEventElapsedTime(&ms, b->events[first[i]], b->events[first[i + 1]]));
-            r[i] = i == 0 ? ms / kTuneSub : ms;
+            CSWGS_CUDA_TRY(cudaEventElapsedTime(&ms, b->events[1 + i], b->events[full ? 2 + i : 1 + kTuneSub]));
+            r[i] = full ? ms : ms / kTuneSub;
         }
-        const bool slow = which(r) > (rep == 0 ? 3.0 : 1.5) * best;   // a first run is a cold one
+        const bool slow = cost(r) > (rep == 0 ? 3.0 : 1.5) * best;   // a first run is a cold one
         if (rep == 0 && !slow) continue;
-        for (int i = 0; i < 3; ++i) t[i] = std::min(t[i], r[i]);
+        for (int i = 0; i < 2; ++i) t[i] = std::min(t[i], r[i]);
         if (slow) break;
     }
     return CSWGS_OK;
@@ -155,29 +157,29 @@ static cswgs_status time_steps(cswgs_plan_s *p, const std::vector<HoloSpec> &spe
 static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double wsub, double wfull,
                              TileShape *best_shape, double *best_ms)
 {
-    std::vector<HoloSpec> specs = synthetic(k, c);
     const int fp16 = p->desc.precision == CSWGS_FP32_FP16SINCOS ? 1 : 0;
     TileShape best{256, 4, 256, fp16};
-    double best_sub = 1e30, best_full = 1e30, t[3];
+    double best_sub = 1e30, best_full = 1e30, t[2];
+    std::vector<HoloSpec> specs = synthetic(k, c, false);
     for (const auto &cand : kSubCandidates) {
         TileShape sh{cand[0], cand[1], best.full_threads, fp16};
         if (!shape_supported(sh)) continue;
         if (shape_max_grid(sh, kLaunchSubset, k.N, p->sm_count) <= 0) continue;
-        CSWGS_TRY(time_steps(p, specs, sh, best_sub, [](const double *r) { return r[0]; }, t));
+        CSWGS_TRY(time_steps(p, specs, sh, false, best_sub, [](const double *r) { return r[0]; }, t));
         if (t[0] < best_sub) {
             best_sub = t[0];
             best.threads = cand[0];
             best.ppt = cand[1];
         }
     }
+    specs = synthetic(k, c, true);
     for (int ft : kFullCandidates) {
         TileShape sh{best.threads, best.ppt, ft, fp16};
         if (shape_max_grid(sh, kLaunchFull, k.N, p->sm_count) <= 0) continue;
-        const auto full_ms = [&](const double *r) { return wfull * r[1] + r[2]; };
-        CSWGS_TRY(time_steps(p, specs, sh, best_full, full_ms, t));
-        const double tf = full_ms(t);
-        if (tf < best_full) {
-            best_full = tf;
+        const auto cost = [&](const double *r) { return wfull * r[0] + r[1]; };
+        CSWGS_TRY(time_steps(p, specs, sh, true, best_full, cost, t));
+        if (cost(t) < best_full) {
+            best_full = cost(t);
             best.full_threads = ft;
         }
     }
