@@ -7,9 +7,9 @@
 // as a full one, so the winner changes with c).  Each candidate runs a
 // synthetic batch of that key's size (three compressed iterations in a row, or
 // one full iteration and the final pass; as a graph, like a user's run); the
-// fastest compressed-iteration shape and the fastest full-pass shape win.
-// Results live in the plan and, when the plan names a cache file, in a small
-// JSON file.
+// fastest compressed-iteration shape and the fastest full-pass shape win, with
+// a margin against the tensor cores.  Results live in the plan and, when the
+// plan names a cache file, in a small JSON file.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -94,6 +94,21 @@ static const int kFullCandidates[] = {128, 256, 512, kFullTcWs};
 // choice changed from run to run: one optics' solves took 680 or 870 us).
 constexpr int kTuneSub = 3;
 
+// The tensor cores' products keep 16 bits of their operands and drop what falls
+// below FP32's last bit, the CUDA cores' kernels work in FP32: the pick is part
+// of what a caller gets for a size.  So it keeps to the lines that the timings
+// drew when the tensor-core launches still summed their partials on one SM per
+// hologram, rather than move with each gain of those launches: they are taken
+// for compressed iterations when 1.25 times as fast, and for full passes when
+// they win by what those sums cost, 0.25 us a pass and spot (7 at least, 25 at
+// most).  Without the margins 48 of 432 sizes (P = 128 to 1152, N = 16 to 512, c
+// = 1 to 1/32, batches of 1 to 64) moved their compressed iterations and 91 their
+// full passes to the tensor cores, and a whole solve of P = 64 came out 1.1e-5
+// from exact instead of 1.5e-6; with them 10 and 4 do (of the old timings' own
+// picks, 5 % differed from one run to the next).
+constexpr double kTcSubGain = 1.25;
+static double tc_full_margin_ms(int N) { return 1e-3 * std::clamp(0.25 * N, 7.0, 25.0); }
+
 // A synthetic batch of the key's size: kTuneSub compressed iterations, or a full
 // iteration and the final pass.
 static std::vector<HoloSpec> synthetic(const TuneKey &k, double c, bool full)
@@ -159,15 +174,18 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
 {
     const int fp16 = p->desc.precision == CSWGS_FP32_FP16SINCOS ? 1 : 0;
     TileShape best{256, 4, 256, fp16};
-    double best_sub = 1e30, best_full = 1e30, t[2];
+    double best_sub = 1e30, best_full = 1e30, ms_sub = 0.0, ms_full = 0.0, t[2];
     std::vector<HoloSpec> specs = synthetic(k, c, false);
     for (const auto &cand : kSubCandidates) {
         TileShape sh{cand[0], cand[1], best.full_threads, fp16};
         if (!shape_supported(sh)) continue;
         if (shape_max_grid(sh, kLaunchSubset, k.N, p->sm_count) <= 0) continue;
-        CSWGS_TRY(time_steps(p, specs, sh, false, best_sub, [](const double *r) { return r[0]; }, t));
-        if (t[0] < best_sub) {
-            best_sub = t[0];
+        const double gain = cand[0] == kSubsetTc ? kTcSubGain : 1.0;
+        const auto cost = [&](const double *r) { return gain * r[0]; };
+        CSWGS_TRY(time_steps(p, specs, sh, false, best_sub, cost, t));
+        if (cost(t) < best_sub) {
+            best_sub = cost(t);
+            ms_sub = t[0];
             best.threads = cand[0];
             best.ppt = cand[1];
         }
@@ -176,15 +194,17 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
     for (int ft : kFullCandidates) {
         TileShape sh{best.threads, best.ppt, ft, fp16};
         if (shape_max_grid(sh, kLaunchFull, k.N, p->sm_count) <= 0) continue;
-        const auto cost = [&](const double *r) { return wfull * r[0] + r[1]; };
+        const double margin = is_full_tc(ft) ? tc_full_margin_ms(k.N) : 0.0;
+        const auto cost = [&](const double *r) { return wfull * (r[0] + margin) + r[1] + margin; };
         CSWGS_TRY(time_steps(p, specs, sh, true, best_full, cost, t));
         if (cost(t) < best_full) {
             best_full = cost(t);
+            ms_full = wfull * t[0] + t[1];
             best.full_threads = ft;
         }
     }
     *best_shape = best;
-    if (best_ms) *best_ms = wsub * best_sub + best_full;
+    if (best_ms) *best_ms = wsub * ms_sub + ms_full;
     return CSWGS_OK;
 }
 

@@ -20,3 +20,21 @@ def test_bounded_wait_test_does_not_reach_the_tuning(polls):
         held = p.autotune(1152, 1000, 0.125)
         p.test_waits(False, 0)
     assert 0.5 * ms < held < 2.0 * ms
+
+
+def test_kernels_of_fp32_products_where_the_tensor_cores_hardly_win(tmp_path):
+    """A choice of the tensor cores (products of 16-bit halves) needs more than a
+    lead of a few percent over the FP32 kernels: full passes at P = 64, N = 10
+    (65 us against 66 for three), a compressed iteration at P = 512, N = 100 (23
+    against 24).  Where they win clearly they stay: P = 1152, N = 100 (28
+    against 48; full passes 92 against 300)."""
+    import json
+    from paper_2003_05293_gb300 import Plan
+    path = tmp_path / "t.json"
+    with Plan(precision="fp32", tune_cache=str(path)) as p:
+        for P, N, c in ((64, 10, 0.25), (512, 100, 0.125), (1152, 100, 0.125)):
+            p.autotune(P, N, c)
+    picks = json.loads(path.read_text())["entries"]
+    assert picks["P128_N16_B1_c2"][0] > 3 and picks["P128_N16_B1_c2"][2] > 2
+    assert picks["P512_N128_B1_c3"][0] > 3
+    assert picks["P1152_N128_B1_c3"][0] == 1 and picks["P1152_N128_B1_c3"][2] == 2
