@@ -175,6 +175,7 @@ struct cswgs_plan_s {
     std::map<std::string, std::unique_ptr<cswgs::Fp32Batch>> solve_cache;
     std::map<std::string, cswgs::TileShape> tune;
     std::string tune_path;
+    bool tune_any_pupil = false;    // the tune cache file's entries hold for every pupil (an older file)
     // FP64 solver workspace
     cswgs::DevBuf f64_mem;
     // small device scratch for results
@@ -208,7 +209,6 @@ namespace cswgs {
 // autotuner
 TileShape tuned_shape(cswgs_plan_s *p, const std::vector<HoloSpec> &specs);
 cswgs_status tune_batch(cswgs_plan_s *p, Fp32Batch *b, double *best_ms);
-std::string tune_key(const std::vector<HoloSpec> &specs, bool fp16);
 void tune_load(cswgs_plan_s *p);
 void tune_save(cswgs_plan_s *p);
 }  // namespace cswgs

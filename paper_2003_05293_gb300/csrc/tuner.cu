@@ -4,7 +4,10 @@
 // count rounded up to a power of two, batch size rounded up to a power of
 // two, subset fraction c as the nearest power of two: a compressed launch on
 // the CUDA cores costs c times a full one, on the tensor cores about as much
-// as a full one, so the winner changes with c).  Each candidate runs a
+// as a full one, so the winner changes with c; and whether the pupil is round
+// and the beam Gaussian, since a round pupil has fewer pixels and dearer draws:
+// the paper's optics took 960 us a solve with the direct-phasor shape that
+// is best on a square of their size and take 668).  Each candidate runs a
 // synthetic batch of that key's size (three compressed iterations in a row, or
 // one full iteration and the final pass; as a graph, like a user's run); the
 // fastest compressed-iteration shape and the fastest full-pass shape win, with
@@ -34,6 +37,7 @@ static int pow2_ceil(int x)
 struct TuneKey {
     int P, N, B;
     int cexp;   // c = 2^-cexp (0 .. 16)
+    bool round, beam;   // most of the work under a round pupil, a Gaussian beam
 };
 
 // The subset fraction of a batch, weighted by each hologram's compressed
@@ -54,12 +58,14 @@ static double batch_c(const std::vector<HoloSpec> &specs)
 static TuneKey key_of(const std::vector<HoloSpec> &specs)
 {
     int P = 0;
-    double wsum = 0.0, nw = 0.0;
+    double wsum = 0.0, nw = 0.0, round = 0.0, beam = 0.0;
     for (auto &s : specs) {
         P = std::max(P, s.P);
         double w = (double)s.P * s.P * s.N;
         wsum += w;
         nw += w * s.N;
+        round += s.aperture == CSWGS_APERTURE_ROUND ? w : 0.0;
+        beam += s.waist > 0.0 ? w : 0.0;
     }
     int N = wsum > 0 ? (int)std::lround(nw / wsum) : 1;
     TuneKey k;
@@ -68,14 +74,18 @@ static TuneKey key_of(const std::vector<HoloSpec> &specs)
     k.B = pow2_ceil((int)specs.size());
     const double c = batch_c(specs);
     k.cexp = std::min(16, std::max(0, (int)std::lround(-std::log2(std::max(c, 1e-9)))));
+    k.round = 2.0 * round > wsum;
+    k.beam = 2.0 * beam > wsum;
     return k;
 }
 
-std::string tune_key(const std::vector<HoloSpec> &specs, bool fp16)
+// The key's name: "P1152_N64_B1_c3", then "_R" (round), "_G" (Gaussian), "_H"
+// (half precision); `pupil` false leaves the pupil's letters out.
+static std::string tune_key(const TuneKey &k, bool fp16, bool pupil = true)
 {
-    TuneKey k = key_of(specs);
     char buf[64];
-    snprintf(buf, sizeof buf, "P%d_N%d_B%d_c%d%s", k.P, k.N, k.B, k.cexp, fp16 ? "_H" : "");
+    snprintf(buf, sizeof buf, "P%d_N%d_B%d_c%d%s%s%s", k.P, k.N, k.B, k.cexp, pupil && k.round ? "_R" : "",
+             pupil && k.beam ? "_G" : "", fp16 ? "_H" : "");
     return buf;
 }
 
@@ -111,17 +121,18 @@ static double tc_full_margin_ms(int N) { return 1e-3 * std::clamp(0.25 * N, 7.0,
 
 // A synthetic batch of the key's size: kTuneSub compressed iterations, or a full
 // iteration and the final pass.
-static std::vector<HoloSpec> synthetic(const TuneKey &k, double c, bool full)
+static cswgs_status synthetic(cswgs_plan_s *p, const TuneKey &k, double c, bool full, std::vector<HoloSpec> *out)
 {
-    std::vector<HoloSpec> v;
+    HoloSpec pupil;
+    pupil.P = std::min(k.P, 4096);
+    cswgs_pupil pu{};
+    pu.aperture = k.round ? CSWGS_APERTURE_ROUND : CSWGS_APERTURE_SQUARE;
+    pu.beam_waist = k.beam ? 0.5 * pupil.P : 0.0;
+    CSWGS_TRY(apply_pupil(p, pu, std::max(c, 2.0 / ((double)pupil.P * pupil.P)), &pupil));   // one pixel at least
+    out->clear();
     for (int b = 0; b < k.B; ++b) {
-        HoloSpec s;
-        s.P = std::min(k.P, 4096);
+        HoloSpec s = pupil;
         s.N = k.N;
-        s.Mp = std::max(1, (int)std::floor(c * (double)s.P * s.P));
-        s.D = s.P * s.P;   // the square uniform pupil
-        s.fa = s.fb = (uint32_t)s.P;
-        s.norm = (double)s.D;
         s.iterations = full ? 1 : kTuneSub;
         s.n_full = full ? 1 : 0;
         s.first_j = 1;
@@ -133,9 +144,9 @@ static std::vector<HoloSpec> synthetic(const TuneKey &k, double c, bool full)
             x = x * 6364136223846793005ull + 1442695040888963407ull;
             q = ((double)(x >> 11) * 0x1.0p-53 - 0.5) * (s.P / 2.0);
         }
-        v.push_back(std::move(s));
+        out->push_back(std::move(s));
     }
-    return v;
+    return CSWGS_OK;
 }
 
 // Device times (ms) of the synthetic schedule's parts: a compressed iteration,
@@ -175,7 +186,8 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
     const int fp16 = p->desc.precision == CSWGS_FP32_FP16SINCOS ? 1 : 0;
     TileShape best{256, 4, 256, fp16};
     double best_sub = 1e30, best_full = 1e30, ms_sub = 0.0, ms_full = 0.0, t[2];
-    std::vector<HoloSpec> specs = synthetic(k, c, false);
+    std::vector<HoloSpec> specs;
+    CSWGS_TRY(synthetic(p, k, c, false, &specs));
     for (const auto &cand : kSubCandidates) {
         TileShape sh{cand[0], cand[1], best.full_threads, fp16};
         if (!shape_supported(sh)) continue;
@@ -190,7 +202,7 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
             best.ppt = cand[1];
         }
     }
-    specs = synthetic(k, c, true);
+    CSWGS_TRY(synthetic(p, k, c, true, &specs));
     for (int ft : kFullCandidates) {
         TileShape sh{best.threads, best.ppt, ft, fp16};
         if (shape_max_grid(sh, kLaunchFull, k.N, p->sm_count) <= 0) continue;
@@ -211,8 +223,10 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
 TileShape tuned_shape(cswgs_plan_s *p, const std::vector<HoloSpec> &specs)
 {
     const bool fp16 = p->desc.precision == CSWGS_FP32_FP16SINCOS;
-    std::string key = tune_key(specs, fp16);
+    const TuneKey k = key_of(specs);
+    const std::string key = tune_key(k, fp16);
     auto it = p->tune.find(key);
+    if (it == p->tune.end() && p->tune_any_pupil) it = p->tune.find(tune_key(k, fp16, false));
     if (it != p->tune.end()) return it->second;
     // tune now, with the schedule's own mix of compressed and full iterations
     double wsub = 0.0, wfull = 0.0;
@@ -221,14 +235,14 @@ TileShape tuned_shape(cswgs_plan_s *p, const std::vector<HoloSpec> &specs)
         wsub += s.iterations - F;
         wfull += F;
     }
-    const double c = std::ldexp(1.0, -key_of(specs).cexp);   // the key's c: one tuning per bucket
+    const double c = std::ldexp(1.0, -k.cexp);   // the key's c: one tuning per bucket
     if (!specs.empty()) {
         wsub /= specs.size();
         wfull /= specs.size();
     }
     TileShape sh{256, 4, 256, fp16 ? 1 : 0};
     double ms = 0.0;
-    if (tune_for(p, key_of(specs), c, wsub, wfull, &sh, &ms) == CSWGS_OK) {
+    if (tune_for(p, k, c, wsub, wfull, &sh, &ms) == CSWGS_OK) {
         p->tune[key] = sh;
         tune_save(p);
     }
@@ -247,7 +261,7 @@ cswgs_status tune_single(cswgs_plan_s *p, int P, int N, double c, double *best_m
     TuneKey k = key_of(v);
     TileShape sh;
     CSWGS_TRY(tune_for(p, k, c, 28.0, 2.0, &sh, best_ms));
-    p->tune[tune_key(v, p->desc.precision == CSWGS_FP32_FP16SINCOS)] = sh;
+    p->tune[tune_key(k, p->desc.precision == CSWGS_FP32_FP16SINCOS)] = sh;
     tune_save(p);
     return CSWGS_OK;
 }
@@ -276,6 +290,8 @@ void tune_load(cswgs_plan_s *p)
         if (got < 4 || st < 0 || st > 4096) st = 0;
         if (shape_supported(TileShape{t, k, f, fp16, st})) p->tune[key] = TileShape{t, k, f, fp16, st};
     }
+    // files before format 4 have no pupil in their keys: an entry holds for every pupil
+    p->tune_any_pupil = !p->tune.empty() && s.find("\"cswgs-tune-4\"") == std::string::npos;
 }
 
 void tune_save(cswgs_plan_s *p)
@@ -284,7 +300,7 @@ void tune_save(cswgs_plan_s *p)
     std::string tmp = p->tune_path + ".tmp";
     FILE *f = fopen(tmp.c_str(), "w");
     if (!f) return;
-    fprintf(f, "{\n  \"format\": \"cswgs-tune-3\",\n  \"entries\": {");
+    fprintf(f, "{\n  \"format\": \"cswgs-tune-%d\",\n  \"entries\": {", p->tune_any_pupil ? 3 : 4);
     bool first = true;
     for (auto &kv : p->tune) {
         fprintf(f, "%s\n    \"%s\": [%d, %d, %d, %d]", first ? "" : ",", kv.first.c_str(), kv.second.threads,

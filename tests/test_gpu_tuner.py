@@ -38,3 +38,26 @@ def test_kernels_of_fp32_products_where_the_tensor_cores_hardly_win(tmp_path):
     assert picks["P128_N16_B1_c2"][0] > 3 and picks["P128_N16_B1_c2"][2] > 2
     assert picks["P512_N128_B1_c3"][0] > 3
     assert picks["P1152_N128_B1_c3"][0] == 1 and picks["P1152_N128_B1_c3"][2] == 2
+
+
+def test_round_pupils_are_tuned_on_round_pupils(tmp_path):
+    """A round pupil or a Gaussian beam has a tuning of its own (fewer pixels, dearer
+    draws than the square's); entries of cache files written before the pupil was
+    in their keys hold for every pupil, as they did."""
+    import json
+    import workloads
+    from gpu_helpers import write_pinned_tune_cache
+    from paper_2003_05293_gb300 import Plan
+    square, rnd = (workloads.problem(256, 20, 5.0, 0.25, 3, seed=1) for _ in range(2))
+    rnd.extra = dict(aperture="round", waist=120.0)
+    path = tmp_path / "new.json"
+    for first in (square, rnd):   # the second plan finds the first one's file
+        with Plan(precision="fp32", tune_cache=str(path)) as p:
+            p.batch([first], None).close()
+    d = json.loads(path.read_text())
+    assert d["format"] == "cswgs-tune-4" and set(d["entries"]) == {"P256_N32_B1_c2", "P256_N32_B1_c2_R_G"}
+    path = write_pinned_tune_cache(tmp_path / "old.json", 1, 1, 2)
+    with Plan(precision="fp32", tune_cache=path) as p:
+        b = p.batch([rnd], None)
+        assert b.tile_shape()["threads"] == 1 and b.tile_shape()["full_threads"] == 2
+        b.close()
