@@ -14,8 +14,8 @@
 // GEMM 1 sets each pixel's phase: its FP32 operands are split into two FP16
 // halves, v = hi + lo, and each real product is kept as hi hi + hi lo + lo hi
 // (22 bits of each operand: 2^-22 relative per product, FP32-class phases; BF16
-// halves, which keep 16 bits, left a 300-spot final pass 1.0e-5 from exact where
-// these leave 3.4e-6).  FP16's range asks for scaled operands: |C| and |u| are
+// halves, which keep 16 bits, left errors of 3e-6 in the spot states where
+// these leave 1e-6).  FP16's range asks for scaled operands: |C| and |u| are
 // at most 1, and R' is scaled per hologram by a power of two (S is needed up
 // to a factor only).  It runs its complex product as two real ones stacked
 // along N (M = 128 rows, N = 128, K = 16 spots):
@@ -726,7 +726,6 @@ struct Info {
     int first, last;   // the first / last tile with products of the strip
     int zero;          // the strip's last tile, and the strip has no products
     uint32_t before;   // tiles with products published before this one
-    int tiles;         // tiles with products of the strip
     LaunchSlot sl;
     HoloDev H;
 };
@@ -1150,7 +1149,6 @@ __device__ __noinline__ void control_load(const HoloDev *__restrict__ holos, con
                     info[j].last = c == cl ? 1 : 0;
                     info[j].zero = (cf < 0 && c == c1 - 1) ? 1 : 0;
                     info[j].before = before;
-                    info[j].tiles = cl - cf + 1;
                     info[j].sl = sl;
                 }
                 uint32_t *dst = reinterpret_cast<uint32_t *>(&info[j].H);
@@ -1531,15 +1529,7 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, ui
 // Z(n, y), one spot per thread over half the 128 rows, while the u warps go on with
 // the next tiles.  In the final pass they also write each tile's phase map
 // (and gray levels) from S, beside the u warps' work on u.
-//
-// Z's accumulation drops the bits below FP32's last towards zero: measured, 3.4e-8
-// of what it holds per product (0.57 units of 2^-24), half that of the final
-// value for a sum that grows evenly, as a spot's does.  The partial is scaled
-// by as much: it is the same for every spot and leaves Eqs. 4-6 alone, but e
-// came out 1.5e-6 low with strips of one tile, 3.1e-6 with three and 8e-6 with nine.
-constexpr float kZLoss = 3.4e-8f;
-
-template <int UG, bool F16>
+template <int UG>
 __device__ __forceinline__ void epilogue_v(const Info *info, float2 (*s_half)[kSpotBlock], uint32_t mb, uint32_t tmem,
                                            unsigned *status)
 {
@@ -1557,8 +1547,6 @@ __device__ __forceinline__ void epilogue_v(const Info *info, float2 (*s_half)[kS
         const int item = info[j].item, empty = info[j].empty, t = info[j].tile, last = info[j].last;
         const int tile_begin = info[j].sl.tile_begin, pass = info[j].sl.pass;
         const int P = info[j].H.P, N = info[j].H.N;
-        // products accumulated per component: per K-step 2 (FP16) or 6
-        const float gain = 1.f + 0.5f * kZLoss * (float)(info[j].tiles * kKSteps * (F16 ? 2 : 6));
         const int4 *coef = info[j].H.coef;
         float2 *part = info[j].H.part;
         double2 *part64 = info[j].H.part64;
@@ -1603,8 +1591,8 @@ __device__ __forceinline__ void epilogue_v(const Info *info, float2 (*s_half)[kS
             ok = warp_and(wait_newest(mbar_at(mb, kDot0 + buf), (n_z + 1u) >> 1));
             if (!ok) break;
             const float2 w = s_half[buf][32 * q + lane];
-            v.x = (v.x + w.x) * gain;
-            v.y = (v.y + w.y) * gain;
+            v.x += w.x;
+            v.y += w.y;
             if (n < N) {
                 const size_t off = (size_t)s_loc * N + n;
                 if (pass == kPassFinal) part64[off] = make_double2((double)v.x, (double)v.y);
@@ -1684,7 +1672,7 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
     } else if (warp < Cfg<UG>::kU) {
         epilogue_u<UG, F16, US>(m, s_info, mb, s_tmem, status);
     } else {
-        epilogue_v<UG, F16>(s_info, s_half, mb, s_tmem, status);
+        epilogue_v<UG>(s_info, s_half, mb, s_tmem, status);
     }
     tc::fence_before();
     __syncthreads();
