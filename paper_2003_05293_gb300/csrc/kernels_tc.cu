@@ -853,13 +853,8 @@ __device__ __forceinline__ bool load_gemm1(Ctl &C, const HoloDev &H, int rb, int
         if (elect_one()) {
             const uint32_t stg = C.ring + s * kStage, full = mbar_at(C.mb, kFull0 + s);
             expect_tx(full, kStage);
-            // every other tile takes the chunks backwards: the accumulation drops the
-            // bits below FP32's last towards zero at each product, so a chunk's
-            // spots lose in proportion to the products after it (5e-6 over the 114
-            // of N = 300); over two tiles of opposite order all lose alike
-            const int cc = ((rb ^ cb) & 1) ? nc - 1 - c : c;
-            bulk_load(stg, H.rwtab + ((size_t)rb * nc + cc) * (4 * kA1), 4 * kA1, full);
-            bulk_load(stg + 4 * kA1, H.ctab + ((size_t)cb * nc + cc) * (2 * kB1), 2 * kB1, full);
+            bulk_load(stg, H.rwtab + ((size_t)rb * nc + c) * (4 * kA1), 4 * kA1, full);
+            bulk_load(stg + 4 * kA1, H.ctab + ((size_t)cb * nc + c) * (2 * kB1), 2 * kB1, full);
         }
         __syncwarp();
         C.ql++;

@@ -60,3 +60,7 @@ def final(tmp_path_factory):
 def test_efficiency(golden, solve, final):
     assert abs(solve["e"] / golden["solve_eu"][0] - 1) < TOL_E
     assert abs(final["e"] / golden["final_eu"][0] - 1) < TOL_E
+
+
+def test_intensities(golden, final):
+    assert np.std(final["I"] / golden["final_I"]) < TOL_I_SPREAD
