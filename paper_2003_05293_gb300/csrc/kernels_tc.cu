@@ -1181,38 +1181,37 @@ __device__ __noinline__ void control_load(const HoloDev *__restrict__ holos, con
     if ((!ok || !drained) && lane0) atomicOr(status, 1u);
 }
 
-// sin and cos of 2 pi T / 2^32 + corr to FP32 rounding (corr small): the top 24
-// bits of T through sincospi, the rest and corr to first order.
-__device__ __forceinline__ float2 phasor_exact(int32_t T, float corr)
+// a b for complex a, b.
+__device__ __forceinline__ float2 cmul(float2 a, float2 b)
 {
-    const int32_t hi = T & ~0xFF;
-    float s, c;
-    sincospif((float)hi * 0x1p-31f, &s, &c);   // hi has 24 significant bits: exact
-    const float r = fmaf((float)(T & 0xFF), kTwoPiF * 0x1p-32f, corr);
-    return make_float2(fmaf(-s, r, c), fmaf(c, r, s));
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
 // The partial V_n = sum_y conj(R_n(y)) Z(n, y) of spot n of a closed Z
 // accumulation (a strip at row block y0) over the tile's rows ys0 .. ys1 - 1.  R_n(y)
-// along the rows by recurrence: its phase is quadratic in y, so R(y + 2) =
-// R(y) D(y) and D(y + 2) = D(y) E with the constant E = e^{i (2 pi 8 Gh / 2^32
-// + 8 gl)}, the even and the odd rows side by side in packed FP32 pairs; R and
-// D are evaluated directly every 8 rows (three steps).  An error of E or D is
-// the same way round in every run and grows with its length: with hardware
-// sine and cosine for E and runs of seven steps every theta_n was off by 2e-6
-// rad rms per iteration, whatever the products' precision; E to FP32 rounding
-// and runs of three leave 2e-7 to 3e-7, as much as phasors of each pixel's own.
+// along the rows by recurrence: its phase is quadratic in y, so R(y + 1) =
+// R(y) D(y) and D(y + 1) = D(y) E with the constant E = e^{i (2 pi 2 Gh / 2^32
+// + 2 gl)}; R and D are evaluated directly every 8 rows (the product's
+// rounding grows with the run length).  Within a run the even and the odd rows
+// go side by side in packed FP32 pairs, which the rows' Z are in as loaded:
+// R(y + 2) = R(y) D2(y) and D2(y + 2) = D2(y) E^4 from D2(y) = D(y) D(y + 1).
 // Every lane computes (a lane past N uses spot N - 1's factors and stores
 // nothing): no divergent branch in the row loop.  A latency-bound chain: for
 // holograms of more than 128 spots GEMM 2 waits for it, once per spot block.
+// (Two runs in a pair instead, rows y and y + 8: seven steps one after the other
+// and Z's rows moved into pairs; 64 holograms of N up to 300 12.34 ms against
+// 11.93.)
 __device__ __forceinline__ float2 strip_dot(uint32_t z_re, uint32_t z_im, const int4 *coef, int n, int N, int y0,
                                             int half, int ys0, int ys1)
 {
     const int4 cf = coef[min(n, N - 1)];
     const int32_t tilt = cf.y, Gh = cf.z;
     const float gl = __int_as_float(cf.w);
-    const float2 E = phasor_exact((int32_t)(8u * (uint32_t)Gh), 8.f * gl);
-    const uint64_t E_c = pack2(E.x, E.x), E_s = pack2(E.y, E.y), nE_s = pack2(-E.y, -E.y);
+    float2 E;
+    sincos_fix(kFixRound + 2u * (uint32_t)Gh, fmaf(2.f, gl, -kTwoPiF), E.y, E.x);
+    const float2 E2 = cmul(E, E), E3 = cmul(E2, E), E4 = cmul(E2, E2);
+    const uint64_t F_c = pack2(E.x, E3.x), F_s = pack2(E.y, E3.y), nF_s = pack2(-E.y, -E3.y);
+    const uint64_t E_c = pack2(E4.x, E4.x), E_s = pack2(E4.y, E4.y), nE_s = pack2(-E4.y, -E4.y);
     uint64_t vr = 0ull, vi = 0ull;   // even and odd rows; vi is the sum's negative imaginary part
 #pragma unroll 1
     for (int ys = ys0; ys < ys1; ys += 16) {
@@ -1222,18 +1221,16 @@ __device__ __forceinline__ float2 strip_dot(uint32_t z_re, uint32_t z_im, const 
         uint64_t Rc[8], Rs[8];
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            const int u0 = y0 + ys + 8 * b - half;
-            // R at rows u0, u0 + 1 and D there: phase of R(u + 2) / R(u), tilt 2 + Gh (4 u + 4)
-            const float2 p0 = spot_factor(tilt, Gh, gl, u0, kFixRound, 1.f);
-            const float2 p1 = spot_factor(tilt, Gh, gl, u0 + 1, kFixRound, 1.f);
-            float2 d0, d1;
-            sincos_fix(kFixRound + 2u * (uint32_t)tilt + (uint32_t)Gh * (uint32_t)(4 * u0 + 4),
-                       fmaf(gl, (float)(4 * u0 + 4), -kTwoPiF), d0.y, d0.x);
-            sincos_fix(kFixRound + 2u * (uint32_t)tilt + (uint32_t)Gh * (uint32_t)(4 * u0 + 8),
-                       fmaf(gl, (float)(4 * u0 + 8), -kTwoPiF), d1.y, d1.x);
-            Rc[4 * b] = pack2(p0.x, p1.x);
-            Rs[4 * b] = pack2(p0.y, p1.y);
-            uint64_t Dc = pack2(d0.x, d1.x), Ds = pack2(d0.y, d1.y);
+            const int u0 = y0 + ys + 8 * b - half, du = 2 * u0 + 1;
+            // R at row u0 and D there: phase of R(u + 1) / R(u), tilt + Gh (2 u + 1)
+            const float2 r = spot_factor(tilt, Gh, gl, u0, kFixRound, 1.f);
+            float2 d;
+            sincos_fix(kFixRound + (uint32_t)tilt + (uint32_t)Gh * (uint32_t)du, fmaf(gl, (float)du, -kTwoPiF), d.y, d.x);
+            const float2 r1 = cmul(r, d), dd = cmul(d, d);
+            const uint64_t dc = pack2(dd.x, dd.x), ds = pack2(dd.y, dd.y);
+            Rc[4 * b] = pack2(r.x, r1.x);
+            Rs[4 * b] = pack2(r.y, r1.y);
+            uint64_t Dc = fma2(dc, F_c, mul2(ds, nF_s)), Ds = fma2(dc, F_s, mul2(ds, F_c));   // D2: D^2 E | D^2 E^3
 #pragma unroll
             for (int q = 4 * b; q < 4 * b + 3; ++q) {
                 const uint64_t nDs = Ds ^ 0x8000000080000000ull;

@@ -64,3 +64,7 @@ def test_efficiency(golden, solve, final):
 
 def test_intensities(golden, final):
     assert np.std(final["I"] / golden["final_I"]) < TOL_I_SPREAD
+
+
+def test_spot_phases(golden, solve):
+    assert rms_wrapped(solve["theta"], golden["solve_theta"]) < TOL_THETA
