@@ -94,11 +94,10 @@ def kernel_name(tile, kind):
 
 
 def dtype_label(tile):
-    """The arithmetic the path computes in: FP32, or FP32-class split-FP16
+    """The arithmetic the path computes in: FP32, or FP32-class split-BF16
     products accumulated in FP32 on the tensor cores."""
     if tile["threads"] == SUBSET_TC or tile["full_threads"] in TC_KERNELS:
-        return ("f32-class: split-fp16 x3 products (in place of split-bf16 x3), f32 accumulate (tensor cores); "
-                "f32 epilogues; f64 e, u")
+        return "f32-class: split-bf16 x3 products, f32 accumulate (tensor cores); f32 epilogues; f64 e, u"
     return "f32 (f64 e, u)"
 
 
@@ -123,14 +122,14 @@ def subset_roofline(tile, pairs_sub_launch, n_sub, sub_ms, full_ms, sm_count, ma
     2 SFU results (sin, cos) per subset pixel-spot pair and pass against the
     SFU peak.  On the tensor cores: algorithmic flops, 8 per subset pair and
     pass (one complex multiply-add), against the dense BF16 peak; the kernel
-    runs every pixel (M / Mp times the subset) with 3 FP16 products per real
+    runs every pixel (M / Mp times the subset) with 3 BF16 products per real
     product."""
     share = 100 * sub_ms / max(1e-9, sub_ms + full_ms)
     if tile["threads"] == SUBSET_TC:
         peak, basis = tensor_peak()
         ach = 8.0 * pairs_sub_launch * n_sub / (sub_ms * 1e-3) / 1e12 if n_sub else 0.0
         Mp = math.floor(args.c * args.P * args.P)
-        return {"bound": "tensor", "pipe": "tcgen05 kind::f16 (FP16 in, FP32 accumulate)", "achieved": ach,
+        return {"bound": "tensor", "pipe": "tcgen05 kind::f16 (BF16 in, FP32 accumulate)", "achieved": ach,
                 "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "traffic": traffic,
                 "peak_basis": "%s dense BF16 peak" % basis,
                 "flops_basis": "8 flops (complex multiply-add) per subset pixel-spot pair and pass",
@@ -185,7 +184,7 @@ def launches_per_step(tile, n_sub, n_full):
 
 def full_roofline(tile, achieved_tflops, fma_peak, sm_count, max_mhz, traffic, n_launches, full_ms):
     """Roofline of the full-iteration and final launches: the tensor-core kernel
-    against the measured dense BF16 peak (FP16, its operands' type, has the same rate), the
+    against the measured dense BF16 peak (its operands are BF16 halves), the
     CUDA-core kernel against the FP32 FMA peak.  Achieved = algorithmic flops:
     8 per pixel-spot pair and pass (one complex multiply-add)."""
     base = {"achieved": achieved_tflops, "unit": "TFLOP/s", "traffic": traffic,
@@ -193,12 +192,12 @@ def full_roofline(tile, achieved_tflops, fma_peak, sm_count, max_mhz, traffic, n
             "ms_per_launch": full_ms / max(1, n_launches)}
     if tile["full_threads"] in TC_KERNELS:
         peak, basis = tensor_peak()
-        base.update({"bound": "tensor", "pipe": "tcgen05 kind::f16 (FP16 in, FP32 accumulate)", "peak": peak,
+        base.update({"bound": "tensor", "pipe": "tcgen05 kind::f16 (BF16 in, FP32 accumulate)", "peak": peak,
                      "frac": achieved_tflops / peak, "peak_basis": "%s dense BF16 peak" % basis,
                      "kernel": "%s, full-iteration and final launches (%d per step)"
                                % (TC_KERNELS[tile["full_threads"]][0], n_launches),
                      "issued_tensor_flops_per_algorithmic": 3,
-                     "note": "each real product is 3 FP16 products (hi hi + hi lo + lo hi) for FP32-class "
+                     "note": "each real product is 3 BF16 products (hi hi + hi lo + lo hi) for FP32-class "
                              "accuracy, so the tensor pipe runs 3x the algorithmic flops",
                      "tile": {"threads": TC_KERNELS[tile["full_threads"]][1], "blocks": tile["full_blocks"],
                               "pixels": "128 rows x 64 columns"}})

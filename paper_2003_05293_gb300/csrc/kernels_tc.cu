@@ -11,23 +11,20 @@
 // A compressed iteration is the same computation with u zero outside the
 // subset S_j, so the sums run over S_j as Eqs. 1 and 3 ask.
 // The accumulators (FP32) live in tensor memory.
-// GEMM 1 sets each pixel's phase: its FP32 operands are split into two FP16
+// GEMM 1 sets each pixel's phase: its FP32 operands are split into two BF16
 // halves, v = hi + lo, and each real product is kept as hi hi + hi lo + lo hi
-// (22 bits of each operand: 2^-22 relative per product, FP32-class phases; BF16
-// halves, which keep 16 bits, left errors of 3e-6 in the spot states where
-// these leave 1e-6).  FP16's range asks for scaled operands: |C| and |u| are
-// at most 1, and R' is scaled per hologram by a power of two (S is needed up
-// to a factor only).  It runs its complex product as two real ones stacked
-// along N (M = 128 rows, N = 128, K = 16 spots):
+// (2^-16 relative per product, FP32-class phases).  It runs its complex
+// product as two real ones stacked along N (M = 128 rows, N = 128, K = 16
+// spots):
 //   [S_re | S_im] = R'_re [C_re | C_im] + R'_im [-C_im | C_re],
 // with the two B operands as two 128-row windows of one 192-row tile
 // [-C_im | C_re | C_im]: 6 instructions per spot chunk.
 // GEMM 2 (the forward projection) is M = 128 spots x N = 128 rows x K = 16
 // columns per instruction (N = 256 where real and imaginary parts share an A
-// operand), with split FP16 operands too (9 instructions per K-step).  The
-// half-precision option (compressed launches only) takes the operands' FP16
-// roundings alone (|u|, |C| <= 1; 3 instructions per K-step): the sums run over many pixels whose
-// rounding errors (2^-12 relative) do not add up coherently.
+// operand), with split BF16 operands too (9 instructions per K-step).  The
+// half-precision option (compressed launches only) takes single FP16 operands
+// instead (|u|, |C| <= 1; 3 instructions per K-step): the sums run over many
+// pixels whose rounding errors (2^-12 relative) do not add up coherently.
 //
 // The operands are factor tables in global memory, laid out block by block
 // exactly as the MMAs read them from shared memory (no-swizzle K-major core
@@ -45,6 +42,7 @@
 // reads, copies and stores of u take 8.0 k of its ~8.8 k cycles (N = 100).  Every wait is bounded
 // and a timeout is recorded in the launch's status word instead of hanging.
 #include <cooperative_groups.h>
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -91,7 +89,7 @@ __host__ __device__ inline size_t cs_table_bytes(int P, int N)
 
 __device__ __forceinline__ uint32_t saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Byte offset of element (row, k) of a [rows][K] FP16 tile in the no-swizzle
+// Byte offset of element (row, k) of a [rows][K] 16-bit tile in the no-swizzle
 // K-major layout: core matrices of 8 rows x 8 elements (16 bytes a row, 128
 // bytes each), the K / 8 cores of a row group side by side.
 __device__ __forceinline__ uint32_t core_off(int row, int k, int K)
@@ -108,11 +106,12 @@ __device__ __forceinline__ uint64_t desc(uint32_t start, uint32_t lbo, uint32_t 
            ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
 }
 
-// Instruction descriptor, kind::f16: D FP32, A and B both FP16 (type 0), both
-// K-major, M x N.
-__host__ __device__ constexpr uint32_t idesc(int M, int N, int neg_a)
+// Instruction descriptor, kind::f16: D FP32, A and B both BF16 (bf16 = 1) or
+// both FP16 (bf16 = 0), both K-major, M x N.
+__host__ __device__ constexpr uint32_t idesc(int M, int N, int neg_a, int bf16 = 1)
 {
-    return (1u << 4) | ((uint32_t)neg_a << 13) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+    return (1u << 4) | ((uint32_t)bf16 << 7) | ((uint32_t)bf16 << 10) | ((uint32_t)neg_a << 13) |
+           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc)
@@ -184,22 +183,27 @@ __device__ __forceinline__ uint32_t h2_bits(__half2 h)
     return (uint32_t)__half_as_ushort(__low2half(h)) | ((uint32_t)__half_as_ushort(__high2half(h)) << 16);
 }
 
-// The FP16 halves of a pair of values, converted together (round to nearest):
-// hi = fp16(v), lo = fp16(v - hi).
+__device__ __forceinline__ uint32_t bf16x2_bits(__nv_bfloat162 h)
+{
+    return (uint32_t)__bfloat16_as_ushort(h.x) | ((uint32_t)__bfloat16_as_ushort(h.y) << 16);
+}
+
+// The BF16 halves of a pair of values, converted together (round to nearest):
+// hi = bf16(v), lo = bf16(v - hi).
 struct Split2 {
-    __half2 hi, lo;
+    __nv_bfloat162 hi, lo;
 };
 
 __device__ __forceinline__ Split2 split2(float a, float b)
 {
     Split2 r;
-    r.hi = __floats2half2_rn(a, b);
-    const float2 f = __half22float2(r.hi);
-    r.lo = __floats2half2_rn(a - f.x, b - f.y);
+    r.hi = __floats2bfloat162_rn(a, b);
+    const float2 f = __bfloat1622float2(r.hi);
+    r.lo = __floats2bfloat162_rn(a - f.x, b - f.y);
     return r;
 }
 
-// Eight complex values -> the four FP16 component rows (re hi, re lo, im hi,
+// Eight complex values -> the four BF16 component rows (re hi, re lo, im hi,
 // im lo), one 16-byte store each, at byte offset `off` of four tiles `stride`
 // bytes apart.
 __device__ __forceinline__ void put8(unsigned char *base, uint32_t stride, uint32_t off, const float2 *v)
@@ -208,10 +212,10 @@ __device__ __forceinline__ void put8(unsigned char *base, uint32_t stride, uint3
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const Split2 re = split2(v[2 * q].x, v[2 * q + 1].x), im = split2(v[2 * q].y, v[2 * q + 1].y);
-        w[0][q] = h2_bits(re.hi);
-        w[1][q] = h2_bits(re.lo);
-        w[2][q] = h2_bits(im.hi);
-        w[3][q] = h2_bits(im.lo);
+        w[0][q] = bf16x2_bits(re.hi);
+        w[1][q] = bf16x2_bits(re.lo);
+        w[2][q] = bf16x2_bits(im.hi);
+        w[3][q] = bf16x2_bits(im.lo);
     }
 #pragma unroll
     for (int c = 0; c < 4; ++c)
@@ -276,11 +280,17 @@ __device__ __forceinline__ float rsqrt_approx(float x)
     return r;
 }
 
-// Eight complex values of u, split for GEMM 2 and packed (the four
-// component rows, or re hi and im hi), to be stored once their slot is free.
+// Eight complex values of u, split for GEMM 2 and packed (the four BF16
+// component rows, or the two FP16 ones), to be stored once their slot is free.
 struct Packed8 {
     uint32_t w[4][4];
 };
+
+// The two values of a BF16 pair as an FP32 pair (a BF16 is an FP32's upper half).
+__device__ __forceinline__ uint64_t bf16x2_floats(uint32_t h)
+{
+    return pack2(__uint_as_float(h << 16), __uint_as_float(h & 0xFFFF0000u));
+}
 
 // |S|^2 of 16 pixels, two by two, and whether every one is a normal FP32
 // number (false for a NaN: min.NaN keeps it).
@@ -333,25 +343,25 @@ __device__ __forceinline__ Packed8 pack8(const uint64_t *ur, const uint64_t *ui)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const float2 a = unpack2(ur[q]), b = unpack2(ui[q]);
-        const __half2 rh = __floats2half2_rn(a.x, a.y), ih = __floats2half2_rn(b.x, b.y);
         if (F16) {
-            p.w[0][q] = h2_bits(rh);
-            p.w[1][q] = h2_bits(ih);
+            p.w[0][q] = h2_bits(__floats2half2_rn(a.x, a.y));
+            p.w[1][q] = h2_bits(__floats2half2_rn(b.x, b.y));
             p.w[2][q] = p.w[3][q] = 0u;
         } else {
-            const float2 rf = __half22float2(rh), jf = __half22float2(ih);
-            const float2 rl = unpack2(sub2(ur[q], pack2(rf.x, rf.y))), il = unpack2(sub2(ui[q], pack2(jf.x, jf.y)));
-            p.w[0][q] = h2_bits(rh);
-            p.w[1][q] = h2_bits(__floats2half2_rn(rl.x, rl.y));
-            p.w[2][q] = h2_bits(ih);
-            p.w[3][q] = h2_bits(__floats2half2_rn(il.x, il.y));
+            const uint32_t rh = bf16x2_bits(__floats2bfloat162_rn(a.x, a.y));
+            const uint32_t ih = bf16x2_bits(__floats2bfloat162_rn(b.x, b.y));
+            const float2 rl = unpack2(sub2(ur[q], bf16x2_floats(rh))), il = unpack2(sub2(ui[q], bf16x2_floats(ih)));
+            p.w[0][q] = rh;
+            p.w[1][q] = bf16x2_bits(__floats2bfloat162_rn(rl.x, rl.y));
+            p.w[2][q] = ih;
+            p.w[3][q] = bf16x2_bits(__floats2bfloat162_rn(il.x, il.y));
         }
     }
     return p;
 }
 
 // The rows of a Packed8 at byte offset `off` of the component tiles `stride`
-// bytes apart: re hi, im hi, re lo, im lo; or re hi, im hi alone.
+// bytes apart: split BF16 re hi, im hi, re lo, im lo; FP16 re, im.
 template <bool F16>
 __device__ __forceinline__ void store8(unsigned char *base, uint32_t stride, uint32_t off, const Packed8 &p)
 {
@@ -366,7 +376,7 @@ __device__ __forceinline__ void store8(unsigned char *base, uint32_t stride, uin
 // Items of eight phasors; consecutive threads take consecutive rows of one
 // core matrix, so a warp's 16-byte stores fill whole 128-byte lines.
 
-// Eight values -> rows of the two FP16 halves (hi, lo) of a stacked C block:
+// Eight values -> rows of the two BF16 halves (hi, lo) of a stacked C block:
 // hi at base, lo at base + kB1, row offsets re_off, im_off (C_im) and
 // neg_off (-C_im); each a 16-byte store.
 __device__ __forceinline__ void put8_stacked(unsigned char *base, uint32_t re_off, uint32_t im_off,
@@ -376,12 +386,12 @@ __device__ __forceinline__ void put8_stacked(unsigned char *base, uint32_t re_of
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const Split2 re = split2(v[2 * q].x, v[2 * q + 1].x), im = split2(v[2 * q].y, v[2 * q + 1].y);
-        w[0][q] = h2_bits(re.hi);
-        w[1][q] = h2_bits(re.lo);
-        w[2][q] = h2_bits(im.hi);
-        w[3][q] = h2_bits(im.lo);
-        w[4][q] = h2_bits(__hneg2(im.hi));   // the split of -v is -(hi), -(lo): exact
-        w[5][q] = h2_bits(__hneg2(im.lo));
+        w[0][q] = bf16x2_bits(re.hi);
+        w[1][q] = bf16x2_bits(re.lo);
+        w[2][q] = bf16x2_bits(im.hi);
+        w[3][q] = bf16x2_bits(im.lo);
+        w[4][q] = bf16x2_bits(__hneg2(im.hi));   // the split of -v is -(hi), -(lo): exact
+        w[5][q] = bf16x2_bits(__hneg2(im.lo));
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -395,8 +405,8 @@ __device__ __forceinline__ void put8_stacked(unsigned char *base, uint32_t re_of
 // C (GEMM 1's B: per block of 64 columns and 16 spots, each half a 192-row
 // tile [-C_im | C_re | C_im] with row = column within each third) and C for
 // GEMM 2 (128 spots x 64 columns per block, stored K-step by K-step: 4 x [the
-// components of 128 spots x 16 columns]; for the half-precision option also
-// the FP16 roundings alone, re and im) of hologram blockIdx.y, from its
+// components of 128 spots x 16 columns]; split BF16, and for the
+// half-precision option also FP16 re and im) of hologram blockIdx.y, from its
 // spot coefficients.
 __global__ void __launch_bounds__(256) const_tables_kernel(const HoloDev *__restrict__ holos, int count)
 {
@@ -598,8 +608,7 @@ __global__ void __launch_bounds__(256) rw_tables_kernel(const HoloDev *__restric
     // one block (128 rows x 16 spots) per pass of the loop: its 16 spots' row
     // coefficients and state are read once into shared memory
     __shared__ int4 s_cf[kChunk];      // {B, Gh, gl, theta + rounding}
-    __shared__ float s_wa[kChunk];     // w a, scaled
-    __shared__ uint32_t s_max[8];
+    __shared__ float s_wa[kChunk];     // w a
     chain_start();
     const LaunchSlot sl = slots[blockIdx.y];
     const HoloDev H = holos[sl.holo];
@@ -609,18 +618,6 @@ __global__ void __launch_bounds__(256) rw_tables_kernel(const HoloDev *__restric
     const int blocks = ((P + kRows - 1) / kRows) * nc;   // (128 rows, 16 spots) blocks, 256 threads each
     const int j = threadIdx.x;
     const int row = (j & 7) + 8 * (j >> 4), g = (j >> 3) & 1;
-    // the hologram's largest |w a|, by the bits (which order like the values)
-    uint32_t mx = 0u;
-    for (int n = j; n < N; n += 256) mx = max(mx, __float_as_uint(fabsf(H.state[n].w * H.state[n].a0)));
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    if ((j & 31) == 0) s_max[j >> 5] = mx;
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 8; ++q) mx = max(mx, s_max[q]);
-    // 2^(8 - e) for a largest value in [2^(e - 1), 2^e): FP16 halves of values up
-    // to 2^8 keep 22 bits of every spot down to 2^-11 of it (and 2^-24 itself)
-    const int e2 = (int)(mx >> 23) - 126;   // 0 and denormals: -126
-    const float scale = mx >= 0x7F800000u ? 1.f : ldexpf(1.f, min(8 - e2, 120));
     for (int blk = blockIdx.x; blk < blocks; blk += gridDim.x) {
         const int rb = blk / nc, c = blk % nc;
         __syncthreads();   // the previous block's spots are read
@@ -632,7 +629,7 @@ __global__ void __launch_bounds__(256) rw_tables_kernel(const HoloDev *__restric
                 const int4 cf = H.coef[n];
                 const SpotState st = H.state[n];
                 v = make_int4(cf.y, cf.z, cf.w, (int)(st.theta + kFixRound));
-                wa = st.w * st.a0 * scale;
+                wa = st.w * st.a0;
             }
             s_cf[j] = v;
             s_wa[j] = wa;
@@ -901,8 +898,8 @@ __device__ __forceinline__ bool gemm1(Ctl &C, int nc, int j)
 // GEMM 2 of one tile: Z = conj(C)^T u, one block of 128 spots at a time, into
 // columns 0..255; each block's C (its four K-steps one after the other)
 // streams in once the MMAs that read the previous one are done (block 0 while
-// u is still being written).  Split operands (4 components each), or their
-// FP16 roundings (re and im) for the half-precision option.  The first tile of a strip (and
+// u is still being written).  Split BF16 operands (4 components each), or FP16
+// re and im for the half-precision option.  The first tile of a strip (and
 // each spot block past the first) opens a Z accumulation, once the epilogue
 // has read the last one; the last tile of a strip (and each spot block but the
 // last) closes it.  After each K-step of the last spot block, u's columns of
@@ -911,8 +908,9 @@ template <bool F16, int US>
 __device__ __forceinline__ bool gemm2(Ctl &C, const G2Info &g)
 {
     const uint32_t comps = F16 ? 2u : 4u, kbytes = comps * kCk;
-    const uint32_t id2 = idesc(kSpotBlock, 2 * kRows, 0), id = idesc(kSpotBlock, kRows, 0),
-                   idn = idesc(kSpotBlock, kRows, 1);
+    constexpr int kBf16 = F16 ? 0 : 1;
+    const uint32_t id2 = idesc(kSpotBlock, 2 * kRows, 0, kBf16), id = idesc(kSpotBlock, kRows, 0, kBf16),
+                   idn = idesc(kSpotBlock, kRows, 1, kBf16);
     const uint32_t z_re = C.tmem, z_im = C.tmem + kRows;
     const uint64_t cs0 = desc(C.cs, 128, 256);                       // [128 spots][16 columns] per component
     const uint64_t u0 = desc(C.u, 128, 256);                         // [128 rows][16 columns] per component

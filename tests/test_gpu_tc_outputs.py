@@ -68,3 +68,8 @@ def test_intensities(golden, final):
 
 def test_spot_phases(golden, solve):
     assert rms_wrapped(solve["theta"], golden["solve_theta"]) < TOL_THETA
+
+
+def test_phase_map(golden, final):
+    d = wrap(final["map"].astype(np.float64) - golden["final_map"])
+    assert np.sqrt(np.mean(d * d)) < TOL_MAP_RMS and np.abs(d).max() < TOL_MAP_MAX
