@@ -1932,17 +1932,13 @@ int full_tc_assign_strips(LaunchSlot *slots, int nslots, const int *P, const int
                           int *chosen)
 {
     using namespace tc;
-    // Z's accumulation in tensor memory drops the bits below FP32's last at every
-    // instruction (24 per tile and component), always towards zero: over 18 tiles
-    // e = sum |V_n|^2 came out 1.1e-5 low, so a strip takes 9 at most
-    constexpr int kMaxStrip = 9;
     grid = std::max(1, grid);
     auto cols = [&](int i) { return (P[i] + kCols - 1) / kCols; };
     auto rows = [&](int i) { return (P[i] + kRows - 1) / kRows; };
-    auto strip_of = [&](int i, int S) { return nspotblocks(N[i]) == 1 ? std::min({S, cols(i), kMaxStrip}) : 1; };
+    auto strip_of = [&](int i, int S) { return nspotblocks(N[i]) == 1 ? std::min(S, cols(i)) : 1; };
     int smax = 1;
     for (int i = 0; i < nslots; ++i)
-        if (nspotblocks(N[i]) == 1) smax = std::max(smax, std::min(cols(i), kMaxStrip));
+        if (nspotblocks(N[i]) == 1) smax = std::max(smax, cols(i));
     // The launch's finish time for strip length S, in tiles: the persistent
     // blocks take the work items in queue order, each the next free block
     // (simulated with a heap of the blocks' finish times); an item costs its
