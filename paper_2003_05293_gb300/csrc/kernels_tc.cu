@@ -674,7 +674,8 @@ __global__ void __launch_bounds__(256) rw_tables_kernel(const HoloDev *__restric
 //   s_empty[2]        the tile's u warps have read that S buffer and info slot, the
 //                     V and GEMM warps that info slot
 //   u_step[4]         the u warps have written u's columns of one K-step of GEMM 2
-//   u_free[2][4]      GEMM 2 has read them, per S buffer
+//   u_free[2][4]      GEMM 2 has read them, by the parity of the tile's number
+//                     among those with products
 //   cs_full           GEMM 2's C block has landed
 //   cs_free           the MMAs that read it are done (its buffer is free)
 //   z_full            a Z accumulation is done: a strip, or one spot block of a tile
@@ -697,7 +698,7 @@ enum Bar {
     kSFull0 = kEmpty0 + kRingMax,
     kSEmpty0 = kSFull0 + 2,
     kUStep0 = kSEmpty0 + 2,       // u's columns of GEMM 2's K-step 0 .. 3 are written
-    kUFree0 = kUStep0 + kKSteps,  // ... and GEMM 2 has read them, per S buffer
+    kUFree0 = kUStep0 + kKSteps,  // ... and GEMM 2 has read them, by the parity of the product tile's number
     kCsFull = kUFree0 + 2 * kKSteps,  // GEMM 2's C block has landed
     kCsFree,                      // the MMAs that read it are done
     kZFull,                       // a Z accumulation is done
@@ -710,7 +711,7 @@ enum Bar {
 // The GEMM 2 warp's work item: a published tile with products.
 struct G2Info {
     const unsigned char *cstab;   // GEMM 2's C blocks in the launch's format
-    int nsb, cb, j;               // j: the tile's S buffer
+    int nsb, cb;
     int first, last;              // the tile opens / closes its strip's Z accumulation
 };
 
@@ -914,6 +915,7 @@ __device__ __forceinline__ bool gemm2(Ctl &C, const G2Info &g)
     const uint32_t z_re = C.tmem, z_im = C.tmem + kRows;
     const uint64_t cs0 = desc(C.cs, 128, 256);                       // [128 spots][16 columns] per component
     const uint64_t u0 = desc(C.u, 128, 256);                         // [128 rows][16 columns] per component
+    const int ufree = kUFree0 + kKSteps * (int)(C.nu & 1u);          // this tile's releases of u
     for (int sb = 0; sb < g.nsb; ++sb) {
         if (C.ncs > 0 && !warp_wait(mbar_at(C.mb, kCsFree), C.ncs - 1u)) return false;
         if (elect_one()) {
@@ -956,7 +958,7 @@ __device__ __forceinline__ bool gemm2(Ctl &C, const G2Info &g)
                     mma(z_im, cih, url, idn, 1u);
                     mma(z_im, cil, urh, idn, 1u);
                 }
-                if (sb == g.nsb - 1) commit(mbar_at(C.mb, kUFree0 + kKSteps * g.j + ks));
+                if (sb == g.nsb - 1) commit(mbar_at(C.mb, ufree + ks));
             }
             __syncwarp();
         }
@@ -1019,7 +1021,6 @@ __device__ __noinline__ void control_gemm2(const SmemWs &m, const Info *info, ui
         g.cstab = F16 ? info[j].H.cstab16 : info[j].H.cstab;
         g.nsb = nspotblocks(info[j].H.N);
         g.cb = info[j].tile % ((P + kCols - 1) / kCols);
-        g.j = j;
         g.first = info[j].first;
         g.last = info[j].last;
         __syncwarp();
@@ -1404,12 +1405,6 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, ui
                     if (H.slm) H.slm[(size_t)r * H.slm_pitch + c] = g0;
                 }
             }
-            // the other buffer's phases are looked at here as well (see below)
-            const uint32_t other = before - ((n_seen >> (16 * j)) & 0xFFFFu);
-            if (UG == 2 && other > 0u)
-                for (int ks = 0; ks < kKSteps && ok; ++ks)
-                    ok = warp_and(wait_newest(mbar_at(mb, kUFree0 + kKSteps * (j ^ 1) + ks), other));
-            if (!ok) break;
             continue;
         }
 
@@ -1427,10 +1422,9 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, ui
             }
         }
         // tiles with products on this S buffer up to this one (s_full[j] completes
-        // once per such tile), and on the other one before it
+        // once per such tile)
         n_seen += 1u << (16 * j);
-        const uint32_t n_s = (n_seen >> (16 * j)) & 0xFFFFu, other = before + 1u - n_s;
-        ok = warp_and(wait_newest(mbar_at(mb, kSFull0 + j), n_s));
+        ok = warp_and(wait_newest(mbar_at(mb, kSFull0 + j), (n_seen >> (16 * j)) & 0xFFFFu));
         if (!ok) break;
         fence_after();
         {
@@ -1484,15 +1478,18 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, ui
                         }
                         pk[g] = pack8<F16>(ur, ui);
                     }
-                    // u's slot of this K-step is free once GEMM 2 has read the
-                    // last u in it: that of the last tile on the other S buffer or on
-                    // this one.  Each buffer has its own phases, and since a group
-                    // looks at both at every tile (UG = 2: at an empty one too) no
-                    // wait is more than one phase short.  (The conditions are the same in every lane,
-                    // so the warp's votes stay matched.)
-                    if (other > 0u && !warp_and(wait_newest(mbar_at(mb, kUFree0 + kKSteps * (j ^ 1) + ks), other)))
-                        return false;
-                    if (n_s > 1u && !warp_and(wait_newest(mbar_at(mb, kUFree0 + kKSteps * j + ks), n_s - 1u)))
+                    // u's slot of this K-step is free once GEMM 2 has read the last u
+                    // in it, that of the last tile with products (number before - 1).
+                    // A wait by parity has to find its phase current or just over:
+                    // GEMM 2 can't be past that tile, since it waits for this one's u;
+                    // and the phase before on that barrier, of tile before - 3, was over
+                    // for tile before - 2's u, which this group wrote, or GEMM 2 took in
+                    // before this tile was published.  (Phases counted per S buffer
+                    // left the two groups without either bound: a group that looked
+                    // late, at an empty tile, found the other's barrier a phase too
+                    // far, and the block stood until its waits ran out.)
+                    if (before > 0u && !warp_and(wait_newest(mbar_at(mb, kUFree0 + kKSteps * (int)((before - 1u) & 1u) + ks),
+                                                             ((before - 1u) >> 1) + 1u)))
                         return false;
                     unsigned char *slot = m.u + (ks % US) * kUSlot;
                     store8<F16>(slot, kUc, core_off(row, 0, 16), pk[0]);
