@@ -11,7 +11,7 @@
 // synthetic batch of that key's size (three compressed iterations in a row, or
 // one full iteration and the final pass; as a graph, like a user's run); the
 // fastest compressed-iteration shape and the fastest full-pass shape win, with
-// a margin against the tensor cores.  Results live in the plan and, when the
+// a handicap of the tensor cores.  Results live in the plan and, when the
 // plan names a cache file, in a small JSON file.
 #include <algorithm>
 #include <cmath>
@@ -107,17 +107,18 @@ constexpr int kTuneSub = 3;
 // The tensor cores' products keep 16 bits of their operands and drop what falls
 // below FP32's last bit, the CUDA cores' kernels work in FP32: the pick is part
 // of what a caller gets for a size.  So it keeps to the lines that the timings
-// drew when the tensor-core launches still summed their partials on one SM per
-// hologram, rather than move with each gain of those launches: they are taken
-// for compressed iterations when 1.25 times as fast, and for full passes when
-// they win by what those sums cost, 0.25 us a pass and spot (7 at least, 25 at
-// most).  Without the margins 48 of 432 sizes (P = 128 to 1152, N = 16 to 512, c
-// = 1 to 1/32, batches of 1 to 64) moved their compressed iterations and 91 their
-// full passes to the tensor cores, and a whole solve of P = 64 came out 1.1e-5
-// from exact instead of 1.5e-6; with them 10 and 4 do (of the old timings' own
-// picks, 5 % differed from one run to the next).
-constexpr double kTcSubGain = 1.25;
-static double tc_full_margin_ms(int N) { return 1e-3 * std::clamp(0.25 * N, 7.0, 25.0); }
+// drew when the tensor-core launches started up serially and summed a hologram's
+// partials on one SM, rather than move with each gain of those launches: a
+// tensor-core launch's time counts with what it cost more then, net of the other
+// kernels' gains (medians over 432 sizes, P = 128 to 1152, N = 16 to 512, c = 1 to
+// 1/32, batches of 1 to 64; ms, by the key's N).  Without it 51 of these sizes take
+// the tensor cores for compressed iterations and 163 for a final pass that did not
+// before, and a whole solve of P = 64 came out 1.1e-5 from exact instead of
+// 1.5e-6; with it 7 and 8 do, and 11 and 8 the other way round (of those timings'
+// own picks, 5 % differed from one run to the next).
+static double tc_sub_extra(int N) { return 1e-3 * (4.0 + N / 40.0); }
+static double tc_full_extra(int N) { return 1e-3 * (4.5 + N / 50.0); }
+static double tc_final_extra(int N) { return 1e-3 * (26.0 + N / 25.0); }
 
 // A synthetic batch of the key's size: kTuneSub compressed iterations, or a full
 // iteration and the final pass.
@@ -192,8 +193,8 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
         TileShape sh{cand[0], cand[1], best.full_threads, fp16};
         if (!shape_supported(sh)) continue;
         if (shape_max_grid(sh, kLaunchSubset, k.N, p->sm_count) <= 0) continue;
-        const double gain = cand[0] == kSubsetTc ? kTcSubGain : 1.0;
-        const auto cost = [&](const double *r) { return gain * r[0]; };
+        const double extra = cand[0] == kSubsetTc ? tc_sub_extra(k.N) : 0.0;
+        const auto cost = [&](const double *r) { return r[0] + extra; };
         CSWGS_TRY(time_steps(p, specs, sh, false, best_sub, cost, t));
         if (cost(t) < best_sub) {
             best_sub = cost(t);
@@ -206,8 +207,8 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
     for (int ft : kFullCandidates) {
         TileShape sh{best.threads, best.ppt, ft, fp16};
         if (shape_max_grid(sh, kLaunchFull, k.N, p->sm_count) <= 0) continue;
-        const double margin = is_full_tc(ft) ? tc_full_margin_ms(k.N) : 0.0;
-        const auto cost = [&](const double *r) { return wfull * (r[0] + margin) + r[1] + margin; };
+        const double extra = is_full_tc(ft) ? wfull * tc_full_extra(k.N) + tc_final_extra(k.N) : 0.0;
+        const auto cost = [&](const double *r) { return wfull * r[0] + r[1] + extra; };
         CSWGS_TRY(time_steps(p, specs, sh, true, best_full, cost, t));
         if (cost(t) < best_full) {
             best_full = cost(t);
