@@ -93,6 +93,7 @@ struct TileShape {
     int full_threads;   // full iterations and final pass: threads per block, or kFullTcWs
     int fp16 = 0;       // compressed iterations use the half-precision sincos
     int strip = 0;      // tensor-core launches: tiles per work item (0: chosen per launch)
+    int exact = 0;      // compressed iterations on the tensor cores with the row factors to FP32 rounding
 };
 
 // full_threads value that selects the tensor-core kernel for full iterations
@@ -177,7 +178,7 @@ int full_tc_max_grid(int variant, int maxN, int sm_count);
 cudaError_t launch_full_tc(int variant, const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles,
                            int maxN, unsigned *queue, int grid, int sm_count, cudaStream_t s);
 cudaError_t launch_subset_tc(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles, int maxN,
-                             unsigned *queue, int grid, int f16, int sm_count, cudaStream_t s);
+                             unsigned *queue, int grid, int f16, int exact, int sm_count, cudaStream_t s);
 void full_tc_table_bytes(int P, int N, size_t *rw, size_t *c, size_t *cs);   // cs: split BF16 (FP16: half)
 cudaError_t launch_tc_const_tables(const HoloDev *holos, int count, int sm_count, cudaStream_t s);
 cudaError_t launch_tc_rw_tables(const HoloDev *holos, const LaunchSlot *slots, int nslots, int maxP, int maxN,

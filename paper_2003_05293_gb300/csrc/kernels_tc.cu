@@ -1186,6 +1186,17 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
+// sin and cos of 2 pi T / 2^32 + corr to FP32 rounding (corr small): the top 24
+// bits of T through sincospi, the rest and corr to first order.
+__device__ __forceinline__ float2 phasor_exact(int32_t T, float corr)
+{
+    const int32_t hi = T & ~0xFF;
+    float s, c;
+    sincospif((float)hi * 0x1p-31f, &s, &c);   // hi has 24 significant bits: exact
+    const float r = fmaf((float)(T & 0xFF), kTwoPiF * 0x1p-32f, corr);
+    return make_float2(fmaf(-s, r, c), fmaf(c, r, s));
+}
+
 // The partial V_n = sum_y conj(R_n(y)) Z(n, y) of spot n of a closed Z
 // accumulation (a strip at row block y0) over the tile's rows ys0 .. ys1 - 1.  R_n(y)
 // along the rows by recurrence: its phase is quadratic in y, so R(y + 1) =
@@ -1200,15 +1211,29 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
 // (Two runs in a pair instead, rows y and y + 8: seven steps one after the other
 // and Z's rows moved into pairs; 64 holograms of N up to 300 12.34 ms against
 // 11.93.)
+// An error of E is the same way round in every run: with the hardware's sine and
+// cosine every theta_n is off by 2e-6 rad rms per iteration.  With EXACT, E^4 is
+// right to FP32 rounding and R and D2 are evaluated for even and odd rows each:
+// 2e-7 to 3e-7, as much as phasors of each pixel's own.  Serving takes it where a
+// request would otherwise run on those: u of 32 requests of N up to 1000 ends
+// 6e-7 from exact (1.6e-6 on FP32 phasors, 2.8e-6 without), in the same time.
+template <bool EXACT>
 __device__ __forceinline__ float2 strip_dot(uint32_t z_re, uint32_t z_im, const int4 *coef, int n, int N, int y0,
                                             int half, int ys0, int ys1)
 {
     const int4 cf = coef[min(n, N - 1)];
     const int32_t tilt = cf.y, Gh = cf.z;
     const float gl = __int_as_float(cf.w);
-    float2 E;
-    sincos_fix(kFixRound + 2u * (uint32_t)Gh, fmaf(2.f, gl, -kTwoPiF), E.y, E.x);
-    const float2 E2 = cmul(E, E), E3 = cmul(E2, E), E4 = cmul(E2, E2);
+    float2 E, E3, E4;
+    if constexpr (EXACT) {
+        E4 = phasor_exact((int32_t)(8u * (uint32_t)Gh), 8.f * gl);
+        E = E3 = E4;   // not used
+    } else {
+        sincos_fix(kFixRound + 2u * (uint32_t)Gh, fmaf(2.f, gl, -kTwoPiF), E.y, E.x);
+        const float2 E2 = cmul(E, E);
+        E3 = cmul(E2, E);
+        E4 = cmul(E2, E2);
+    }
     const uint64_t F_c = pack2(E.x, E3.x), F_s = pack2(E.y, E3.y), nF_s = pack2(-E.y, -E3.y);
     const uint64_t E_c = pack2(E4.x, E4.x), E_s = pack2(E4.y, E4.y), nE_s = pack2(-E4.y, -E4.y);
     uint64_t vr = 0ull, vi = 0ull;   // even and odd rows; vi is the sum's negative imaginary part
@@ -1220,16 +1245,35 @@ __device__ __forceinline__ float2 strip_dot(uint32_t z_re, uint32_t z_im, const 
         uint64_t Rc[8], Rs[8];
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            const int u0 = y0 + ys + 8 * b - half, du = 2 * u0 + 1;
-            // R at row u0 and D there: phase of R(u + 1) / R(u), tilt + Gh (2 u + 1)
+            // R at the run's first rows u0 and u0 + 1, and D2 there
+            const int u0 = y0 + ys + 8 * b - half;
             const float2 r = spot_factor(tilt, Gh, gl, u0, kFixRound, 1.f);
-            float2 d;
-            sincos_fix(kFixRound + (uint32_t)tilt + (uint32_t)Gh * (uint32_t)du, fmaf(gl, (float)du, -kTwoPiF), d.y, d.x);
-            const float2 r1 = cmul(r, d), dd = cmul(d, d);
-            const uint64_t dc = pack2(dd.x, dd.x), ds = pack2(dd.y, dd.y);
+            float2 r1;
+            uint64_t Dc, Ds;
+            if constexpr (EXACT) {
+                // phase of R(u + 2) / R(u): tilt 2 + Gh (4 u + 4)
+                float2 d0, d1;
+                r1 = spot_factor(tilt, Gh, gl, u0 + 1, kFixRound, 1.f);
+                sincos_fix(kFixRound + 2u * (uint32_t)tilt + (uint32_t)Gh * (uint32_t)(4 * u0 + 4),
+                           fmaf(gl, (float)(4 * u0 + 4), -kTwoPiF), d0.y, d0.x);
+                sincos_fix(kFixRound + 2u * (uint32_t)tilt + (uint32_t)Gh * (uint32_t)(4 * u0 + 8),
+                           fmaf(gl, (float)(4 * u0 + 8), -kTwoPiF), d1.y, d1.x);
+                Dc = pack2(d0.x, d1.x);
+                Ds = pack2(d0.y, d1.y);
+            } else {
+                // D, the phase of R(u + 1) / R(u): tilt + Gh (2 u + 1); D2 = D^2 E and D^2 E^3
+                const int du = 2 * u0 + 1;
+                float2 d;
+                sincos_fix(kFixRound + (uint32_t)tilt + (uint32_t)Gh * (uint32_t)du, fmaf(gl, (float)du, -kTwoPiF), d.y,
+                           d.x);
+                r1 = cmul(r, d);
+                const float2 dd = cmul(d, d);
+                const uint64_t dc = pack2(dd.x, dd.x), ds = pack2(dd.y, dd.y);
+                Dc = fma2(dc, F_c, mul2(ds, nF_s));
+                Ds = fma2(dc, F_s, mul2(ds, F_c));
+            }
             Rc[4 * b] = pack2(r.x, r1.x);
             Rs[4 * b] = pack2(r.y, r1.y);
-            uint64_t Dc = fma2(dc, F_c, mul2(ds, nF_s)), Ds = fma2(dc, F_s, mul2(ds, F_c));   // D2: D^2 E | D^2 E^3
 #pragma unroll
             for (int q = 4 * b; q < 4 * b + 3; ++q) {
                 const uint64_t nDs = Ds ^ 0x8000000080000000ull;
@@ -1516,7 +1560,7 @@ __device__ __forceinline__ void epilogue_u(const SmemWs &m, const Info *info, ui
 // Z(n, y), one spot per thread over half the 128 rows, while the u warps go on with
 // the next tiles.  In the final pass they also write each tile's phase map
 // (and gray levels) from S, beside the u warps' work on u.
-template <int UG>
+template <int UG, bool EXACT>
 __device__ __forceinline__ void epilogue_v(const Info *info, float2 (*s_half)[kSpotBlock], uint32_t mb, uint32_t tmem,
                                            unsigned *status)
 {
@@ -1562,8 +1606,8 @@ __device__ __forceinline__ void epilogue_v(const Info *info, float2 (*s_half)[kS
             if (!ok) break;
             fence_after();
             const int n = sb * kSpotBlock + 32 * q + lane;
-            float2 v = strip_dot(tmem + lanes, tmem + kRows + lanes, coef, n, N, y0, half, hv * (kRows / 2),
-                                       (hv + 1) * (kRows / 2));
+            float2 v = strip_dot<EXACT>(tmem + lanes, tmem + kRows + lanes, coef, n, N, y0, half, hv * (kRows / 2),
+                                        (hv + 1) * (kRows / 2));
             fence_before();
             const uint32_t buf = n_z & 1u;
             if (hv) s_half[buf][32 * q + lane] = v;
@@ -1595,7 +1639,7 @@ __device__ __forceinline__ void epilogue_v(const Info *info, float2 (*s_half)[kS
 
 }  // namespace tc
 
-template <int UG, bool F16, int US>
+template <int UG, bool F16, int US, bool EXACT>
 __global__ void __launch_bounds__(tc::ws::Cfg<UG>::kThreads, 1)
 iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__restrict__ slots, int nslots,
                       int total_tiles, unsigned *queue)
@@ -1659,7 +1703,7 @@ iter_full_tcws_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__res
     } else if (warp < Cfg<UG>::kU) {
         epilogue_u<UG, F16, US>(m, s_info, mb, s_tmem, status);
     } else {
-        epilogue_v<UG>(s_info, s_half, mb, s_tmem, status);
+        epilogue_v<UG, EXACT>(s_info, s_half, mb, s_tmem, status);
     }
     tc::fence_before();
     __syncthreads();
@@ -1836,20 +1880,18 @@ tcws_tails_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__restric
     cluster.sync();   // s_out is read before any block of the cluster leaves
 }
 
-template <int UG, bool F16, int US>
+template <int UG, bool F16, bool EXACT>
 static int tcws_max_grid_of(int maxN, int sm_count)
 {
+    const auto kernel = iter_full_tcws_kernel<UG, F16, tc::ws::kKSteps, EXACT>;
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, iter_full_tcws_kernel<UG, F16, US>) != cudaSuccess) return 0;
+    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return 0;
     const size_t limit = 227 * 1024 - fa.sharedSizeBytes;
-    const size_t smem = tc::ws::Lay<US>::kSmem;
+    const size_t smem = tc::ws::Lay<tc::ws::kKSteps>::kSmem;
     if (smem > limit || maxN > kTailMaxN) return 0;
-    if (cudaFuncSetAttribute(iter_full_tcws_kernel<UG, F16, US>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)limit) != cudaSuccess)
-        return 0;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess) return 0;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, iter_full_tcws_kernel<UG, F16, US>,
-                                                      tc::ws::Cfg<UG>::kThreads, smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, tc::ws::Cfg<UG>::kThreads, smem) != cudaSuccess)
         return 0;
     return std::min(per_sm, 1) * sm_count;   // a block holds all 512 tensor-memory columns
 }
@@ -1857,17 +1899,17 @@ static int tcws_max_grid_of(int maxN, int sm_count)
 // Resident blocks of the kernel (all forms; sets their shared-memory limits).
 static int tcws_max_grid(int maxN, int sm_count)
 {
-    constexpr int K4 = tc::ws::kKSteps;
-    return std::min({tcws_max_grid_of<1, false, K4>(maxN, sm_count), tcws_max_grid_of<1, true, K4>(maxN, sm_count),
-                     tcws_max_grid_of<2, false, K4>(maxN, sm_count), tcws_max_grid_of<2, true, K4>(maxN, sm_count)});
+    return std::min({tcws_max_grid_of<1, false, false>(maxN, sm_count), tcws_max_grid_of<1, true, false>(maxN, sm_count),
+                     tcws_max_grid_of<2, false, false>(maxN, sm_count), tcws_max_grid_of<2, true, false>(maxN, sm_count),
+                     tcws_max_grid_of<1, false, true>(maxN, sm_count), tcws_max_grid_of<2, false, true>(maxN, sm_count)});
 }
 
-template <int UG, bool F16>
+template <int UG, bool F16, bool EXACT>
 static cudaError_t tcws_launch_one(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles,
                                    unsigned *queue, int grid, bool chain, cudaStream_t s)
 {
     constexpr int K4 = tc::ws::kKSteps;
-    return launch_chained(iter_full_tcws_kernel<UG, F16, K4>, dim3(grid), dim3(tc::ws::Cfg<UG>::kThreads),
+    return launch_chained(iter_full_tcws_kernel<UG, F16, K4, EXACT>, dim3(grid), dim3(tc::ws::Cfg<UG>::kThreads),
                           tc::ws::Lay<K4>::kSmem, chain, s, holos, slots, nslots, total_tiles, queue);
 }
 
@@ -1900,7 +1942,8 @@ cudaError_t launch_tc_tails(const HoloDev *holos, const LaunchSlot *slots, int n
 }
 
 static cudaError_t tcws_launch(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles, int maxN,
-                               unsigned *queue, int grid, bool subset, int f16, int sm_count, cudaStream_t s)
+                               unsigned *queue, int grid, bool subset, int f16, int exact, int sm_count,
+                               cudaStream_t s)
 {
     (void)cudaGetLastError();
     // two groups of u warps where they pay (kVWarps' comment): more than one
@@ -1908,8 +1951,9 @@ static cudaError_t tcws_launch(const HoloDev *holos, const LaunchSlot *slots, in
     // block's few tiles, where latency counts)
     const bool ug2 = tc::nspotblocks(maxN) > 1 || total_tiles < 8 * grid;
     const bool chain = chain_launch(nslots, sm_count);
-    const auto one = f16 ? (ug2 ? tcws_launch_one<2, true> : tcws_launch_one<1, true>)
-                         : (ug2 ? tcws_launch_one<2, false> : tcws_launch_one<1, false>);
+    const auto one = f16     ? (ug2 ? tcws_launch_one<2, true, false> : tcws_launch_one<1, true, false>)
+                     : exact ? (ug2 ? tcws_launch_one<2, false, true> : tcws_launch_one<1, false, true>)
+                             : (ug2 ? tcws_launch_one<2, false, false> : tcws_launch_one<1, false, false>);
     const cudaError_t e = one(holos, slots, nslots, total_tiles, queue, grid, chain, s);
     if (e != cudaSuccess) return e;
     return launch_tc_tails(holos, slots, nslots, total_tiles, maxN, subset, sm_count, s);
@@ -2076,16 +2120,16 @@ cudaError_t launch_tc_mask_scatter(const HoloDev *holos, const LaunchSlot *slots
 }
 
 cudaError_t launch_subset_tc(const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles, int maxN,
-                             unsigned *queue, int grid, int f16, int sm_count, cudaStream_t s)
+                             unsigned *queue, int grid, int f16, int exact, int sm_count, cudaStream_t s)
 {
-    return tcws_launch(holos, slots, nslots, total_tiles, maxN, queue, grid, true, f16, sm_count, s);
+    return tcws_launch(holos, slots, nslots, total_tiles, maxN, queue, grid, true, f16, exact, sm_count, s);
 }
 
 cudaError_t launch_full_tc(int variant, const HoloDev *holos, const LaunchSlot *slots, int nslots, int total_tiles,
                            int maxN, unsigned *queue, int grid, int sm_count, cudaStream_t s)
 {
     if (variant != kFullTcWs) return cudaErrorInvalidValue;
-    return tcws_launch(holos, slots, nslots, total_tiles, maxN, queue, grid, false, 0, sm_count, s);
+    return tcws_launch(holos, slots, nslots, total_tiles, maxN, queue, grid, false, 0, 0, sm_count, s);
 }
 
 }  // namespace cswgs

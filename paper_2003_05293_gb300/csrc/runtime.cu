@@ -229,7 +229,8 @@ cudaError_t shape_launch(TileShape shape, int kind, const HoloDev *holos, const 
     if (kind == kLaunchFull && is_full_tc(shape.full_threads))
         return launch_full_tc(shape.full_threads, holos, slots, nslots, total_tiles, maxN, queue, grid, sm_count, s);
     if (kind == kLaunchSubset && shape.threads == kSubsetTc)
-        return launch_subset_tc(holos, slots, nslots, total_tiles, maxN, queue, grid, shape.fp16, sm_count, s);
+        return launch_subset_tc(holos, slots, nslots, total_tiles, maxN, queue, grid, shape.fp16, shape.exact, sm_count,
+                                s);
     if (kind == kLaunchSubset && shape.threads == kSubsetGather)
         return launch_subset_gather(holos, slots, nslots, total_tiles, maxN, queue, grid, sm_count, s);
     return launch_iter_fp32(shape, kind, holos, slots, nslots, total_tiles, maxN, queue, grid, sm_count, s);

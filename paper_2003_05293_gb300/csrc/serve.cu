@@ -144,8 +144,9 @@ cswgs_status Server::start()
 // 1152 in full launches: direct phasors 0.95 c N, tensor cores 3.3 (N = 10),
 // 3.8 (100), 11.3 (300) and ~35 (1000) ps per pixel and iteration: they meet
 // at c N = 4 per spot block.  (32 requests of N = 10, 100, 1000 at c = 1/8,
-// N = 10 first: 31 ms with every compressed iteration on the CUDA cores, 11.9
-// with this choice.)
+// N = 10 first: 31 ms with every compressed iteration on the CUDA cores, 11.3
+// with this choice.)  The other way round, a loop shaped by a heavy request runs
+// light ones on its kernel too; nothing chooses there.
 bool Server::tc_subset(const HoloSpec &s) const
 {
     if (shape_.fp16 || uses_masks(shape_) || !is_full_tc(shape_.full_threads)) return false;
@@ -436,6 +437,7 @@ void Server::loop()
         TileShape tc_shape = shape_;
         tc_shape.threads = kSubsetTc;
         tc_shape.ppt = 1;
+        tc_shape.exact = 1;   // in place of FP32 phasors: no precision lost
         const TileShape group_shape[kGroups] = {shape_, tc_shape, shape_, lean_shape(), lean_shape()};
         int nslots = 0, group_slots[kGroups] = {}, group_tiles[kGroups] = {}, group_maxN[kGroups] = {},
             group_maxP[kGroups] = {};
