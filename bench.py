@@ -74,8 +74,10 @@ def measured_traffic(args, tile):
 
 
 # full_threads markers of the tensor-core kernels: kernel name, threads per block
-TC_KERNELS = {2: ("iter_full_tcws_kernel (warp-specialised: 8 epilogue warps, a producer warp, a GEMM 1 warp "
-                   "and a GEMM 2 warp)", 352)}
+# (of its 480-thread form, which the default workload's launches take; launches
+# of few tiles or more than 128 spots take one of 608 threads, 16 epilogue warps)
+TC_KERNELS = {2: ("iter_full_tcws_kernel (warp-specialised: 12 epilogue warps, a producer warp, a GEMM 1 warp "
+                   "and a GEMM 2 warp)", 480)}
 
 
 def kernel_name(tile, kind):

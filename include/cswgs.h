@@ -285,11 +285,10 @@ cswgs_status cswgs_batch_pairs(cswgs_batch b, double *pairs_total, double *pairs
  * thread; for full iterations and the final pass threads per block of the
  * CUDA-core kernel, or a tensor-core kernel (tiles of 128 x 64 pixels,
  * split-BF16 products accumulated in FP32): 2 = the warp-specialised kernel,
- * pipelined across tiles (8 epilogue warps, a producer warp and two MMA
- * warps); compressed
- * iterations report threads = 1 when they run on that kernel too (u zero
- * outside the subset); and the persistent blocks of each per launch.  Any
- * pointer may be NULL. */
+ * pipelined across tiles (12 or 16 epilogue warps, a producer warp and two
+ * MMA warps); compressed iterations report threads = 1 when they run on that
+ * kernel too (u zero outside the subset); and the persistent blocks of each
+ * per launch.  Any pointer may be NULL. */
 cswgs_status cswgs_batch_tile_shape(cswgs_batch b, int *threads, int *pixels_per_thread, int *full_threads,
                                     int *blocks, int *full_blocks);
 
@@ -342,7 +341,9 @@ cswgs_status cswgs_solve_batch(cswgs_plan p, const cswgs_request *reqs, int coun
  * and leave between launches.  The serving loop starts on the first submit. */
 
 /* Queues a request (inputs are copied).  *ticket identifies it.  A request
- * whose footprint can never fit mem_cap_bytes fails with CSWGS_ENOMEM. */
+ * whose footprint can never fit mem_cap_bytes fails with CSWGS_ENOMEM.  One that
+ * fits only without the tensor-core kernel's factor tables or the subset mask
+ * runs on kernels that need none, which are slower. */
 cswgs_status cswgs_submit(cswgs_plan p, const cswgs_request *r, uint64_t *ticket);
 
 /* CSWGS_EBUSY while pending; CSWGS_OK with *res filled once finished (the
@@ -371,7 +372,8 @@ cswgs_status cswgs_serve_stats_get(cswgs_plan p, cswgs_serve_stats *s);
 
 /* Times the candidate tile shapes (threads per block, pixels per thread) of
  * the FP32 iteration kernel on a synthetic hologram of this size, keeps the
- * fastest for the (P, N) bucket and writes the tune cache if the plan has one.
+ * fastest for the (P, N) bucket (the tensor-core kernel, whose products are less
+ * precise, only by a margin) and writes the tune cache if the plan has one.
  * *best_ms (may be NULL) receives the best per-iteration time. */
 cswgs_status cswgs_autotune(cswgs_plan p, int P, int N, double subset_fraction, double *best_ms);
 

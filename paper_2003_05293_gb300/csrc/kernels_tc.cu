@@ -457,9 +457,6 @@ __global__ void __launch_bounds__(256) const_tables_kernel(const HoloDev *__rest
     }
 }
 
-// R' = w a e^{i theta} R (GEMM 1's A: 128 rows x 16 spots per block) of the
-// hologram of each slot, from its current spot state (rw_tables_kernel below).
-
 // The Mp draws of S_j (Section 3) of the slot's hologram, each setting its
 // pixel's bit in the iteration's mask, which is clear before (the tails of the
 // last launch that used it cleared it).  Grid: blocks x slots.
@@ -602,6 +599,8 @@ __global__ void __launch_bounds__(kLocalThreads) mask_local_kernel(const HoloDev
     }
 }
 
+// R' = w a e^{i theta} R (GEMM 1's A: 128 rows x 16 spots per block) of the
+// hologram of each slot, from its current spot state.
 __global__ void __launch_bounds__(256) rw_tables_kernel(const HoloDev *__restrict__ holos,
                                                         const LaunchSlot *__restrict__ slots)
 {
@@ -650,8 +649,8 @@ __global__ void __launch_bounds__(256) rw_tables_kernel(const HoloDev *__restric
 // ----------------------------------------------------------- warp roles --
 // Tiles are pipelined by warp roles: a producer warp (takes the work items and
 // loads GEMM 1's operand stages), a GEMM 1 warp, a GEMM 2 warp (one elected
-// lane of each issues its bulk copies and MMAs), 4 u warps (epilogue 1) and 4
-// V warps (epilogue 2).  The producer runs ahead of the GEMM 1 warp by the
+// lane of each issues its bulk copies and MMAs), 4 or 8 u warps (epilogue 1)
+// and 8 V warps (epilogue 2).  The producer runs ahead of the GEMM 1 warp by the
 // ring's depth: a tcgen05.mma issue waits for the tensor pipe, so copies
 // issued from the MMA warp would start one stage late.
 // A work item is a strip: LaunchSlot::strip consecutive tiles of one row block
@@ -1775,7 +1774,8 @@ tcws_tails_kernel(const HoloDev *__restrict__ holos, const LaunchSlot *__restric
     const HoloDev &H = holos[sl.holo];
     const int rank = blockIdx.x % CL, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     chain_start();
-    if (tid < 32) asm volatile("prefetch.global.L1 [%0];" :: "l"(reinterpret_cast<const char *>(&H) + 8 * tid));
+    if (8 * tid < (int)sizeof(HoloDev))
+        asm volatile("prefetch.global.L1 [%0];" :: "l"(reinterpret_cast<const char *>(&H) + 8 * tid));
     chain_wait();
     if (blockIdx.y > 0) {   // a whole cluster of its own
         if (sl.pass == kPassSubset && H.mask) {
