@@ -39,7 +39,7 @@
 // (epilogue 1), eight reduce Z to the spot fields (epilogue 2) once per strip of
 // tiles along a row block and, in the final pass, write the phase map from S.
 // The shared-memory pipe bounds a long launch of N <= 128: a tile's operand
-// reads, copies and stores of u take 8.0 k of its ~8.8 k cycles (N = 100).  Every wait is bounded
+// reads, copies and stores of u take 8.0 k of its ~8.6 k cycles (N = 100).  Every wait is bounded
 // and a timeout is recorded in the launch's status word instead of hanging.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
@@ -490,11 +490,12 @@ __global__ void __launch_bounds__(256) mask_scatter_kernel(const HoloDev *__rest
 // most P values: the four rounds' F are tabled first (4 P hashes instead of
 // 4 Mp / G; 16 bits an entry, halves and entries carried doubled so that they
 // are byte offsets), and a draw is four table loads, four additions modulo a
-// half's range and the OR.  Bound by the shared-memory path (random 16-bit
-// loads and ORs, three to four lanes to a bank); with the hashes made per draw
-// it was bound by the ALU, and with G > 1 it ended in an OR of every word in
-// global memory: 46.7 us for 64 masks of P = 1152, c = 1/8. (A 64-hologram
-// batch of 31 launches: 11.70 ms with that form, 11.09 with this.)
+// half's range and the OR.  Bound by the latency of these dependent loads (32
+// warps an SM wait for them most of the time; random, three to four lanes to a
+// bank, they take half of the shared-memory pipe): 33 us for 64 masks of P =
+// 1152, c = 1/8.  With the hashes made per draw it was bound by the ALU, and
+// with G > 1 it ended in an OR of every word in global memory: 47 us.  (A
+// 64-hologram batch of 31 launches: 11.70 ms with that form, 11.09 with this.)
 constexpr int kLocalThreads = 1024;
 
 // (L + F(R)) mod p with everything doubled: byte offsets into the round tables.
