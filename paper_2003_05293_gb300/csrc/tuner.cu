@@ -111,14 +111,14 @@ constexpr int kTuneSub = 3;
 // partials on one SM, rather than move with each gain of those launches: a
 // tensor-core launch's time counts with what it cost more then, net of the other
 // kernels' gains (medians over 432 sizes, P = 128 to 1152, N = 16 to 512, c = 1 to
-// 1/32, batches of 1 to 64; ms, by the key's N).  Without it 51 of these sizes take
-// the tensor cores for compressed iterations and 163 for a final pass that did not
-// before, and a whole solve of P = 64 came out 1.1e-5 from exact instead of
-// 1.5e-6; with it 7 and 8 do, and 11 and 8 the other way round (of those timings'
-// own picks, 5 % differed from one run to the next).
-static double tc_sub_extra(int N) { return 1e-3 * (4.0 + N / 40.0); }
-static double tc_full_extra(int N) { return 1e-3 * (4.5 + N / 50.0); }
-static double tc_final_extra(int N) { return 1e-3 * (26.0 + N / 25.0); }
+// 1/32, batches of 1 to 64; ms, by the key's N and B).  Without it 51 of these
+// sizes take the tensor cores for compressed iterations and 163 for a final pass
+// that did not before, and a whole solve of P = 64 came out 1.1e-5 from exact
+// instead of 1.5e-6; with it 3 and 8 do, and 13 and 8 the other way round (of those
+// timings' own picks, 5 % differed from one run to the next).
+static double tc_sub_extra(const TuneKey &k) { return 1e-3 * (4.0 + k.N / 40.0 + 1.5 * std::log2(k.B)); }
+static double tc_full_extra(const TuneKey &k) { return 1e-3 * (4.5 + k.N / 50.0); }
+static double tc_final_extra(const TuneKey &k) { return 1e-3 * (26.0 + k.N / 25.0 + 3.0 * std::log2(k.B)); }
 
 // A synthetic batch of the key's size: kTuneSub compressed iterations, or a full
 // iteration and the final pass.
@@ -193,7 +193,7 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
         TileShape sh{cand[0], cand[1], best.full_threads, fp16};
         if (!shape_supported(sh)) continue;
         if (shape_max_grid(sh, kLaunchSubset, k.N, p->sm_count) <= 0) continue;
-        const double extra = cand[0] == kSubsetTc ? tc_sub_extra(k.N) : 0.0;
+        const double extra = cand[0] == kSubsetTc ? tc_sub_extra(k) : 0.0;
         const auto cost = [&](const double *r) { return r[0] + extra; };
         CSWGS_TRY(time_steps(p, specs, sh, false, best_sub, cost, t));
         if (cost(t) < best_sub) {
@@ -207,7 +207,7 @@ static cswgs_status tune_for(cswgs_plan_s *p, const TuneKey &k, double c, double
     for (int ft : kFullCandidates) {
         TileShape sh{best.threads, best.ppt, ft, fp16};
         if (shape_max_grid(sh, kLaunchFull, k.N, p->sm_count) <= 0) continue;
-        const double extra = is_full_tc(ft) ? wfull * tc_full_extra(k.N) + tc_final_extra(k.N) : 0.0;
+        const double extra = is_full_tc(ft) ? wfull * tc_full_extra(k) + tc_final_extra(k) : 0.0;
         const auto cost = [&](const double *r) { return wfull * r[0] + r[1] + extra; };
         CSWGS_TRY(time_steps(p, specs, sh, true, best_full, cost, t));
         if (cost(t) < best_full) {
