@@ -133,9 +133,11 @@ inline int mask_words_of(int P) { return (P + 31) / 32; }
 // kernel before it in the stream still runs (programmatic dependent launch):
 // its launch, set-up and loads of what no kernel of the chain writes (slots,
 // hologram records) overlap that kernel's end.  Each kernel of the chain calls
-// chain_wait() before it reads or writes anything else, and chain_start() first
-// of all, so that its successor may do the same; since every one of them waits
-// for its predecessor to have completed, so do they all, in order.  (Without
+// chain_wait() before it reads or writes anything else, and chain_start() so that
+// its successor may do the same: first of all, or after its own wait where its
+// successor is the same kernel (else a whole chain's blocks would pile up).  Since
+// every one of them waits for its predecessor to have completed, so do they all,
+// in order.  (Without
 // `chain` an ordinary launch; the two calls then do nothing.)  A lone hologram's
 // iteration is three such kernels of 3 to 16 us: 30 iterations at P = 1152,
 // N = 100 took 860 us unchained and take 789.
