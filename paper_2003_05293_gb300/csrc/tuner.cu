@@ -6,8 +6,8 @@
 // the CUDA cores costs c times a full one, on the tensor cores about as much
 // as a full one, so the winner changes with c; and whether the pupil is round
 // and the beam Gaussian, since a round pupil has fewer pixels and dearer draws:
-// the paper's optics took 960 us a solve with the direct-phasor shape that
-// is best on a square of their size and take 668).  Each candidate runs a
+// the paper's optics take 769 us a solve with the direct-phasor shape that is
+// best on a square of their size and 634 with their own).  Each candidate runs a
 // synthetic batch of that key's size (three compressed iterations in a row, or
 // one full iteration and the final pass; as a graph, like a user's run); the
 // fastest compressed-iteration shape and the fastest full-pass shape win, with
